@@ -307,23 +307,19 @@ sts_status build_plan(sts_jac_s *h, int dir, bool with_streams) {
     P.h_row_off = row_off;
     P.h_pslot_slot = pslot_slot;
     P.h_blk = blk;
-    std::vector<int> pat_ptr(2 * (b + 1)), pat_idx, pat_src;
+    std::vector<int> pat_ptr(2 * (b + 1)), pat_idx;
     for (int k = 0; k < 2; ++k) {
         std::copy(kp[k].begin(), kp[k].end(), pat_ptr.begin() + k * (b + 1));
         pat_idx.insert(pat_idx.end(), ki[k].begin(), ki[k].end());
-        pat_src.insert(pat_src.end(), ks[k].begin(), ks[k].end());
     }
     STS_TRY(upload(h, &P.nbr, nbr));
     STS_TRY(upload(h, &P.blk, blk));
     STS_TRY(upload(h, &P.slot_mask, mask));
     STS_TRY(upload(h, &P.grp_rows, grp));
     STS_TRY(upload(h, &P.row_off, row_off));
-    STS_TRY(upload(h, &P.pslot_slot, pslot_slot));
-    STS_TRY(upload(h, &P.pslot_local, pslot_local));
     STS_TRY(upload(h, &P.dtask_slot, dtask_slot));
     STS_TRY(upload(h, &P.pat_ptr, pat_ptr));
     STS_TRY(upload(h, &P.pat_idx, pat_idx));
-    STS_TRY(upload(h, &P.pat_src, pat_src));
     if (with_streams) {
         if (b > 0xffff) return set_error(STS_ERR_INVALID_ARG, "block_size above 65535 is not supported");
         std::vector<unsigned> desc(P.structured ? 1 : pos_kind.size(), 0u);
@@ -349,17 +345,15 @@ sts_status build_plan(sts_jac_s *h, int dir, bool with_streams) {
                                      "add an explicit zero to the pattern", p);
         }
         STS_TRY(upload(h, &P.desc, desc));
-        STS_TRY(upload(h, &P.pos_kind, pos_kind));
-        STS_TRY(upload(h, &P.pos_arg, pos_arg));
-        STS_TRY(upload(h, &P.dpos_kind, dpos_kind));
-        STS_TRY(upload(h, &P.dpos_arg, dpos_arg));
+        STS_TRY(values_plan(h, P, pos_kind, pos_arg, dpos_kind, dpos_arg, ks, pslot_slot, pslot_local));
         const size_t nm = (size_t)nt * P.tile_len * kTile;
         const size_t nd = (size_t)nt * P.n_dtasks * Lp * kTile;
-        STS_TRY(dalloc(h, &P.main64, nm));
-        STS_TRY(dalloc(h, &P.dotv64, nd));
+        // zeroed here: values_load writes only the positions that hold a value
+        STS_TRY(dalloc_zero(h, &P.main64, nm));
+        STS_TRY(dalloc_zero(h, &P.dotv64, nd));
         if (h->dtype == STS_MIXED) {
-            STS_TRY(dalloc(h, &P.main32, nm));
-            STS_TRY(dalloc(h, &P.dotv32, nd));
+            STS_TRY(dalloc_zero(h, &P.main32, nm));
+            STS_TRY(dalloc_zero(h, &P.dotv32, nd));
         }
     }
     return STS_OK;
@@ -432,9 +426,9 @@ sts_status load_values(sts_jac_s *h, const double *S, const double *U, const dou
     }
     sts_status st = STS_OK;
     if (h->rep == STS_REP_FACTORED) {
-        st = mv_repack(h, 0, dS, dU, dV);
-        if (st == STS_OK && h->has_T) st = mv_repack(h, 1, dS, dU, dV);
-        if (st == STS_OK) st = smw_repack(h, dS, dU, dV);
+        h->smw.ready = false;
+        st = values_load(h, 0, dS, dU, dV);
+        if (st == STS_OK && h->has_T) st = values_load(h, 1, dS, dU, dV);
         h->streams_dirty = true;
     } else {
         st = dense_build(h, dS, dU, dV);

@@ -445,46 +445,6 @@ done:
     }
 }
 
-// Repack the public values into one stream of one direction.  Each stream
-// position (per tile and lane) is an S entry of a block slot, an entry of a
-// pair vector (the axpy vectors in the main stream, the dot vectors in the
-// pass-1 stream), or a zero.  A block with fewer pairs than its kind's
-// largest count gets zero vectors in the remaining pair slots.  With vec > 1 each run of vec positions of a
-// lane is contiguous ([tile][position / vec][lane][vec]), for 16-byte loads.
-template <typename T>
-__global__ void k_repack(T *out, const double *S, const double *AX, const int *blk,
-                              const long long *soff, const int *pbase, const int *pos_kind,
-                              const int *pos_arg, const int *pat_src, const int *pslot_slot,
-                              const int *pslot_local, long long tile_len, int n_tiles, int n_slots,
-                              int b, int vec) {
-    const long long per_tile = tile_len * kTile;
-    const long long total = (long long)n_tiles * per_tile;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total;
-         i += (long long)gridDim.x * blockDim.x) {
-        // element i is (tile, position / vec, lane, position % vec)
-        const int t = (int)(i / per_tile);
-        const long long e = i - (long long)t * per_tile;
-        const long long vb = e / (kTile * vec);
-        const int rem = (int)(e - vb * kTile * vec);
-        const int lane = rem / vec;
-        const long long pos = vb * vec + rem % vec;
-        const int kind = pos_kind[pos], arg = pos_arg[pos];
-        double v = 0.0;
-        if (kind == kPosZero) {
-            v = 0.0;
-        } else if (kind >= 0) {
-            const int k = blk[((size_t)t * n_slots + kind) * kTile + lane];
-            if (k >= 0) v = S[soff[k] + pat_src[arg]];
-        } else {
-            const int ps = -1 - kind;
-            const int k = blk[((size_t)t * n_slots + pslot_slot[ps]) * kTile + lane];
-            const int l = pslot_local[ps];
-            if (k >= 0 && l < pbase[k + 1] - pbase[k]) v = AX[(size_t)(pbase[k] + l) * b + arg];
-        }
-        out[i] = (T)v;
-    }
-}
-
 // Public vector -> internal [b][ncp].  Cell-major input is transposed through
 // shared memory in 32 x 32 tiles so that both sides are coalesced.
 template <typename T>
@@ -665,28 +625,6 @@ sts_status mv_launch(sts_jac_s *h, const MvArgs<T> &args) {
 }
 
 }  // namespace
-
-sts_status mv_repack(sts_jac_s *h, int dir, const double *S, const double *U, const double *V) {
-    MvPlan &P = h->mv[dir];
-    const double *AX = dir == 0 ? U : V;   // axpy vectors (main stream)
-    const double *DV = dir == 0 ? V : U;   // dot vectors (pass-1 stream)
-    const long long nm = (long long)h->n_tiles * P.tile_len * kTile;
-    const long long nd = (long long)h->n_tiles * P.n_dtasks * P.Lp * kTile;
-    auto rp = [&](auto *out, const double *vec, const int *pk, const int *pa, long long len, long long total,
-                  int vw) {
-        using T = std::remove_pointer_t<decltype(out)>;
-        k_repack<T><<<grid_for(total, 256), 256, 0, h->stream>>>(out, S, vec, P.blk, h->d_soff, h->d_pbase, pk, pa,
-                                                                 P.pat_src, P.pslot_slot, P.pslot_local, len,
-                                                                 h->n_tiles, P.n_slots, h->b, vw);
-    };
-    // the pass-1 stream is read with loads of DotVec<T>::n positions per lane
-    const long long dlen = (long long)P.n_dtasks * P.Lp;
-    if (P.main64) { rp(P.main64, AX, P.pos_kind, P.pos_arg, P.tile_len, nm, 1); STS_LAUNCHED(); }
-    if (P.main32) { rp(P.main32, AX, P.pos_kind, P.pos_arg, P.tile_len, nm, 1); STS_LAUNCHED(); }
-    if (nd > 0 && P.dotv64) { rp(P.dotv64, DV, P.dpos_kind, P.dpos_arg, dlen, nd, DotVec<double>::n); STS_LAUNCHED(); }
-    if (nd > 0 && P.dotv32) { rp(P.dotv32, DV, P.dpos_kind, P.dpos_arg, dlen, nd, DotVec<float>::n); STS_LAUNCHED(); }
-    return STS_OK;
-}
 
 sts_status mv_apply64(sts_jac_s *h, int dir, const double *x, double *y, double *c) {
     const MvPlan &P = h->mv[dir];

@@ -2,13 +2,7 @@
 // (Section 6).  Each diagonal block is A_k = A_k^0 + U_k V_k^T with A_k^0 = S_kk
 // sparse (Eq. R1_Block_Jacobian).
 //
-// Setup (all cells share one schedule; thread index = cell, fastest):
-//   LU of A_k^0 without pivoting on the symbolic schedule of the shared
-//   pattern (natural order; for the paper's arrow pattern there is no fill),
-//   one thread per cell;
-//   W_k = (A_k^0)^-1 U_k   (SMW-1, r sparse solves), one thread per solve;
-//   C_k = I + V_k^T W_k    (FP64), one thread per entry; C_k^-1 by Gauss-Jordan
-//   with pivoting, one thread per cell.
+// Setup: kernels_smw_setup.cu.
 // Apply (SMW-1..3): x0 = (A_k^0)^-1 b_k, t = V_k^T x0, z = C_k^-1 t (FP64),
 //   x_k = x0 - W_k z.  The paper prints "+ W_k z"; with C_k = I + V^T A0^-1 U the
 //   Woodbury identity needs the minus sign, which is what is computed here.
@@ -16,7 +10,6 @@
 //   A0^T (solved from the same LU factors), U and V swapped and C_k^T.
 #include <cuda_runtime.h>
 
-#include <climits>
 #include <cmath>
 #include <cstdio>
 #include <type_traits>
@@ -28,192 +21,6 @@
 
 namespace sts {
 namespace {
-
-struct SetupArgs {
-    const double *Sd, *Ud, *Vd;
-    double *lu, *dinv, *W, *Wt, *Cinv;
-    const int *lu_diag, *src_slot, *d_ptr;
-    const int *colL_ptr, *colL_slot, *upd_ptr, *upd_tgt, *upd_src;
-    const int *fwd_ptr0, *fwd_col0, *fwd_slot0, *bwd_ptr0, *bwd_col0, *bwd_slot0;
-    const int *fwd_ptr1, *fwd_col1, *fwd_slot1, *bwd_ptr1, *bwd_col1, *bwd_slot1;
-    int *err_cell;
-    int nc, ncp, b, r, nnz_lu, nnz_d, with_T;
-};
-
-// Solve A0 w = rhs in place on w[q * ncp + cell] (column of W), N direction.
-__device__ void lu_solve_N(const SetupArgs &a, double *w, int cell) {
-    const size_t P = a.ncp;
-    for (int i = 0; i < a.b; ++i) {
-        double acc = w[i * P + cell];
-        for (int e = a.fwd_ptr0[i]; e < a.fwd_ptr0[i + 1]; ++e)
-            acc = fma(-a.lu[(size_t)a.fwd_slot0[e] * P + cell], w[(size_t)a.fwd_col0[e] * P + cell], acc);
-        w[i * P + cell] = acc;
-    }
-    for (int r = 0; r < a.b; ++r) {
-        const int i = a.b - 1 - r;
-        double acc = w[i * P + cell];
-        for (int e = a.bwd_ptr0[r]; e < a.bwd_ptr0[r + 1]; ++e)
-            acc = fma(-a.lu[(size_t)a.bwd_slot0[e] * P + cell], w[(size_t)a.bwd_col0[e] * P + cell], acc);
-        w[i * P + cell] = acc * a.dinv[i * P + cell];
-    }
-}
-
-// Solve A0^T w = rhs in place: U^T (forward, with the pivots), then L^T (unit).
-__device__ void lu_solve_T(const SetupArgs &a, double *w, int cell) {
-    const size_t P = a.ncp;
-    for (int i = 0; i < a.b; ++i) {
-        double acc = w[i * P + cell];
-        for (int e = a.fwd_ptr1[i]; e < a.fwd_ptr1[i + 1]; ++e)
-            acc = fma(-a.lu[(size_t)a.fwd_slot1[e] * P + cell], w[(size_t)a.fwd_col1[e] * P + cell], acc);
-        w[i * P + cell] = acc * a.dinv[i * P + cell];
-    }
-    for (int r = 0; r < a.b; ++r) {
-        const int i = a.b - 1 - r;
-        double acc = w[i * P + cell];
-        for (int e = a.bwd_ptr1[r]; e < a.bwd_ptr1[r + 1]; ++e)
-            acc = fma(-a.lu[(size_t)a.bwd_slot1[e] * P + cell], w[(size_t)a.bwd_col1[e] * P + cell], acc);
-        w[i * P + cell] = acc;
-    }
-}
-
-// Setup step 1, one thread per cell: the static-pivot LU of S_kk on the shared
-// schedule.  A padding cell gets the identity, so steps 2 and 3 give it W = 0 and
-// C^-1 = I without a special case.
-__global__ void k_smw_lu(SetupArgs a) {
-    const int cell = blockIdx.x * blockDim.x + threadIdx.x;
-    if (cell >= a.ncp) return;
-    const size_t P = a.ncp;
-    for (int s = 0; s < a.nnz_lu; ++s) a.lu[s * P + cell] = 0.0;
-    if (cell >= a.nc) {
-        for (int i = 0; i < a.b; ++i) {
-            a.lu[(size_t)a.lu_diag[i] * P + cell] = 1.0;
-            a.dinv[i * P + cell] = 1.0;
-        }
-        return;
-    }
-    for (int e = 0; e < a.nnz_d; ++e) a.lu[(size_t)a.src_slot[e] * P + cell] = a.Sd[e * P + cell];
-    for (int k = 0; k < a.b; ++k) {
-        double rowmax = 0.0;
-        for (int e = a.d_ptr[k]; e < a.d_ptr[k + 1]; ++e) rowmax = fmax(rowmax, fabs(a.Sd[e * P + cell]));
-        const double piv = a.lu[(size_t)a.lu_diag[k] * P + cell];
-        if (!(fabs(piv) > 1e-14 * rowmax)) {
-            atomicMin(a.err_cell, cell);
-            return;
-        }
-        const double d = 1.0 / piv;
-        a.dinv[k * P + cell] = d;
-        for (int e = a.colL_ptr[k]; e < a.colL_ptr[k + 1]; ++e) {
-            const size_t sl = (size_t)a.colL_slot[e] * P + cell;
-            const double l = a.lu[sl] * d;
-            a.lu[sl] = l;
-            for (int u = a.upd_ptr[e]; u < a.upd_ptr[e + 1]; ++u)
-                a.lu[(size_t)a.upd_tgt[u] * P + cell] =
-                    fma(-l, a.lu[(size_t)a.upd_src[u] * P + cell], a.lu[(size_t)a.upd_tgt[u] * P + cell]);
-        }
-    }
-}
-
-// Setup step 2, one thread per (cell, pair k, direction): W_k = A0^-1 U_k (SMW-1)
-// and, for the adjoint, Wt_k = A0^-T V_k.  Consecutive threads take consecutive
-// cells, so every [slot][cell] access of a warp is one coalesced request.
-__global__ void k_smw_w(SetupArgs a) {
-    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const long long per_dir = (long long)a.ncp * a.r;
-    if (t >= per_dir * (a.with_T ? 2 : 1)) return;
-    const int dir = (int)(t / per_dir);
-    const long long u = t - dir * per_dir;
-    const int k = (int)(u / a.ncp), cell = (int)(u - (long long)k * a.ncp);
-    const size_t P = a.ncp;
-    double *w = (dir ? a.Wt : a.W) + (size_t)k * a.b * P;
-    const double *src = (dir ? a.Vd : a.Ud) + (size_t)k * a.b * P;
-    for (int q = 0; q < a.b; ++q) w[q * P + cell] = src[q * P + cell];
-    if (dir) lu_solve_T(a, w, cell);
-    else lu_solve_N(a, w, cell);
-}
-
-// Setup step 3a, one thread per (cell, k, l): C_kl = delta_kl + V_k . W_l (FP64),
-// written into the C^-1 array, which step 3b inverts in place.
-__global__ void k_smw_cmat(SetupArgs a) {
-    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const int r = a.r;
-    if (t >= (long long)a.ncp * r * r) return;
-    const int kl = (int)(t / a.ncp), cell = (int)(t - (long long)kl * a.ncp);
-    const int k = kl / r, l = kl - k * r;
-    const size_t P = a.ncp;
-    const double *v = a.Vd + (size_t)k * a.b * P + cell, *w = a.W + (size_t)l * a.b * P + cell;
-    double acc = k == l ? 1.0 : 0.0;
-    for (int q = 0; q < a.b; ++q) acc = fma(v[q * P], w[q * P], acc);
-    a.Cinv[(size_t)kl * P + cell] = acc;
-}
-
-// Setup step 3b, one thread per cell: C^-1 by Gauss-Jordan with partial pivoting,
-// in place in the C^-1 array.
-__global__ void k_smw_cinv(SetupArgs a) {
-    const int cell = blockIdx.x * blockDim.x + threadIdx.x;
-    if (cell >= a.ncp) return;
-    const size_t P = a.ncp;
-    const int r = a.r;
-    double C[kMaxPairsDiag][kMaxPairsDiag], X[kMaxPairsDiag][kMaxPairsDiag];
-    double cmax = 0.0;
-    for (int k = 0; k < r; ++k)
-        for (int l = 0; l < r; ++l) {
-            C[k][l] = a.Cinv[((size_t)k * r + l) * P + cell];
-            X[k][l] = k == l ? 1.0 : 0.0;
-            cmax = fmax(cmax, fabs(C[k][l]));
-        }
-    for (int k = 0; k < r; ++k) {
-        int pr = k;
-        for (int i = k + 1; i < r; ++i)
-            if (fabs(C[i][k]) > fabs(C[pr][k])) pr = i;
-        if (!(fabs(C[pr][k]) > 1e-14 * cmax)) {
-            atomicMin(a.err_cell, cell);
-            return;
-        }
-        if (pr != k)
-            for (int j = 0; j < r; ++j) {
-                double t = C[k][j]; C[k][j] = C[pr][j]; C[pr][j] = t;
-                t = X[k][j]; X[k][j] = X[pr][j]; X[pr][j] = t;
-            }
-        const double d = 1.0 / C[k][k];
-        for (int j = 0; j < r; ++j) { C[k][j] *= d; X[k][j] *= d; }
-        for (int i = 0; i < r; ++i) {
-            if (i == k) continue;
-            const double f = C[i][k];
-            for (int j = 0; j < r; ++j) { C[i][j] -= f * C[k][j]; X[i][j] -= f * X[k][j]; }
-        }
-    }
-    for (int k = 0; k < r; ++k)
-        for (int l = 0; l < r; ++l) a.Cinv[((size_t)k * r + l) * P + cell] = X[k][l];
-}
-
-// Write the apply streams: forward coefficients, then per backward row its
-// pivot inverse followed by its coefficients (scaled by the row's dinv where the
-// program asks for it).
-template <typename T>
-__global__ void k_smw_pack(T *out, const double *lu, const double *dinv, const int *pk_slot,
-                           const int *pk_scale, int len, int ncp) {
-    const long long total = (long long)len * ncp;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total;
-         i += (long long)gridDim.x * blockDim.x) {
-        const int cell = (int)(i % ncp), pos = (int)(i / ncp);
-        const int sl = pk_slot[pos], sc = pk_scale[pos];
-        double v;
-        if (sl >= 0) {
-            v = lu[(size_t)sl * ncp + cell];
-            if (sc >= 0) v *= dinv[(size_t)sc * ncp + cell];
-        } else {
-            v = dinv[(size_t)sc * ncp + cell];
-        }
-        out[i] = (T)v;
-    }
-}
-
-template <typename T>
-__global__ void k_round(T *out, const double *in, long long n) {
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x)
-        out[i] = (T)in[i];
-}
 
 template <typename T>
 struct ApplyArgs {
@@ -686,87 +493,6 @@ fail:
     cp_async_wait<0>();
 }
 
-// Structured stream packing: per position a source code and argument
-//   src >= 0: LU slot (times the pivot inverse of row arg if arg >= 0)
-//   src = -1: pivot inverse of row arg      src = -2: dot vector entry arg
-//   src = -3: W entry arg                   src = -4: zero
-//   src = -5: folded tail entry arg = a * b + q: (W C^-1)[q][a] =
-//             sum_l W[l][q] C^-1[l][a], or for the transposed operator
-//             sum_l W'[l][q] C^-1[a][l] (C^-T), in FP64
-// Output element i is (tile, vector, lane, element) of the layout above.
-template <typename T>
-__global__ void k_smw_spack(T *out, const double *lu, const double *dinv, const double *DV, const double *WW,
-                            const double *Cinv, const int *src, const int *arg, int Lt, int ncp, int b, int r,
-                            int trans) {
-    constexpr int VEC = 16 / (int)sizeof(T);
-    const long long per_tile = (long long)Lt * kTile;
-    const long long total = per_tile * (ncp / kTile);
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total;
-         i += (long long)gridDim.x * blockDim.x) {
-        const long long tile = i / per_tile;
-        const int e = (int)(i - tile * per_tile);
-        const int pv = e / (kTile * VEC), rem = e - pv * kTile * VEC;
-        const int lane = rem / VEC, pos = pv * VEC + rem % VEC;
-        const int cell = (int)tile * kTile + lane;
-        const int sv = src[pos], ag = arg[pos];
-        double v = 0.0;
-        if (sv >= 0) {
-            v = lu[(size_t)sv * ncp + cell];
-            if (ag >= 0) v *= dinv[(size_t)ag * ncp + cell];
-        } else if (sv == -1) {
-            v = dinv[(size_t)ag * ncp + cell];
-        } else if (sv == -2) {
-            v = DV[(size_t)ag * ncp + cell];
-        } else if (sv == -3) {
-            v = WW[(size_t)ag * ncp + cell];
-        } else if (sv == -5) {
-            const int aa = ag / b, q = ag - aa * b;
-            for (int l = 0; l < r; ++l) {
-                const double c = Cinv[(size_t)(trans ? aa * r + l : l * r + aa) * ncp + cell];
-                v = fma(WW[((size_t)l * b + q) * ncp + cell], c, v);
-            }
-        }
-        out[i] = (T)v;
-    }
-}
-
-// Repack diagonal-block values into [entry][cell] and the diagonal pairs into
-// [k][q][cell]; a cell with fewer than r pairs gets zero pairs (u = v = 0 leaves
-// A_k unchanged and adds an identity row and column to C_k).
-__global__ void k_smw_repack(double *Sd, double *Ud, double *Vd, const double *S, const double *U,
-                             const double *V, const int *diag_blk, const long long *soff,
-                             const int *pbase, int nc, int ncp, int nnz_d, int b, int r) {
-    const long long nS = (long long)nnz_d * ncp, nP = (long long)r * b * ncp;
-    const long long total = nS + nP;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total;
-         i += (long long)gridDim.x * blockDim.x) {
-        if (i < nS) {
-            const int cell = (int)(i % ncp), e = (int)(i / ncp);
-            Sd[i] = cell < nc ? S[soff[diag_blk[cell]] + e] : 0.0;
-        } else {
-            const long long j = i - nS;
-            const int cell = (int)(j % ncp);
-            const long long kq = j / ncp;
-            const int q = (int)(kq % b), k = (int)(kq / b);
-            double u = 0.0, v = 0.0;
-            if (cell < nc && k < pbase[diag_blk[cell] + 1] - pbase[diag_blk[cell]]) {
-                const size_t src = (size_t)(pbase[diag_blk[cell]] + k) * b + q;
-                u = U[src];
-                v = V[src];
-            }
-            Ud[j] = u;
-            Vd[j] = v;
-        }
-    }
-}
-
-inline int grid_for(long long n, int block) {
-    long long g = (n + block - 1) / block;
-    if (g > 152LL * 64) g = 152LL * 64;
-    if (g < 1) g = 1;
-    return (int)g;
-}
-
 }  // namespace
 
 // Host: symbolic factorisation of the shared diagonal pattern and the programs
@@ -1008,6 +734,26 @@ sts_status smw_build(sts_jac_s *h) {
                     if (src[e] < -5 || (src[e] >= 0 && src[e] >= M.nnz_lu))
                         return set_error(STS_ERR_INVALID_ARG, "internal: structured apply table");
                 M.s_lt[prec] = (int)src.size();
+                if (sap_fold(RMAX, sw) && dir == 0) {       // positions of the folded tail, alike in both directions
+                    std::vector<int> tp((size_t)std::max(r, 1) * b, 0);
+                    for (size_t e = 0; e < src.size(); ++e)
+                        if (src[e] == -5) tp[arg[e]] = (int)e;
+                    STS_TRY(upload(h, &M.tail_pos[prec], tp));
+                }
+                // vectors to pack: those that scale an entry first; none for all zeros or folded tails
+                std::vector<int> list, plain;
+                for (int v = 0; v < (int)src.size() / vec; ++v) {
+                    bool any = false, scaled = false;
+                    for (int e = v * vec; e < (v + 1) * vec; ++e) {
+                        any = any || src[e] > -4;
+                        scaled = scaled || (src[e] >= 0 && arg[e] >= 0);
+                    }
+                    if (any) (scaled ? list : plain).push_back(v);
+                }
+                M.spk_scaled[prec][dir] = (int)list.size();
+                list.insert(list.end(), plain.begin(), plain.end());
+                M.spk_n[prec][dir] = (int)list.size();
+                STS_TRY(upload(h, &M.spk_list[prec][dir], list));
                 STS_TRY(upload(h, &M.spk_src[prec][dir], src));
                 STS_TRY(upload(h, &M.spk_arg[prec][dir], arg));
             }
@@ -1023,9 +769,11 @@ sts_status smw_build(sts_jac_s *h) {
     STS_TRY(upload(h, &M.f_upd_src, upd_src));
     const size_t P = h->ncp;
     const int r = h->r_diag;
-    STS_TRY(dalloc(h, &M.Sd, (size_t)h->nnz_d * P));
-    STS_TRY(dalloc(h, &M.Ud, (size_t)std::max(r, 1) * b * P));
-    STS_TRY(dalloc(h, &M.Vd, (size_t)std::max(r, 1) * b * P));
+    // zero in the padding cells and in the pairs that a block does not have (u = v = 0
+    // leaves A_k unchanged and adds an identity row and column to C_k)
+    STS_TRY(dalloc_zero(h, &M.Sd, (size_t)h->nnz_d * P));
+    STS_TRY(dalloc_zero(h, &M.Ud, (size_t)std::max(r, 1) * b * P));
+    STS_TRY(dalloc_zero(h, &M.Vd, (size_t)std::max(r, 1) * b * P));
     STS_TRY(dalloc(h, &M.lu, (size_t)M.nnz_lu * P));
     STS_TRY(dalloc(h, &M.dinv, (size_t)b * P));
     STS_TRY(dalloc(h, &M.W, (size_t)std::max(r, 1) * b * P));
@@ -1035,111 +783,15 @@ sts_status smw_build(sts_jac_s *h) {
         if (dir == 1 && !h->has_T) continue;
         const size_t len = M.structured ? (size_t)M.s_lt[0] : (size_t)M.n_fwd[dir] + M.n_bwd[dir] + b;
         const size_t len32 = M.structured ? (size_t)M.s_lt[1] : len;
-        STS_TRY(dalloc(h, &M.ap64[dir], len * P));
+        // the structured streams' zero padding is written here and never again
+        STS_TRY(dalloc_zero(h, &M.ap64[dir], len * P));
         if (h->dtype == STS_MIXED) {
-            STS_TRY(dalloc(h, &M.ap32[dir], len32 * P));
+            STS_TRY(dalloc_zero(h, &M.ap32[dir], len32 * P));
             STS_TRY(dalloc(h, &M.W32[dir], (size_t)std::max(r, 1) * b * P));
             STS_TRY(dalloc(h, &M.DV32[dir], (size_t)std::max(r, 1) * b * P));
         }
     }
     STS_TRY(dalloc(h, &M.err_cell, 1));
-    std::vector<int> diag_blk(h->nc);
-    for (int c = 0; c < h->nc; ++c)
-        for (int k = h->bptr[c]; k < h->bptr[c + 1]; ++k)
-            if (h->bidx[k] == c) diag_blk[c] = k;
-    STS_TRY(upload(h, &M.diag_blk, diag_blk));
-    return STS_OK;
-}
-
-sts_status smw_repack(sts_jac_s *h, const double *S, const double *U, const double *V) {
-    SmwPlan &M = h->smw;
-    M.ready = false;
-    const long long total = (long long)h->nnz_d * h->ncp + (long long)h->r_diag * h->b * h->ncp;
-    k_smw_repack<<<grid_for(total, 256), 256, 0, h->stream>>>(
-        M.Sd, M.Ud, M.Vd, S, U, V, M.diag_blk, h->d_soff, h->d_pbase, h->nc, h->ncp, h->nnz_d,
-        h->b, h->r_diag);
-    STS_LAUNCHED();
-    return STS_OK;
-}
-
-sts_status smw_setup(sts_jac_s *h) {
-    SmwPlan &M = h->smw;
-    M.ready = false;
-    SetupArgs a;
-    a.Sd = M.Sd; a.Ud = M.Ud; a.Vd = M.Vd;
-    a.lu = M.lu; a.dinv = M.dinv; a.W = M.W; a.Wt = M.Wt; a.Cinv = M.Cinv;
-    a.lu_diag = M.lu_diag; a.src_slot = M.src_slot; a.d_ptr = M.d_ptr;
-    a.colL_ptr = M.f_colL_ptr; a.colL_slot = M.f_colL_slot;
-    a.upd_ptr = M.f_upd_ptr; a.upd_tgt = M.f_upd_tgt; a.upd_src = M.f_upd_src;
-    a.fwd_ptr0 = M.ap_fwd_ptr[0]; a.fwd_col0 = M.ap_fwd_col[0]; a.fwd_slot0 = M.ap_fwd_slot[0];
-    a.bwd_ptr0 = M.ap_bwd_ptr[0]; a.bwd_col0 = M.ap_bwd_col[0]; a.bwd_slot0 = M.ap_bwd_slot[0];
-    a.fwd_ptr1 = M.ap_fwd_ptr[1]; a.fwd_col1 = M.ap_fwd_col[1]; a.fwd_slot1 = M.ap_fwd_slot[1];
-    a.bwd_ptr1 = M.ap_bwd_ptr[1]; a.bwd_col1 = M.ap_bwd_col[1]; a.bwd_slot1 = M.ap_bwd_slot[1];
-    a.err_cell = M.err_cell;
-    a.nc = h->nc; a.ncp = h->ncp; a.b = h->b; a.r = h->r_diag; a.nnz_lu = M.nnz_lu;
-    a.nnz_d = h->nnz_d; a.with_T = h->has_T ? 1 : 0;
-    const int big = INT_MAX;
-    STS_CK(cudaMemcpyAsync(M.err_cell, &big, sizeof(int), cudaMemcpyHostToDevice, h->stream));
-    k_smw_lu<<<(h->ncp + 63) / 64, 64, 0, h->stream>>>(a);
-    STS_LAUNCHED();
-    const long long nw = (long long)h->ncp * a.r * (a.with_T ? 2 : 1);
-    if (nw > 0) {
-        k_smw_w<<<(unsigned)((nw + 63) / 64), 64, 0, h->stream>>>(a);
-        STS_LAUNCHED();
-        const long long nc2 = (long long)h->ncp * a.r * a.r;
-        k_smw_cmat<<<(unsigned)((nc2 + 255) / 256), 256, 0, h->stream>>>(a);
-        STS_LAUNCHED();
-        k_smw_cinv<<<(h->ncp + 63) / 64, 64, 0, h->stream>>>(a);
-        STS_LAUNCHED();
-    }
-    int bad = INT_MAX;
-    STS_CK(cudaMemcpyAsync(&bad, M.err_cell, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
-    STS_CK(cudaStreamSynchronize(h->stream));
-    if (bad != INT_MAX)
-        return set_error(STS_ERR_SINGULAR,
-                         "block-Jacobi setup: cell %d has a pivot below 1e-14 x its row maximum "
-                         "(static pivot order) or a singular capacitance matrix C_k", bad);
-    const size_t P = h->ncp;
-    const int b = h->b, r = h->r_diag;
-    for (int dir = 0; dir < 2; ++dir) {
-        if (dir == 1 && !h->has_T) continue;
-        const double *DV = dir == 0 ? M.Vd : M.Ud;
-        const double *WW = dir == 0 ? M.W : M.Wt;
-        if (M.structured) {
-            const long long n64 = (long long)M.s_lt[0] * P;
-            k_smw_spack<double><<<grid_for(n64, 256), 256, 0, h->stream>>>(
-                M.ap64[dir], M.lu, M.dinv, DV, WW, M.Cinv, M.spk_src[0][dir], M.spk_arg[0][dir], M.s_lt[0],
-                h->ncp, b, r, dir);
-            STS_LAUNCHED();
-            if (M.ap32[dir]) {
-                const long long n32 = (long long)M.s_lt[1] * P;
-                k_smw_spack<float><<<grid_for(n32, 256), 256, 0, h->stream>>>(
-                    M.ap32[dir], M.lu, M.dinv, DV, WW, M.Cinv, M.spk_src[1][dir], M.spk_arg[1][dir], M.s_lt[1],
-                    h->ncp, b, r, dir);
-                STS_LAUNCHED();
-            }
-            continue;
-        }
-        const int len = M.n_fwd[dir] + M.n_bwd[dir] + b;
-        const long long n = (long long)len * P;
-        k_smw_pack<double><<<grid_for(n, 256), 256, 0, h->stream>>>(M.ap64[dir], M.lu, M.dinv, M.pk_slot[dir],
-                                                                     M.pk_scale[dir], len, h->ncp);
-        STS_LAUNCHED();
-        if (M.ap32[dir]) {
-            k_smw_pack<float><<<grid_for(n, 256), 256, 0, h->stream>>>(M.ap32[dir], M.lu, M.dinv, M.pk_slot[dir],
-                                                                       M.pk_scale[dir], len, h->ncp);
-            STS_LAUNCHED();
-            const long long nw = (long long)r * b * P;
-            if (nw > 0) {
-                k_round<float><<<grid_for(nw, 256), 256, 0, h->stream>>>(M.W32[dir], WW, nw);
-                STS_LAUNCHED();
-                k_round<float><<<grid_for(nw, 256), 256, 0, h->stream>>>(M.DV32[dir], DV, nw);
-                STS_LAUNCHED();
-            }
-        }
-    }
-    M.ready = true;
-    h->streams_dirty = true;
     return STS_OK;
 }
 

@@ -36,7 +36,7 @@ constexpr int kMaxPairsDiag = 16;  // rank-one pairs per diagonal block handled 
 //   kDescPair  the position is a pair term u_k[p] * c_k
 //   kDescEnd   the row is complete after this position
 constexpr unsigned kDescPair = 1u << 29;
-constexpr int kPosZero = -2147483647 - 1;     // repack code of a zero (padding) stream position
+constexpr int kPosZero = -2147483647 - 1;     // code of a zero (padding) stream position
 
 // Structured pattern family (the paper's StS blocks): the last kStructNF rows
 // of a block are dense "flow" rows; a level row p < N = b - kStructNF holds the
@@ -142,15 +142,12 @@ struct MvPlan {
     unsigned *slot_mask = nullptr;           // [n_tiles]: bit s set if any lane has slot s
     int *grp_rows = nullptr;                 // [n_groups+1]
     long long *row_off = nullptr;            // [b+1]
-    int *pslot_slot = nullptr;               // [n_pslots]
-    int *pslot_local = nullptr;              // [n_pslots]: index of the pair within its block
     int *pat_ptr = nullptr;                  // [2][b+1] pattern rows (kind 0 diag, 1 off), this direction
     int *pat_idx = nullptr;                  // [nnz_d + nnz_o] column indices (kind 1 after kind 0)
-    int *pat_src = nullptr;                  // [nnz_d + nnz_o] public entry index of each pattern entry
     int *dtask_slot = nullptr;               // [n_dtasks]: block slot whose x a dot task reads
-    int *dpos_kind = nullptr, *dpos_arg = nullptr;   // [n_dtasks*Lp]: pass-1 stream positions
-    int *pos_kind = nullptr;                 // [tile_len]: 0..n_slots-1 = S of that slot, -1-k = pair slot k
-    int *pos_arg = nullptr;                  // [tile_len]: pattern entry (S) or row p (pair)
+    int n_units = 0;                         // units of the values load (kernels_values.cu)
+    int4 *unit = nullptr;                    // [n_units]: slot, pair within its block or -1, first entry, entries
+    int2 *unit_dst = nullptr;                // [n_units][32]: pass-2 and pass-1 position of each entry, -1: none
     unsigned *desc = nullptr;                // [tile_len]: main-pass program (see kDescPair)
     double *main64 = nullptr;
     float *main32 = nullptr;
@@ -183,7 +180,6 @@ struct SmwPlan {
     int *d_ptr = nullptr;                        // diag pattern indptr (row max of S_ii)
     int *f_colL_ptr = nullptr, *f_colL_slot = nullptr;    // L entries of column k: slots (rows > k)
     int *f_upd_ptr = nullptr, *f_upd_tgt = nullptr, *f_upd_src = nullptr;  // per L entry: (i,j) -= l * (k,j)
-    int *diag_blk = nullptr;     // [nc] public block id of each cell's diagonal block
     // Apply programs per direction: forward rows i = 0..b-1 and backward rows
     // i = b-1..0 (index r = b-1-i), each a list of (column, LU slot).
     int *ap_fwd_ptr[2] = {nullptr, nullptr}, *ap_fwd_col[2] = {nullptr, nullptr};
@@ -216,6 +212,9 @@ struct SmwPlan {
     int s_w = 0, s_lt[2] = {0, 0};
     int *spk_src[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};
     int *spk_arg[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};
+    int *spk_list[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};   // vectors to pack, spk_scaled of them first
+    int spk_scaled[2][2] = {{0, 0}, {0, 0}}, spk_n[2][2] = {{0, 0}, {0, 0}};
+    int *tail_pos[2] = {nullptr, nullptr};      // [prec][r*b] stream positions of the folded tail (see k_smw_fold)
 };
 
 // Dense-BSR baseline (Section 3.4 storage).
@@ -318,14 +317,25 @@ inline sts_status dalloc(sts_jac_s *h, T **p, size_t n) {
     return dev_alloc(h, reinterpret_cast<void **>(p), n * sizeof(T));
 }
 template <typename T>
+inline sts_status dalloc_zero(sts_jac_s *h, T **p, size_t n) {
+    STS_TRY(dalloc(h, p, n));
+    if (n) STS_CK(cudaMemsetAsync(*p, 0, n * sizeof(T), h->stream));
+    return STS_OK;
+}
+template <typename T>
 inline sts_status upload(sts_jac_s *h, T **p, const std::vector<T> &v) {
     STS_TRY(dalloc(h, p, v.size() ? v.size() : 1));
     if (!v.empty()) STS_CK(cudaMemcpyAsync(*p, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice, h->stream));
     return STS_OK;
 }
 
+// kernels_values.cu
+sts_status values_plan(sts_jac_s *h, MvPlan &P, const std::vector<int> &pk, const std::vector<int> &pa,
+                       const std::vector<int> &dk, const std::vector<int> &da, const std::vector<int> (&src)[2],
+                       const std::vector<int> &pslot_slot, const std::vector<int> &pslot_local);
+sts_status values_load(sts_jac_s *h, int dir, const double *S, const double *U, const double *V);
+
 // kernels_matvec.cu
-sts_status mv_repack(sts_jac_s *h, int dir, const double *S, const double *U, const double *V);
 sts_status mv_apply64(sts_jac_s *h, int dir, const double *x, double *y, double *c);
 sts_status mv_apply32(sts_jac_s *h, int dir, const float *x, float *y, float *c);
 sts_status mv_dots64(sts_jac_s *h, int dir, const double *x, double *c);   // pass 1 only
@@ -337,7 +347,6 @@ sts_status from_internal32(sts_jac_s *h, const float *xi, float *x);
 
 // kernels_smw.cu
 sts_status smw_build(sts_jac_s *h);                       // host schedule + device tables
-sts_status smw_repack(sts_jac_s *h, const double *S, const double *U, const double *V);
 sts_status smw_setup(sts_jac_s *h);
 sts_status check_device(sts_jac_s *h);                   // STS_ERR_TIMEOUT if a bounded device wait gave up
 sts_status smw_apply64(sts_jac_s *h, int dir, const double *x, double *z);
