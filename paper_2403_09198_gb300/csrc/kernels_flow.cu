@@ -2,25 +2,25 @@
 // model (Section 2.1 model, Section 3.2 Eq. HLL_flux, Section 3.3 Eq.
 // system_residual, Section 4.1 Eqs. r1_flux_left / r1_flux_right).
 //
-// One warp per cell: the lanes sum the species terms of a state (mixture
-// density, gas constant, heat capacity, energy at T = 0) with a fixed
-// shuffle tree and broadcast lane 0's result, so every lane holds the same
-// scalars and takes the same wave-speed branch.  Per face the warp forms the
-// HLL bounds s_L, s_R, the coefficients a_f, c_f and their gradients, writes the
-// face's two rank-one pairs into the diagonal block of its cell and into the
-// neighbour block, and the neighbour block's sparse part dt A0_R; the diagonal
-// block's sparse part H + dt (sum A0_L + K) is written last.  Every face is
-// evaluated from both of its cells (once per block row), which keeps the writes
-// of a block row in one warp: no atomics, deterministic.
+// k_flow_mix forms every cell's mixture scalars (lane = cell), k_flow_face_* the
+// scalars of 8 cells and their 32 directed faces (lane = (cell, face)); k_flow_jac and
+// k_flow_res then run one warp per cell, lanes over the species.
+// Every face is evaluated from both of its cells (once per block row), which keeps
+// the writes of a block row in one warp: no atomics, deterministic.
 //
-// These kernels are bound by the FP64 pipe (a warp-wide FP64 instruction holds
-// a sub-partition's pipe for 64 cycles), so the FP64 work per entry is kept
-// small.  A_n is linear in the normal, so the diagonal block's face sum
-// sum_f (1/2 + a_f) A_{n_f}(q_i) is A_n(q_i) at the summed normal.  Level rows,
-// whose entries of A_n and H are u_n, rho_p n and 1, are written from four
-// per-face coefficient sums with lanes over rows; only the three dense flow rows
-// evaluate A_n and H entry by entry (lanes over columns), once per block;
-// reciprocals are formed once per face and per state, not per component.
+// A warp-wide FP64 instruction holds a sub-partition's pipe for 64 cycles whatever the
+// number of lanes that need it, so nothing scalar is computed by a whole warp, and
+// every entry that varies over the species is written as an affine form of q_c, r_c,
+// cv_c and e0_c with coefficients formed once per face: about 72 FP64 operations per
+// cell and species (10 per face for the four pair vectors, 5 per block for S).  A_n is
+// linear in the normal, so the diagonal block's face sum sum_f (1/2 + a_f) A_{n_f}(q_i)
+// is A_n(q_i) at the summed normal.
+//
+// Measured on 128 x 128 cells, N = 60 (band 2): Jacobian (571 MB written) 1326 us with the
+// scalars formed by every warp and every entry on its own, now 27 + 28 + 238 us (scalars
+// of cells, of faces, entries); residual 540 us, now 33 + 12 + 47.  The entries keep the
+// FP64 pipe 63% busy (134 of the 238 us are pipe time); more warps per SM or four faces
+// at once without branches between them left the time as it was.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -33,130 +33,129 @@
 namespace sts {
 namespace {
 
-constexpr int kFlowWarps = 4;     // cells (warps) per block
+constexpr int kMixCells = 32;     // cells per block of k_flow_mix
+constexpr int kFlowCells = 8;     // cells per warp of k_flow_face (8 x 4 faces) and per block of the kernels after it
+
+// Per-cell scalars, component-major: M[field * nc + cell].
+enum { mRho, mR, mC, mU, mV, mT, mKe, mP, mE, mA, mG0, mG1, mG2, mGT, mKap, mSb, kMixFields };
 
 struct FlowDev {
     int Lx, nc, N, b, w, nnz_d, nnz_o;
     const double *r, *cv, *e0, *beta, *ws, *K;
+    const double *dtK;      // dt K, plus 1 on the diagonal
     double A, theta, dt;
     const int *bptr, *bidx, *pip;
     const long long *soff;
     const int *d_ptr;       // row starts of the diagonal pattern (the neighbour pattern's are 4p, then 4N + b (p-N))
+    const short2 *d_pq;     // (row, column) of the diagonal pattern's level-row entries
+    double *mix;            // [2][kMixFields][nc]: scalars of Q, then of Qn
+    double *face;           // [blocks of 8 cells][kFaceFields][32 faces]: coefficients of the faces
+    double *cell;           // [blocks of 8 cells][kCellFields][8 cells]: of the diagonal blocks
 };
 
 struct Mix {
-    double rho, Rt, Ct, E0, u, v, T, ke, p, rhoetot, g, a;
-    double cga, gaT;        // T / (2 a rho C) and a / (2 T): the factors of da/dq
+    double rho, R, C, u, v, T, ke, p, e, a;      // e: rho e_tot
 };
 
-// Sum over the warp, the same value on every lane (tree to lane 0, then broadcast).
-__device__ __forceinline__ double warp_total(double x) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
-    return __shfl_sync(0xffffffffu, x, 0);
-}
-
-__device__ Mix mixture(const FlowDev &F, const double *q, int lane) {
-    double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
-    for (int k = lane; k < F.N; k += 32) {
-        const double rk = q[k];
-        s0 += rk;
-        s1 += rk * F.r[k];
-        s2 += rk * F.cv[k];
-        s3 += rk * F.e0[k];
-    }
+__device__ __forceinline__ Mix mix_of(const double *M, int nc, int i) {
     Mix m;
-    m.rho = warp_total(s0);
-    m.Rt = warp_total(s1);
-    m.Ct = warp_total(s2);
-    m.E0 = warp_total(s3);
-    m.u = q[F.N];
-    m.v = q[F.N + 1];
-    m.T = q[F.N + 2];
-    m.ke = 0.5 * (m.u * m.u + m.v * m.v);
-    m.p = m.Rt * m.T;
-    m.rhoetot = m.E0 + m.Ct * m.T + m.rho * m.ke;
-    m.g = (m.Ct + m.Rt) * m.Rt / (m.rho * m.Ct);
-    m.a = sqrt(m.g * m.T);
-    m.cga = m.T / (2.0 * m.a * m.rho * m.Ct);
-    m.gaT = m.a / (2.0 * m.T);
+    m.rho = M[mRho * (size_t)nc + i];
+    m.R = M[mR * (size_t)nc + i];
+    m.C = M[mC * (size_t)nc + i];
+    m.u = M[mU * (size_t)nc + i];
+    m.v = M[mV * (size_t)nc + i];
+    m.T = M[mT * (size_t)nc + i];
+    m.ke = M[mKe * (size_t)nc + i];
+    m.p = M[mP * (size_t)nc + i];
+    m.e = M[mE * (size_t)nc + i];
+    m.a = M[mA * (size_t)nc + i];
     return m;
 }
 
-// component c of the conserved variables u(q) and of the normal flux f_n(q)
-__device__ __forceinline__ double cons_c(const FlowDev &F, const double *q, const Mix &m, int c) {
-    if (c < F.N) return q[c];
-    if (c == F.N) return m.rho * m.u;
-    if (c == F.N + 1) return m.rho * m.v;
-    return m.rhoetot;
-}
-
-__device__ __forceinline__ double flux_c(const FlowDev &F, const double *q, const Mix &m, double nx, double ny,
-                                         int c) {
-    const double un = nx * m.u + ny * m.v;
-    if (c < F.N) return q[c] * un;
-    if (c == F.N) return m.rho * m.u * un + m.p * nx;
-    if (c == F.N + 1) return m.rho * m.v * un + m.p * ny;
-    return (m.rhoetot + m.p) * un;
-}
-
-// entry (p, c) of H = du/dq
-__device__ double H_e(const FlowDev &F, const Mix &m, int p, int c) {
-    const int N = F.N;
-    if (p < N) return c == p ? 1.0 : 0.0;
-    if (p == N) return c < N ? m.u : c == N ? m.rho : 0.0;
-    if (p == N + 1) return c < N ? m.v : c == N + 1 ? m.rho : 0.0;
-    if (c < N) return F.e0[c] + F.cv[c] * m.T + m.ke;
-    if (c == N) return m.rho * m.u;
-    if (c == N + 1) return m.rho * m.v;
-    return m.Ct;
-}
-
-// entry (p, c) of A_n = d f_n / dq
-__device__ double An_e(const FlowDev &F, const double *q, const Mix &m, double nx, double ny, int p, int c) {
-    const int N = F.N;
-    const double un = nx * m.u + ny * m.v;
-    if (p < N) {
-        if (c == p) return un;
-        if (c == N) return q[p] * nx;
-        if (c == N + 1) return q[p] * ny;
-        return 0.0;
+// Species sums and scalars of the states Q (blockIdx.y = 0) and Qn (1), one lane per
+// cell: the 32 rows are staged in shared memory with an odd stride, each of four
+// warps adds every fourth species in four interleaved sums.  A warp-wide sum over
+// species, one cell at a time, costs 28 FP64 instructions a state against 5 N / 32,
+// and the Jacobian needed it at the cell and at each of its neighbours.
+// da/dq_c = G0 + G1 cv_c + G2 r_c for a species (from a^2 = T g, g = (C + R) R / (rho C),
+// with R - g rho = -R^2 / C), GT for T, 0 for the velocities.
+__global__ void __launch_bounds__(128) k_flow_mix(FlowDev F, const double *Q, const double *Qn) {
+    extern __shared__ double rows[];             // [32][b | 1], species constants [N][4], partial sums [4][5][32]
+    const int b = F.b, N = F.N, st = b | 1, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int c0 = blockIdx.x * kMixCells, n = min(kMixCells, F.nc - c0);
+    const double *src = (blockIdx.y ? Qn : Q) + (size_t)c0 * b;
+    double *cst = rows + 32 * st;
+    double(*part)[5][32] = reinterpret_cast<double(*)[5][32]>(cst + 4 * N);
+    for (int k = threadIdx.x; k < N; k += 128) {
+        cst[4 * k] = __ldg(F.r + k);
+        cst[4 * k + 1] = __ldg(F.cv + k);
+        cst[4 * k + 2] = __ldg(F.e0 + k);
+        cst[4 * k + 3] = __ldg(F.beta + k);
     }
-    if (p == N) {
-        if (c < N) return m.u * un + F.r[c] * m.T * nx;
-        if (c == N) return m.rho * un + m.rho * m.u * nx;
-        if (c == N + 1) return m.rho * m.u * ny;
-        return m.Rt * nx;
+#pragma unroll 4
+    for (int e = threadIdx.x; e < n * b; e += 128) {
+        const int c = e / b;
+        rows[c * st + e - c * b] = __ldg(src + e);
     }
-    if (p == N + 1) {
-        if (c < N) return m.v * un + F.r[c] * m.T * ny;
-        if (c == N) return m.rho * m.v * nx;
-        if (c == N + 1) return m.rho * un + m.rho * m.v * ny;
-        return m.Rt * ny;
+    __syncthreads();
+    const double *q = rows + min(lane, n - 1) * st;
+    double s[4][5] = {};
+    for (int k = warp; k < N; k += 16) {
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+            const int kk = k + 4 * h;
+            if (kk >= N) break;
+            const double x = q[kk];
+            s[h][0] += x;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) s[h][j + 1] = fma(x, cst[4 * kk + j], s[h][j + 1]);
+        }
     }
-    if (c < N) return (F.e0[c] + F.cv[c] * m.T + m.ke + F.r[c] * m.T) * un;
-    if (c == N) return m.rho * m.u * un + (m.rhoetot + m.p) * nx;
-    if (c == N + 1) return m.rho * m.v * un + (m.rhoetot + m.p) * ny;
-    return (m.Ct + m.Rt) * un;
-}
-
-// component c of da/dq: a^2 = T g, g = (C + R) R / (rho C)
-__device__ double grad_a_c(const FlowDev &F, const Mix &m, int c) {
-    if (c < F.N) {
-        const double dn = (F.cv[c] + F.r[c]) * m.Rt + (m.Ct + m.Rt) * F.r[c];
-        const double dd = m.Ct + m.rho * F.cv[c];
-        return m.cga * (dn - m.g * dd);
+#pragma unroll
+    for (int j = 0; j < 5; ++j) part[warp][j][lane] = (s[0][j] + s[1][j]) + (s[2][j] + s[3][j]);
+    __syncthreads();
+    if (lane >= n) return;
+    auto total = [&](int j) { return (part[0][j][lane] + part[1][j][lane]) + (part[2][j][lane] + part[3][j][lane]); };
+    const double T = q[N + 2];
+    double *M = F.mix + (size_t)blockIdx.y * kMixFields * F.nc + c0 + lane;
+    const size_t P = F.nc;
+    // the scalars' dependent chains on a warp each
+    if (warp == 0) {
+        const double rho = total(0), R = total(1), C = total(2);
+        const double g = (C + R) * R / (rho * C), a = sqrt(g * T);
+        M[mA * P] = a;
+        if (blockIdx.y) return;                  // Qn gives the conserved variables only
+        const double cga = T / (2.0 * a * rho * C);
+        M[mG0 * P] = -cga * ((C + R) * R / rho);
+        M[mG1 * P] = -cga * (R * R / C);
+        M[mG2 * P] = cga * (2.0 * R + C);
+        M[mGT * P] = a / (2.0 * T);
+    } else if (warp == 1) {
+        const double rho = total(0), R = total(1), C = total(2), u = q[N], v = q[N + 1];
+        const double ke = 0.5 * (u * u + v * v);
+        M[mRho * P] = rho;
+        M[mR * P] = R;
+        M[mC * P] = C;
+        M[mU * P] = u;
+        M[mV * P] = v;
+        M[mT * P] = T;
+        M[mKe * P] = ke;
+        M[mP * P] = R * T;
+        M[mE * P] = total(3) + C * T + rho * ke;
+    } else if (warp == 2) {
+        M[mKap * P] = F.A * exp(-F.theta / T);
+        M[mSb * P] = total(4);
     }
-    return c == F.N + 2 ? m.gaT : 0.0;
 }
 
 struct Face {
-    double nx, ny, sL, sR, af, cf, inv_den, inv_den2;
+    double nx, ny, sL, sR, inv_den;
     int iL, iR;
 };
 
-// HLL bounds and coefficients of the face from cell L to cell R
-__device__ Face face_of(const Mix &mL, const Mix &mR, double nx, double ny) {
+// HLL bounds of the face from cell L to cell R: the extreme of 0, L's and R's
+// wave speed, ties to the first; iL, iR name the one taken
+__device__ __forceinline__ Face face_of(const Mix &mL, const Mix &mR, double nx, double ny) {
     Face f;
     f.nx = nx;
     f.ny = ny;
@@ -169,14 +168,7 @@ __device__ Face face_of(const Mix &mL, const Mix &mR, double nx, double ny) {
     f.iR = 0;
     if (unL + mL.a > f.sR) { f.sR = unL + mL.a; f.iR = 1; }
     if (unR + mR.a > f.sR) { f.sR = unR + mR.a; f.iR = 2; }
-    // a_f and c_f by division: on a supersonic face a_f is exactly +-1/2 and the
-    // upwind side's weight 1/2 -+ a_f exactly zero; the per-component products
-    // use the reciprocal
-    const double den = f.sR - f.sL;
-    f.af = 0.5 * (f.sL + f.sR) / den;
-    f.cf = f.sL * f.sR / den;
-    f.inv_den = 1.0 / den;
-    f.inv_den2 = f.inv_den * f.inv_den;
+    f.inv_den = 1.0 / (f.sR - f.sL);
     return f;
 }
 
@@ -190,155 +182,393 @@ __device__ __forceinline__ void normal_of(int Lx, int i, int j, double &nx, doub
     }
 }
 
-__global__ void __launch_bounds__(kFlowWarps * 32) k_flow_jac(FlowDev F, const double *Q, double *S, double *U,
-                                                               double *V) {
-    const int lane = threadIdx.x & 31;
-    const int i = blockIdx.x * kFlowWarps + (threadIdx.x >> 5);
-    if (i >= F.nc) return;
-    const int b = F.b, N = F.N, w = F.w;
-    const double dt = F.dt;
-    const double *qi = Q + (size_t)i * b;
-    const Mix mi = mixture(F, qi, lane);
-    const int k0 = F.bptr[i], k1 = F.bptr[i + 1];
-    int kd = k0;
+// Lane = (cell, face) of a block's cells: the face's neighbour block, its cell and
+// the number of faces; false for a lane without a face.
+struct FaceLane {
+    int i, f, nf, kd, k, j;
+    bool on;
+};
+__device__ __forceinline__ FaceLane face_lane(const FlowDev &F, int blk, int lane) {
+    FaceLane L;
+    L.i = blk * kFlowCells + (lane >> 2);
+    L.f = lane & 3;
+    L.on = L.i < F.nc;
+    if (!L.on) L.i = F.nc - 1;
+    const int k0 = F.bptr[L.i], k1 = F.bptr[L.i + 1];
+    L.nf = k1 - k0 - 1;
+    L.kd = k0;
     for (int k = k0; k < k1; ++k)
-        if (F.bidx[k] == i) kd = k;
-    int nf = 0;
-    // sums over the faces for the diagonal block:
-    // sum (1/2 + a_f) u_n(q_i), sum c_f, sum (1/2 + a_f) n_x, sum (1/2 + a_f) n_y
-    double cun = 0.0, ccf = 0.0, cnx = 0.0, cny = 0.0;
-    for (int k = k0; k < k1 && nf < 4; ++k) {
-        const int j = F.bidx[k];
-        if (j == i) continue;
-        const double *qj = Q + (size_t)j * b;
-        const Mix mj = mixture(F, qj, lane);
-        double nx, ny;
-        normal_of(F.Lx, i, j, nx, ny);
-        const Face f = face_of(mi, mj, nx, ny);
-        const double wL = 0.5 + f.af, wR = 0.5 - f.af;
-        cun += wL * (nx * mi.u + ny * mi.v);
-        ccf += f.cf;
-        cnx += wL * nx;
-        cny += wL * ny;
-        // neighbour block dt A0_R = dt ((1/2 - a_f) A_n(q_j) + c_f H(q_j)):
-        // level row p holds (p, p) = u_n(q_j) and 1, (p, N) = rho_p n_x, (p, N+1) = rho_p n_y, (p, N+2) = 0
-        double *Sk = S + F.soff[k];
-        const double unj = nx * mj.u + ny * mj.v;
-        for (int p = lane; p < N; p += 32) {
-            const double wq = wR * qj[p];
-            Sk[4 * p] = dt * (wR * unj + f.cf);
-            Sk[4 * p + 1] = dt * (wq * nx);
-            Sk[4 * p + 2] = dt * (wq * ny);
-            Sk[4 * p + 3] = 0.0;
-        }
-        for (int e = lane; e < 3 * b; e += 32) {
-            const int p = N + e / b, c = e - (e / b) * b;
-            Sk[4 * N + e] = dt * (wR * An_e(F, qj, mj, nx, ny, p, c) + f.cf * H_e(F, mj, p, c));
-        }
-        // the face's two pairs: into the diagonal block (d/dq_i) and the neighbour block (d/dq_j)
-        const size_t pd = (size_t)(F.pip[kd] + 1 + 2 * nf), po = (size_t)F.pip[k];
-        for (int c = lane; c < b; c += 32) {
-            const double u1 = -(flux_c(F, qj, mj, nx, ny, c) - flux_c(F, qi, mi, nx, ny, c));
-            const double u2 = cons_c(F, qj, mj, c) - cons_c(F, qi, mi, c);
-            const double gun = c == N ? nx : c == N + 1 ? ny : 0.0;
-            const double gaL = grad_a_c(F, mi, c), gaR = grad_a_c(F, mj, c);
-            const double dsLL = f.iL == 1 ? gun - gaL : 0.0, dsLR = f.iL == 2 ? gun - gaR : 0.0;
-            const double dsRL = f.iR == 1 ? gun + gaL : 0.0, dsRR = f.iR == 2 ? gun + gaR : 0.0;
-            U[pd * b + c] = dt * u1;
-            V[pd * b + c] = (f.sR * dsLL - f.sL * dsRL) * f.inv_den2;
-            U[(pd + 1) * b + c] = dt * u2;
-            V[(pd + 1) * b + c] = (f.sR * f.sR * dsLL - f.sL * f.sL * dsRL) * f.inv_den2;
-            U[po * b + c] = dt * u1;
-            V[po * b + c] = (f.sR * dsLR - f.sL * dsRR) * f.inv_den2;
-            U[(po + 1) * b + c] = dt * u2;
-            V[(po + 1) * b + c] = (f.sR * f.sR * dsLR - f.sL * f.sL * dsRR) * f.inv_den2;
-        }
-        ++nf;
-    }
-    // diagonal block H(q_i) + dt K + sum over faces dt A0_L: level row p holds the
-    // band (K, plus H = 1 and the face terms on the diagonal), then (p, N), (p, N+1), (p, N+2)
-    double *Sd = S + F.soff[kd];
-    for (int p = lane; p < N; p += 32) {
-        double *row = Sd + F.d_ptr[p];
-        const int c0 = max(0, p - w), c1 = min(N - 1, p + w);
-        const double *Kp = F.K + (size_t)p * (2 * w + 1) - p + w;      // Kp[c] = K[p][c - p + w]
-        for (int c = c0; c <= c1; ++c) {
-            const double kb = dt * Kp[c];
-            row[c - c0] = c == p ? (1.0 + kb) + dt * (cun - ccf) : kb;
-        }
-        const double qp = dt * qi[p];
-        row[c1 - c0 + 1] = qp * cnx;
-        row[c1 - c0 + 2] = qp * cny;
-        row[c1 - c0 + 3] = 0.0;
-    }
-    // flow rows: A_n is linear in n, so sum_f (1/2 + a_f) A_{n_f}(q_i) = A_{(cnx, cny)}(q_i)
-    // (K is zero on the flow rows)
-    double *Sf = Sd + F.d_ptr[N];
-    for (int e = lane; e < 3 * b; e += 32) {
-        const int p = N + e / b, c = e - (e / b) * b;
-        const double h = H_e(F, mi, p, c);
-        Sf[e] = h + dt * (An_e(F, qi, mi, cnx, cny, p, c) - ccf * h);
-    }
-    // source pair (-dt ws, d omega / dq)
-    double sb = 0.0;
-    for (int k = lane; k < N; k += 32) sb += F.beta[k] * qi[k];
-    sb = warp_total(sb);
-    const double kap = F.A * exp(-F.theta / mi.T);
-    const double kT = kap * F.theta / (mi.T * mi.T) * sb;
-    const size_t ps = (size_t)F.pip[kd];
-    for (int c = lane; c < b; c += 32) {
-        U[ps * b + c] = c < N ? -dt * F.ws[c] : 0.0;
-        V[ps * b + c] = c < N ? kap * F.beta[c] : c == N + 2 ? kT : 0.0;
-    }
+        if (F.bidx[k] == L.i) L.kd = k;
+    L.on = L.on && L.f < L.nf;
+    L.k = L.on ? k0 + L.f + (k0 + L.f >= L.kd ? 1 : 0) : L.kd;
+    L.j = F.bidx[L.k];
+    return L;
 }
 
-__global__ void __launch_bounds__(kFlowWarps * 32) k_flow_res(FlowDev F, const double *Q, const double *Qn,
-                                                               double *R) {
-    const int lane = threadIdx.x & 31;
-    const int i = blockIdx.x * kFlowWarps + (threadIdx.x >> 5);
-    if (i >= F.nc) return;
-    const int b = F.b, N = F.N;
-    const double *qi = Q + (size_t)i * b, *qn = Qn + (size_t)i * b;
-    const Mix mi = mixture(F, qi, lane), mn = mixture(F, qn, lane);
-    double sb = 0.0;
-    for (int k = lane; k < N; k += 32) sb += F.beta[k] * qi[k];
-    sb = warp_total(sb);
-    const double omega = F.A * exp(-F.theta / mi.T) * sb;
-    // components c = lane + 32 t, at most 8 per lane (b <= 256)
-    constexpr int kMaxPerLane = 8;
-    double fsum[kMaxPerLane];
+// Sum of x over a cell's faces, in face order, on the lane of its first face.
+__device__ __forceinline__ double face_sum(double x, int lane, int nf) {
+    double s = x;
 #pragma unroll
-    for (int t = 0; t < kMaxPerLane; ++t) fsum[t] = 0.0;
-    const int k0 = F.bptr[i], k1 = F.bptr[i + 1];
-    for (int k = k0; k < k1; ++k) {
-        const int j = F.bidx[k];
-        if (j == i) continue;
-        const double *qj = Q + (size_t)j * b;
-        const Mix mj = mixture(F, qj, lane);
-        double nx, ny;
-        normal_of(F.Lx, i, j, nx, ny);
-        const Face f = face_of(mi, mj, nx, ny);
+    for (int f = 1; f < 4; ++f) {
+        const double y = __shfl_sync(0xffffffffu, x, (lane & ~3) + f);
+        if (f < nf) s += y;
+    }
+    return s;
+}
+
+// Coefficients of one block's entries: with q the block's state, level row p
+// holds diag on (p, p) and cx q_p, cy q_p in the first two flow columns; flow row N + e
+// holds mx + mxr r_c, my + myr r_c and h0 + he e0_c + hc cv_c + hr r_c in the level
+// columns and corner[e][.] in the flow columns.
+struct BlockCoef {
+    double diag, cx, cy, mx, mxr, my, myr, h0, he, hc, hr, corner[3][3];
+};
+
+// Block ax A_x + ay A_y + h H of the state m (H = du/dq, A_n the flux Jacobian, linear
+// in the normal), where (ax, ay) is the weighted normal.
+__device__ __forceinline__ BlockCoef block_coef(const Mix &m, double ax, double ay, double h) {
+    const double un = ax * m.u + ay * m.v, w = un + h, H = m.e + m.p;
+    BlockCoef B;
+    B.diag = w;
+    B.cx = ax;
+    B.cy = ay;
+    B.mx = m.u * w;
+    B.mxr = m.T * ax;
+    B.my = m.v * w;
+    B.myr = m.T * ay;
+    B.he = w;
+    B.h0 = w * m.ke;
+    B.hc = w * m.T;
+    B.hr = un * m.T;
+    const double ru = m.rho * m.u, rv = m.rho * m.v;
+    B.corner[0][0] = fma(m.rho, w, ru * ax);
+    B.corner[0][1] = ru * ay;
+    B.corner[0][2] = m.R * ax;
+    B.corner[1][0] = rv * ax;
+    B.corner[1][1] = fma(m.rho, w, rv * ay);
+    B.corner[1][2] = m.R * ay;
+    B.corner[2][0] = fma(ru, w, H * ax);
+    B.corner[2][1] = fma(rv, w, H * ay);
+    B.corner[2][2] = fma(m.C, w, m.R * un);
+    return B;
+}
+
+// Fields of the coefficient arrays.  Block coefficients take kBlockFields from their first.
+constexpr int kBlockFields = 20;
+enum { fUi, fUj,            // U of the first pair: ui q_i - uj q_j (both with dt)
+       fG,                  // V of a species: g da/dq, pairs 1 and 2 of q_i, pairs 1 and 2 of q_j
+       fU = fG + 4,         // flow components of the pairs: U [2][3], V [4][3]
+       fV = fU + 6,
+       fB = fV + 12,        // the neighbour block
+       fH = fB + kBlockFields,      // da/dq of q_j: G0, G1, G2
+       kFaceFields = fH + 3 };
+enum { cKap, cVT,           // source pair: kap beta_c, and its T component
+       cB,                  // the diagonal block (without the band K and H's identity)
+       kCellFields = cB + kBlockFields };
+enum { rB, rD };            // residual: fields of a face (of the same array) ...
+enum { rA, rOm };           // ... and of a cell
+enum { bDiag, bCx, bCy, bMx, bMxr, bMy, bMyr, bH0, bHe, bHc, bHr, bCorner };      // BlockCoef in order
+static_assert(bCorner + 9 == kBlockFields, "block coefficients");
+
+// Scalars of 8 cells and their 32 directed faces, one warp, lane = (cell, face), each
+// face from both of its cells.  In a kernel of its own: as the first step of the
+// kernels that use the coefficients it left seven of eight warps waiting at a barrier
+// (k_flow_jac 280 us on 128 x 128 cells, N = 60).
+__global__ void __launch_bounds__(64) k_flow_face_jac(FlowDev F) {
+    const int lane = threadIdx.x & 31, blk = blockIdx.x * 2 + (threadIdx.x >> 5), nc = F.nc;
+    if (blk * kFlowCells >= nc) return;
+    const double dt = F.dt;
+    const double *M = F.mix;
+    const FaceLane L = face_lane(F, blk, lane);
+    const Mix mi = mix_of(M, nc, L.i), mj = mix_of(M, nc, L.j);
+    double nx, ny;
+    normal_of(F.Lx, L.i, L.j, nx, ny);
+    const Face f = face_of(mi, mj, nx, ny);
+    // a_f and c_f by division: on a supersonic face a_f is exactly +-1/2 and the
+    // upwind side's weight 1/2 -+ a_f exactly zero
+    const double den = f.sR - f.sL, sum = f.sL + f.sR;
+    const double af = L.on ? 0.5 * sum / den : -0.5, cf = L.on ? f.sL * f.sR / den : 0.0;
+    const double wL = 0.5 + af, wR = 0.5 - af;
+    const double uni = nx * mi.u + ny * mi.v, unj = nx * mj.u + ny * mj.v;
+    double *o = F.face + (size_t)blk * kFaceFields * 32 + lane;
+    auto put = [&](int field, double v) { o[field * 32] = v; };
+    put(fUi, dt * uni);
+    put(fUj, dt * unj);
+    const double fi[3] = {mi.rho * mi.u * uni + mi.p * nx, mi.rho * mi.v * uni + mi.p * ny, (mi.e + mi.p) * uni};
+    const double fj[3] = {mj.rho * mj.u * unj + mj.p * nx, mj.rho * mj.v * unj + mj.p * ny, (mj.e + mj.p) * unj};
+    const double ci[3] = {mi.rho * mi.u, mi.rho * mi.v, mi.e}, cj[3] = {mj.rho * mj.u, mj.rho * mj.v, mj.e};
 #pragma unroll
-        for (int t = 0; t < kMaxPerLane; ++t) {
-            const int c = lane + 32 * t;
-            if (c < b) {
-                const double fL = flux_c(F, qi, mi, nx, ny, c), fR = flux_c(F, qj, mj, nx, ny, c);
-                const double uL = cons_c(F, qi, mi, c), uR = cons_c(F, qj, mj, c);
-                fsum[t] = fsum[t] + (f.sR * fL - f.sL * fR + f.sL * f.sR * (uR - uL)) * f.inv_den;
+    for (int e = 0; e < 3; ++e) {
+        put(fU + e, dt * (fi[e] - fj[e]));
+        put(fU + 3 + e, dt * (cj[e] - ci[e]));
+    }
+    // V = (sR^k dsL - sL^k dsR) / den^2 (k = 1, 2) with dsL = n - da where this side
+    // gives s_L, dsR = n + da where it gives s_R: A n - G da, n along the velocities
+    const double i2 = f.inv_den * f.inv_den;
+    auto pair = [&](bool l, bool r, int s, double gT) {
+        double A1 = 0.0, G1 = 0.0, A2 = 0.0, G2 = 0.0;
+        if (l && r) {
+            A1 = f.inv_den;
+            G1 = sum * i2;
+            A2 = sum * f.inv_den;
+            G2 = (f.sR * f.sR + f.sL * f.sL) * i2;
+        } else if (l) {
+            A1 = G1 = f.sR * i2;
+            A2 = G2 = f.sR * f.sR * i2;
+        } else if (r) {
+            G1 = f.sL * i2;
+            G2 = f.sL * f.sL * i2;
+            A1 = -G1;
+            A2 = -G2;
+        }
+        put(fG + s, -G1);
+        put(fG + s + 1, -G2);
+        put(fV + 3 * s, A1 * nx);
+        put(fV + 3 * s + 1, A1 * ny);
+        put(fV + 3 * s + 2, -G1 * gT);
+        put(fV + 3 * s + 3, A2 * nx);
+        put(fV + 3 * s + 4, A2 * ny);
+        put(fV + 3 * s + 5, -G2 * gT);
+    };
+    pair(f.iL == 1, f.iR == 1, 0, M[mGT * (size_t)nc + L.i]);
+    pair(f.iL == 2, f.iR == 2, 2, M[mGT * (size_t)nc + L.j]);
+    auto put_block = [&](double *to, int stride, const BlockCoef &B) {
+        const double v[bCorner] = {B.diag, B.cx, B.cy, B.mx, B.mxr, B.my, B.myr, B.h0, B.he, B.hc, B.hr};
+#pragma unroll
+        for (int e = 0; e < bCorner; ++e) to[e * stride] = v[e];
+#pragma unroll
+        for (int e = 0; e < 9; ++e) to[(bCorner + e) * stride] = B.corner[e / 3][e % 3];
+    };
+#pragma unroll
+    for (int e = 0; e < 3; ++e) put(fH + e, M[(mG0 + e) * (size_t)nc + L.j]);
+    put_block(o + fB * 32, 32, block_coef(mj, dt * (wR * nx), dt * (wR * ny), dt * cf));
+    // the diagonal block's face sum is A_n at the summed weighted normal
+    const double sx = face_sum(L.on ? wL * nx : 0.0, lane, L.nf), sy = face_sum(L.on ? wL * ny : 0.0, lane, L.nf);
+    const double sc = face_sum(cf, lane, L.nf);
+    if (L.f) return;
+    BlockCoef X = block_coef(mi, dt * sx, dt * sy, -(dt * sc));
+    // H itself on the flow rows (the level rows' identity is added to the band)
+    const double he = 1.0 + X.he;
+    X.mx += mi.u;
+    X.my += mi.v;
+    X.he = he;
+    X.h0 = he * mi.ke;
+    X.hc = he * mi.T;
+    X.corner[0][0] += mi.rho;
+    X.corner[1][1] += mi.rho;
+    X.corner[2][0] += mi.rho * mi.u;
+    X.corner[2][1] += mi.rho * mi.v;
+    X.corner[2][2] += mi.C;
+    double *c = F.cell + (size_t)blk * kCellFields * kFlowCells + (lane >> 2);
+    const double kap = M[mKap * (size_t)nc + L.i];
+    c[cKap * kFlowCells] = kap;
+    c[cVT * kFlowCells] = kap * F.theta / (mi.T * mi.T) * M[mSb * (size_t)nc + L.i];
+    put_block(c + cB * kFlowCells, kFlowCells, X);
+}
+
+// Jacobian entries, one warp per cell, lanes over the species.
+__global__ void __launch_bounds__(kFlowCells * 32) k_flow_jac(FlowDev F, const double *Q, double *S, double *U,
+                                                              double *V) {
+    __shared__ double sh[kFlowCells][kFaceFields * 4 + kCellFields];
+    __shared__ long long sk[kFlowCells][4];          // neighbour blocks: first S value,
+    __shared__ int sj[kFlowCells][4], spo[kFlowCells][4];      // cell and first pair
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int b = F.b, N = F.N, w = F.w, nc = F.nc;
+    const double dt = F.dt;
+    const double *M = F.mix;
+    const int i = blockIdx.x * kFlowCells + warp;
+    if (i >= nc) return;
+    // this cell's coefficients: fc[field * 4 + face], cc[field]
+    double *fc = sh[warp], *cc = fc + kFaceFields * 4;
+    const double *gf = F.face + (size_t)blockIdx.x * kFaceFields * 32 + warp * 4;
+    for (int e = lane; e < kFaceFields * 4; e += 32) fc[e] = gf[(e >> 2) * 32 + (e & 3)];
+    if (lane < kCellFields) cc[lane] = F.cell[((size_t)blockIdx.x * kCellFields + lane) * kFlowCells + warp];
+    const int k0 = F.bptr[i], nf = F.bptr[i + 1] - k0 - 1;
+    // lane k of the row's at most five blocks
+    const int col = lane <= nf ? F.bidx[k0 + lane] : -1;
+    const int at = __ffs(__ballot_sync(0xffffffffu, col == i)) - 1, kd = k0 + at;
+    if (lane <= nf && lane != at) {
+        const int f = lane - (lane > at ? 1 : 0);
+        sj[warp][f] = col;
+        spo[warp][f] = F.pip[k0 + lane];
+        sk[warp][f] = F.soff[k0 + lane];
+    }
+    __syncwarp();
+    const double *qi = Q + (size_t)i * b;
+    const double g0 = M[mG0 * (size_t)nc + i], g1 = M[mG1 * (size_t)nc + i], g2 = M[mG2 * (size_t)nc + i];
+    const size_t ps = (size_t)F.pip[kd];
+    double *Sd = S + F.soff[kd];
+    // ---- level columns of the flow rows and level components of the pairs, lanes over species
+    for (int c0 = 0; c0 < N; c0 += 32) {
+        const int c = c0 + lane;
+        const bool on = c < N;
+        const double x = on ? qi[c] : 0.0, rc = on ? __ldg(F.r + c) : 0.0, cvc = on ? __ldg(F.cv + c) : 0.0,
+                     e0c = on ? __ldg(F.e0 + c) : 0.0;
+        double ys[4];
+#pragma unroll
+        for (int f = 0; f < 4; ++f) ys[f] = on && f < nf ? __ldg(Q + (size_t)sj[warp][f] * b + c) : 0.0;
+        const double ga = fma(g2, rc, fma(g1, cvc, g0));
+        if (on) {
+            const double *B = cc + cB;
+            double *Sf = Sd + F.d_ptr[N] + c;
+            Sf[0] = fma(B[bMxr], rc, B[bMx]);
+            Sf[b] = fma(B[bMyr], rc, B[bMy]);
+            Sf[2 * b] = fma(B[bHr], rc, fma(B[bHc], cvc, fma(B[bHe], e0c, B[bH0])));
+            U[ps * b + c] = -dt * __ldg(F.ws + c);
+            V[ps * b + c] = cc[cKap] * __ldg(F.beta + c);
+        }
+#pragma unroll
+        for (int f = 0; f < 4; ++f) {
+            if (f >= nf) break;
+            const int j = sj[warp][f];
+            const bool horizontal = F.Lx > 1 && (j == i + 1 || j == i - 1);
+            const double *o = fc + f, *B = o + fB * 4;              // field e at o[4 e]
+            const double y = ys[f];
+            const double gj = fma(o[4 * (fH + 2)], rc, fma(o[4 * (fH + 1)], cvc, o[4 * fH]));
+            const size_t pd = ps + 1 + 2 * f, po = (size_t)spo[warp][f];
+            double *Sk = S + sk[warp][f];
+            if (on) {
+                const double u1 = fma(o[4 * fUi], x, -(o[4 * fUj] * y)), u2 = dt * (y - x);
+                U[pd * b + c] = u1;
+                U[(pd + 1) * b + c] = u2;
+                U[po * b + c] = u1;
+                U[(po + 1) * b + c] = u2;
+                V[pd * b + c] = o[4 * fG] * ga;
+                V[(pd + 1) * b + c] = o[4 * fG + 4] * ga;
+                V[po * b + c] = o[4 * fG + 8] * gj;
+                V[(po + 1) * b + c] = o[4 * fG + 12] * gj;
+                // the normal is along one axis: one momentum row is constant over the species
+                const int m = horizontal ? bMx : bMy;
+                const double t = fma(B[4 * (m + 1)], rc, B[4 * m]), u = B[4 * (bMx + bMy - m)];
+                double *Sf = Sk + 4 * N + c;
+                Sf[0] = horizontal ? t : u;
+                Sf[b] = horizontal ? u : t;
+                Sf[2 * b] = fma(B[4 * bHr], rc, fma(B[4 * bHc], cvc, fma(B[4 * bHe], e0c, B[4 * bH0])));
+            }
+            // neighbour block's level rows [diag, cx q, cy q, 0]: 32 rows are 128 consecutive
+            // entries; one of cx, cy is zero
+            const double z = B[4 * (horizontal ? bCx : bCy)] * y, d = B[4 * bDiag];
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const double zr = __shfl_sync(0xffffffffu, z, r * 8 + (lane >> 2));
+                const int col = lane & 3;
+                if (c0 + r * 8 + (lane >> 2) < N)
+                    Sk[4 * c0 + r * 32 + lane] = col == 0 ? d : col == (horizontal ? 1 : 2) ? zr : 0.0;
             }
         }
     }
-#pragma unroll
-    for (int t = 0; t < kMaxPerLane; ++t) {
-        const int c = lane + 32 * t;
-        if (c >= b) break;
-        double src = 0.0;
-        if (c < N) {
-            for (int l = max(0, c - F.w); l < min(N, c + F.w + 1); ++l)
-                src -= F.K[(size_t)c * (2 * F.w + 1) + (l - c + F.w)] * qi[l];
-            src += F.ws[c] * omega;
+    // ---- flow components: computed by k_flow_face_jac, only written here
+    for (int f = 0; f < nf; ++f) {
+        const double *o = fc + f;
+        const size_t pd = ps + 1 + 2 * f, po = (size_t)spo[warp][f];
+        if (lane < 24) {
+            const int row = lane / 3, e = lane - 3 * row;         // U pd, pd+1, po, po+1, then V of the same
+            const size_t at = ((row & 2 ? po : pd) + (row & 1)) * b + N + e;
+            if (row < 4) U[at] = o[4 * (fU + 3 * (row & 1) + e)];
+            else V[at] = o[4 * (fV + 3 * (row & 3) + e)];
         }
-        R[(size_t)i * b + c] = (cons_c(F, qi, mi, c) - cons_c(F, qn, mn, c)) + F.dt * (fsum[t] - src);
+        if (lane < 9) S[sk[warp][f] + 4 * N + (size_t)(lane / 3) * b + N + lane % 3] = o[4 * (fB + bCorner + lane)];
+    }
+    if (lane < 9) Sd[F.d_ptr[N] + (lane / 3) * b + N + lane % 3] = cc[cB + bCorner + lane];
+    if (lane < 3) {
+        U[ps * b + N + lane] = 0.0;
+        V[ps * b + N + lane] = lane == 2 ? cc[cVT] : 0.0;
+    }
+    // ---- the diagonal block's level rows: band K (plus H = 1 and the face terms on the
+    // diagonal) and the flow columns, lanes over the pattern's consecutive entries
+    const int nl = F.d_ptr[N];
+#pragma unroll 4
+    for (int e = lane; e < nl; e += 32) {
+        const short2 pq = F.d_pq[e];
+        const int p = pq.x, c = pq.y;
+        double base = 0.0, coef = 0.0, x = 1.0;
+        if (c < N) {
+            base = __ldg(F.dtK + (size_t)p * (2 * w + 1) + (c - p + w));
+            coef = c == p ? cc[cB + bDiag] : 0.0;
+        } else {
+            coef = c == N ? cc[cB + bCx] : c == N + 1 ? cc[cB + bCy] : 0.0;
+            x = qi[p];
+        }
+        Sd[e] = fma(coef, x, base);
+    }
+}
+
+// Residual scalars, as k_flow_face_jac; the flow components are complete here.  With
+// the flux (s_R f_i - s_L f_j + s_L s_R (u_j - u_i)) / (s_R - s_L) the species flux of a
+// face is ca q_i - cb q_j + cd (q_j - q_i).
+__global__ void __launch_bounds__(64) k_flow_face_res(FlowDev F, double *R) {
+    const int lane = threadIdx.x & 31, blk = blockIdx.x * 2 + (threadIdx.x >> 5), nc = F.nc;
+    if (blk * kFlowCells >= nc) return;
+    const double *M = F.mix, *Mn = F.mix + (size_t)kMixFields * nc;
+    const FaceLane L = face_lane(F, blk, lane);
+    const Mix mi = mix_of(M, nc, L.i), mj = mix_of(M, nc, L.j);
+    double nx, ny;
+    normal_of(F.Lx, L.i, L.j, nx, ny);
+    const Face f = face_of(mi, mj, nx, ny);
+    const double uni = nx * mi.u + ny * mi.v, unj = nx * mj.u + ny * mj.v;
+    const double ca = f.sR * f.inv_den, cb = f.sL * f.inv_den, cd = f.sL * f.sR * f.inv_den;
+    const double fi[3] = {mi.rho * mi.u * uni + mi.p * nx, mi.rho * mi.v * uni + mi.p * ny, (mi.e + mi.p) * uni};
+    const double fj[3] = {mj.rho * mj.u * unj + mj.p * nx, mj.rho * mj.v * unj + mj.p * ny, (mj.e + mj.p) * unj};
+    const double ci[3] = {mi.rho * mi.u, mi.rho * mi.v, mi.e}, cj[3] = {mj.rho * mj.u, mj.rho * mj.v, mj.e};
+    double *o = F.face + (size_t)blk * kFaceFields * 32 + lane;
+    o[rB * 32] = cb * unj;
+    o[rD * 32] = cd;
+    const double sum = face_sum(L.on ? ca * uni : 0.0, lane, L.nf);
+    double fl[3];
+#pragma unroll
+    for (int e = 0; e < 3; ++e)
+        fl[e] = face_sum(L.on ? (ca * fi[e] - cb * fj[e]) + cd * (cj[e] - ci[e]) : 0.0, lane, L.nf);
+    if (L.f || blk * kFlowCells + (lane >> 2) >= nc) return;
+    double *c = F.cell + (size_t)blk * kCellFields * kFlowCells + (lane >> 2);
+    c[rA * kFlowCells] = sum;
+    c[rOm * kFlowCells] = M[mKap * (size_t)nc + L.i] * M[mSb * (size_t)nc + L.i];
+    const Mix mn = mix_of(Mn, nc, L.i);
+    const double cn[3] = {mn.rho * mn.u, mn.rho * mn.v, mn.e};
+#pragma unroll
+    for (int e = 0; e < 3; ++e) R[(size_t)L.i * F.b + F.N + e] = (ci[e] - cn[e]) + F.dt * fl[e];
+}
+
+// Residual of the species, one warp per cell, lanes over the species.
+__global__ void __launch_bounds__(kFlowCells * 32) k_flow_res(FlowDev F, const double *Q, const double *Qn,
+                                                              double *R) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int b = F.b, N = F.N, w = F.w, bw = 2 * w + 1;
+    const int i = blockIdx.x * kFlowCells + warp;
+    if (i >= F.nc) return;
+    const int k0 = F.bptr[i], nf = F.bptr[i + 1] - k0 - 1;
+    int j[4];                                   // neighbours in block order
+#pragma unroll
+    for (int f = 0, k = k0; f < 4; ++f, ++k) {
+        if (f < nf && F.bidx[k] == i) ++k;
+        j[f] = f < nf ? F.bidx[k] : i;
+    }
+    const double *gf = F.face + (size_t)blockIdx.x * kFaceFields * 32 + warp * 4;
+    const double *gc = F.cell + (size_t)blockIdx.x * kCellFields * kFlowCells + warp;
+    double fb[4], fd[4];
+#pragma unroll
+    for (int f = 0; f < 4; ++f) {
+        fb[f] = gf[rB * 32 + f];
+        fd[f] = gf[rD * 32 + f];
+    }
+    const double ca = gc[rA * kFlowCells], omega = gc[rOm * kFlowCells];
+    const double *qi = Q + (size_t)i * b, *qn = Qn + (size_t)i * b;
+    for (int c = lane; c < N; c += 32) {
+        const double x = qi[c], xn = qn[c];
+        double y[4];
+#pragma unroll
+        for (int f = 0; f < 4; ++f) y[f] = __ldg(Q + (size_t)j[f] * b + c);
+        double acc = ca * x;
+#pragma unroll
+        for (int f = 0; f < 4; ++f) {
+            if (f >= nf) break;
+            acc = fma(-fb[f], y[f], acc);
+            acc = fma(fd[f], y[f] - x, acc);
+        }
+        double src = 0.0;
+        for (int l = max(0, c - w); l < min(N, c + w + 1); ++l)
+            src = fma(-__ldg(F.K + (size_t)c * bw + (l - c + w)), qi[l], src);
+        src = fma(__ldg(F.ws + c), omega, src);
+        R[(size_t)i * b + c] = (x - xn) + F.dt * (acc - src);
     }
 }
 
@@ -398,11 +628,39 @@ sts_status flow_alloc(sts_flow_s *f, double **p, size_t n) {
     cudaError_t e = cudaMalloc(&q, (n ? n : 1) * sizeof(double));
     if (e != cudaSuccess) {
         cudaGetLastError();
-        return set_error(STS_ERR_ALLOC, "sts_flow_newton: cudaMalloc of %zu doubles failed: %s", n,
+        return set_error(STS_ERR_ALLOC, "flow generator: cudaMalloc of %zu doubles failed: %s", n,
                          cudaGetErrorString(e));
     }
     f->bufs.push_back(q);
     *p = static_cast<double *>(q);
+    return STS_OK;
+}
+
+sts_status flow_mix(sts_flow_s *f, const double *Q, const double *Qn) {
+    const int b = f->dev.b;
+    const size_t smem = (32 * (size_t)(b | 1) + 4 * (size_t)f->dev.N + 4 * 5 * 32) * sizeof(double);
+    if (smem > 48 * 1024)
+        STS_CK(cudaFuncSetAttribute(k_flow_mix, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    k_flow_mix<<<dim3((f->dev.nc + kMixCells - 1) / kMixCells, Qn ? 2 : 1), 128, smem, f->stream>>>(f->dev, Q, Qn);
+    STS_LAUNCHED();
+    return STS_OK;
+}
+
+sts_status flow_res(sts_flow_s *f, const double *Q, const double *Qn, double *R) {
+    STS_TRY(flow_mix(f, Q, Qn));
+    k_flow_face_res<<<(f->dev.nc + 2 * kFlowCells - 1) / (2 * kFlowCells), 64, 0, f->stream>>>(f->dev, R);
+    STS_LAUNCHED();
+    k_flow_res<<<(f->dev.nc + kFlowCells - 1) / kFlowCells, kFlowCells * 32, 0, f->stream>>>(f->dev, Q, Qn, R);
+    STS_LAUNCHED();
+    return STS_OK;
+}
+
+sts_status flow_jac(sts_flow_s *f, const double *Q, double *S, double *U, double *V) {
+    STS_TRY(flow_mix(f, Q, nullptr));
+    k_flow_face_jac<<<(f->dev.nc + 2 * kFlowCells - 1) / (2 * kFlowCells), 64, 0, f->stream>>>(f->dev);
+    STS_LAUNCHED();
+    k_flow_jac<<<(f->dev.nc + kFlowCells - 1) / kFlowCells, kFlowCells * 32, 0, f->stream>>>(f->dev, Q, S, U, V);
+    STS_LAUNCHED();
     return STS_OK;
 }
 
@@ -450,10 +708,9 @@ sts_status flow_newton(sts_flow_s *f, sts_jac_t jac, double *Q, const double *Qn
         STS_TRY(flow_alloc(f, &f->partial, kNormBlocks));
         STS_CK(cudaMallocHost(&f->h_partial, kNormBlocks * sizeof(double)));
     }
-    const unsigned grid = (unsigned)((f->dev.nc + kFlowWarps - 1) / kFlowWarps), eg = flow_grid(n);
+    const unsigned eg = flow_grid(n);
     sts_newton_info inf{0, 0, 0, 0, 0.0, 0.0};
-    k_flow_res<<<grid, kFlowWarps * 32, 0, f->stream>>>(f->dev, Q, Qn, f->R);
-    STS_LAUNCHED();
+    STS_TRY(flow_res(f, Q, Qn, f->R));
     double r = 0.0;
     STS_TRY(flow_norm(f, f->R, n, &r));
     inf.res0 = inf.res = r;
@@ -475,8 +732,7 @@ sts_status flow_newton(sts_flow_s *f, sts_jac_t jac, double *Q, const double *Qn
         if (inf.iterations >= max_newton) break;
         NvtxRange nvtx_it("newton iteration");
         // Jacobian at Q into the handle, block-Jacobi, then J dQ = -R
-        k_flow_jac<<<grid, kFlowWarps * 32, 0, f->stream>>>(f->dev, Q, f->S, f->U, f->V);
-        STS_LAUNCHED();
+        STS_TRY(flow_jac(f, Q, f->S, f->U, f->V));
         k_flow_axpy<<<eg, 256, 0, f->stream>>>(f->rhs, nullptr, 0.0, f->R, n, 1);
         STS_LAUNCHED();
         STS_CK(cudaMemsetAsync(f->dQ, 0, n * sizeof(double), f->stream));
@@ -502,8 +758,7 @@ sts_status flow_newton(sts_flow_s *f, sts_jac_t jac, double *Q, const double *Qn
         for (int hv = 0; hv <= max_halvings; ++hv) {
             k_flow_axpy<<<eg, 256, 0, f->stream>>>(f->Qt, Q, alpha, f->dQ, n, 0);
             STS_LAUNCHED();
-            k_flow_res<<<grid, kFlowWarps * 32, 0, f->stream>>>(f->dev, f->Qt, Qn, f->Rt);
-            STS_LAUNCHED();
+            STS_TRY(flow_res(f, f->Qt, Qn, f->Rt));
             STS_TRY(flow_norm(f, f->Rt, n, &rt));
             if (std::isfinite(rt) && rt < r) {
                 accepted = true;
@@ -629,8 +884,19 @@ sts_status flow_create(const sts_flow_desc *d, sts_flow_t *out) {
     D.A = d->A;
     D.theta = d->theta;
     D.dt = d->dt;
+    std::vector<double> dtK((size_t)N * (2 * w + 1));
+    for (size_t e = 0; e < dtK.size(); ++e) dtK[e] = d->dt * d->K[e] + ((int)(e % (2 * w + 1)) == w ? 1.0 : 0.0);
+    std::vector<short2> pq;
+    for (int p = 0; p < N; ++p)
+        for (int e = f->dptr[p]; e < f->dptr[p + 1]; ++e) pq.push_back(make_short2((short)p, (short)f->didx[e]));
     sts_status st = STS_OK;
     do {
+        if ((st = flow_alloc(f, &D.mix, 2 * (size_t)kMixFields * nc)) != STS_OK) break;
+        const size_t blocks = (nc + kFlowCells - 1) / kFlowCells;
+        if ((st = flow_alloc(f, &D.face, blocks * kFaceFields * 32)) != STS_OK) break;
+        if ((st = flow_alloc(f, &D.cell, blocks * kCellFields * kFlowCells)) != STS_OK) break;
+        if ((st = flow_upload(f, &D.dtK, dtK.data(), dtK.size())) != STS_OK) break;
+        if ((st = flow_upload(f, &D.d_pq, pq.data(), pq.size())) != STS_OK) break;
         if ((st = flow_upload(f, &D.r, d->r, N)) != STS_OK) break;
         if ((st = flow_upload(f, &D.cv, d->cv, N)) != STS_OK) break;
         if ((st = flow_upload(f, &D.e0, d->e0, N)) != STS_OK) break;
@@ -702,19 +968,13 @@ sts_status sts_flow_get_layout(sts_flow_t f, int *block_indptr, int *block_indic
 sts_status sts_flow_residual(sts_flow_t f, const double *Q, const double *Qn, double *R) {
     NvtxRange nvtx_range("sts_flow_residual");
     if (!f || !Q || !Qn || !R) return set_error(STS_ERR_INVALID_ARG, "sts_flow_residual: NULL argument");
-    const unsigned grid = (unsigned)((f->dev.nc + kFlowWarps - 1) / kFlowWarps);
-    k_flow_res<<<grid, kFlowWarps * 32, 0, f->stream>>>(f->dev, Q, Qn, R);
-    STS_LAUNCHED();
-    return STS_OK;
+    return flow_res(f, Q, Qn, R);
 }
 
 sts_status sts_flow_jacobian(sts_flow_t f, const double *Q, double *S, double *U, double *V) {
     NvtxRange nvtx_range("sts_flow_jacobian");
     if (!f || !Q || !S || !U || !V) return set_error(STS_ERR_INVALID_ARG, "sts_flow_jacobian: NULL argument");
-    const unsigned grid = (unsigned)((f->dev.nc + kFlowWarps - 1) / kFlowWarps);
-    k_flow_jac<<<grid, kFlowWarps * 32, 0, f->stream>>>(f->dev, Q, S, U, V);
-    STS_LAUNCHED();
-    return STS_OK;
+    return flow_jac(f, Q, S, U, V);
 }
 
 sts_status sts_flow_newton(sts_flow_t f, sts_jac_t jac, double *Q, const double *Qn, const sts_newton_opts *opts,

@@ -1,0 +1,39 @@
+"""The HLL-flux generator where its kernels' tiles end: cells about the 8 of a face
+warp and the 32 of a mixture block, species about the 32 lanes, the largest block
+(b = 256), and a uniform state, where every wave-speed candidate ties between the two
+sides of a face.  Same oracle, scales and tolerance as tests/test_gpu_flow.py.
+"""
+import numpy as np
+import pytest
+
+from oracle import flux
+from paper_2403_09198_gb300 import inputs
+from paper_2403_09198_gb300.binding import StsFlow
+from tests._gpu import dev, host
+from tests.test_gpu_flow import TOL_RES, _res_err, _scaled_err
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    import __graft_entry__
+    __graft_entry__.build()
+
+
+@pytest.mark.parametrize("Lx,Ly,N,w", [(3, 3, 31, 2), (11, 3, 32, 4), (8, 5, 33, 2), (2, 16, 64, 0), (5, 2, 65, 3),
+                                       (2, 2, 253, 2), (1, 33, 7, 1)])
+@pytest.mark.parametrize("uniform", [False, True])
+def test_edges(Lx, Ly, N, w, uniform):
+    c = inputs.make_flow_case(Lx, Ly, N=N, w=w, seed=21, dt=0.3)
+    if uniform:
+        c.Q[:] = c.Q[0]
+    m = flux.model_of(c)
+    f = StsFlow(c)
+    ref = flux.jacobian_blocks(m, Lx, Ly, c.Q)
+    for _ in range(2):                       # the second call finds the first one's scalars in its workspace
+        R = host(f.residual(dev(c.Q), dev(c.Qn)))
+        for key, got in zip("SUV", f.jacobian(dev(c.Q))):
+            assert _scaled_err(host(got), ref[key], ref["scales"][key]) <= TOL_RES, key
+        assert _res_err(R, m, c) <= TOL_RES
+    f.close()
