@@ -2,8 +2,8 @@
 //
 // Section 6 (Eq. right_precond_system): solve (A M) y = b, x = M y.  Each
 // cycle starts from the true FP64 residual r = b - A x, builds the Krylov basis
-// by classical Gram-Schmidt with a second pass (CGS2: two fused multi-dot +
-// update sweeps per step, same result as modified Gram-Schmidt in exact
+// by classical Gram-Schmidt with a second pass (CGS2: dots, update and dots
+// in one sweep, update and norm; same result as modified Gram-Schmidt in exact
 // arithmetic), reduces the Hessenberg matrix with Givens rotations on the host
 // in FP64 and updates x += Z y with Z = [M v_0, ..., M v_{k-1}] (for a fixed M
 // this equals x += M (V y)).  Convergence is declared on the recomputed true
@@ -18,226 +18,264 @@
 // and the block that finishes last adds them in a fixed order.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
+#include <utility>
 #include <vector>
 
+#include "ring.cuh"
 #include "sts_internal.h"
 
 namespace sts {
 namespace {
 
-constexpr int kRedBlocks = 304;     // 2 x 152 SMs
 constexpr int kRedThreads = 256;
-constexpr int kDotChunk = 16;       // vectors per multi-dot sweep
+constexpr int kRedMax = 304;        // blocks of a reduction at most: two per SM
+constexpr int kOrthChunk = 31;      // vectors per sweep: their dots and w . w fill a warp's 32 lanes
 
-// Per-block sums of the first NV of the values v at once: every warp reduces
-// them with shuffles, then thread i < NV adds the warps' results in warp order
-// and writes row[i].  One barrier for all NV values.  sh: 8 * NV doubles.
-template <int NV, int NA>
-__device__ __forceinline__ void block_partials(double (&v)[NA], double *row, double *sh) {
-    static_assert(NV <= NA, "values to reduce");
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-#pragma unroll
-    for (int i = 0; i < NV; ++i) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v[i] += __shfl_down_sync(0xffffffffu, v[i], o);
-        if (lane == 0) sh[w * NV + i] = v[i];
-    }
-    __syncthreads();
-    if (threadIdx.x < NV) {
-        double s = 0.0;
-        for (int k = 0; k < (int)(blockDim.x >> 5); ++k) s += sh[k * NV + threadIdx.x];
-        row[threadIdx.x] = s;
-    }
+// Blocks of the sweeps over n elements and cnt vectors, one element per thread at
+// least.  The sums depend on this number: it is a function of n and cnt alone, so that
+// every caller gets the same bits.  Above kTwoBlocks vectors the accumulators leave
+// room for one block per SM.
+constexpr int kTwoBlocks = 24;
+inline int orth_blocks(long long n, int cnt) {
+    const long long most = cnt <= kTwoBlocks ? kRedMax : kRedMax / 2;
+    return (int)std::max(1LL, std::min(most, (n + kRedThreads - 1) / kRedThreads));
 }
 
-// The block that finishes last adds the per-block partial sums of `cnt`
-// outputs (partial[b * ld + o], o = o0 .. o0 + cnt - 1) into out[o]: warp w
-// takes outputs w, w + 8, ...; lane l adds blocks l, l + 32, ... and the
-// shuffle tree adds the lanes, so the order of additions never depends on
-// which block is last or on scheduling.  The ticket counts finished blocks
-// and is reset for the next launch.
-__device__ __forceinline__ void last_block_reduce(double *partial, int ld, int o0, int cnt, double *out,
-                                                  unsigned int *ticket) {
+// Whether a sweep is launched early (programmatic dependent launch): on small grids,
+// where its blocks wait beside the previous kernel's.  On full ones they take the
+// place of blocks that have work (measured on 125 x 121 cells, N = 60: GMRES 1.55 -> 1.59 ms).
+inline bool early_start(int blocks) { return blocks < kRedMax / 2; }
+
+// Sum each of the NV values of v over the warp: lane l returns the sum of value
+// l >> (5 - log2 of NV rounded up to a power of two).  Every exchange halves the values
+// that a lane still carries, so NV values take NV - 1 + (5 - log2 NV) FP64 additions
+// instead of 5 NV (an FP64 addition holds the pipe for 64 cycles whatever the lanes).
+template <int NV>
+__device__ __forceinline__ double warp_sums(double (&v)[NV], int lane) {
+    static_assert(NV >= 1 && NV <= 32 && (NV & (NV - 1)) == 0, "a power of two");
+    int mask = 16;
+#pragma unroll
+    for (int half = NV / 2; half >= 1; half /= 2, mask /= 2) {
+        const bool up = lane & mask;
+#pragma unroll
+        for (int i = 0; i < half; ++i) {
+            const double send = up ? v[i] : v[i + half], keep = up ? v[i + half] : v[i];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, mask);
+        }
+    }
+    double s = v[0];
+    for (; mask >= 1; mask /= 2) s += __shfl_xor_sync(0xffffffffu, s, mask);
+    return s;
+}
+
+// Totals of NV values over the whole grid, into out[0..NV), by the block that finishes
+// last; true in that block (after its stores).  Every block's sums go to
+// partial[block][0..NV); the last block adds them in a fixed order (warp w takes
+// blocks w, w + 8, ..., lane = value, then the warps in order), so the result never
+// depends on which block is last.  The ticket counts finished blocks and is reset.
+template <int NV>
+__device__ __forceinline__ bool grid_totals(double (&v)[NV], int used, double *partial, double *out,
+                                            unsigned int *ticket) {
+    constexpr int NW = kRedThreads / 32, SH = NV == 32 ? 0 : NV == 16 ? 1 : NV == 8 ? 2 : NV == 4 ? 3 : NV == 2 ? 4 : 5;
+    __shared__ double sh[NW][NV];
     __shared__ bool last;
-    __threadfence();
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const double s = warp_sums<NV>(v, lane);
+    if ((lane & ((1 << SH) - 1)) == 0) sh[w][lane >> SH] = s;
+    __syncthreads();
+    if (threadIdx.x < NV) {
+        double t = sh[0][threadIdx.x];
+#pragma unroll
+        for (int k = 1; k < NW; ++k) t += sh[k][threadIdx.x];
+        partial[(size_t)blockIdx.x * NV + threadIdx.x] = t;
+        __threadfence();
+    }
     __syncthreads();
     if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == gridDim.x - 1;
     __syncthreads();
-    if (!last) return;
+    if (!last) return false;
     __threadfence();
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    for (int o = o0 + w; o < o0 + cnt; o += nw) {
-        double s = 0.0;
-        for (int b = lane; b < (int)gridDim.x; b += 32) s += __ldcg(partial + (size_t)b * ld + o);
+    // 32 / NV blocks side by side in a warp, so that every lane adds
+    const int per = 1 << SH, o = lane & (NV - 1), b0 = w * per + lane / NV;
+    double t = 0.0;
+    for (int b = b0; b < (int)gridDim.x; b += NW * per) t += __ldcg(partial + (size_t)b * NV + o);
 #pragma unroll
-        for (int k = 16; k > 0; k >>= 1) s += __shfl_down_sync(0xffffffffu, s, k);
-        if (lane == 0) out[o] = s;
-    }
+    for (int m = 16; m >= NV; m /= 2) t += __shfl_xor_sync(0xffffffffu, t, m);
+    if (lane < NV) sh[w][lane] = t;
     __syncthreads();
+    if (threadIdx.x < used) {
+        t = sh[0][threadIdx.x];
+#pragma unroll
+        for (int k = 1; k < NW; ++k) t += sh[k][threadIdx.x];
+        out[threadIdx.x] = t;
+    }
     if (threadIdx.x == 0) *ticket = 0u;
+    __syncthreads();
+    return true;
 }
 
-// partial[blk * ld + i0 + i] = sum over this block's elements of V_{i0+i} . w,
-// for i < CNT (CNT <= kDotChunk).  With SELF the next slot holds w . w.  The
-// count is a template parameter: a predicated-off FP64 FMA still occupies the
-// FP64 pipe, so the loop must issue exactly CNT (+ SELF) FMAs per element.
-template <int CNT, bool SELF>
-__global__ void __launch_bounds__(kRedThreads) k_mdot(const double *V, long long n, int i0,
-                                                      const double *w, double *partial, int ld, double *out,
-                                                      unsigned int *ticket) {
-    // elements per thread and iteration: all their loads are issued before the
-    // FMAs, so a thread keeps several memory requests in flight
-    constexpr int U = CNT + 1 <= 3 ? 4 : CNT + 1 <= 7 ? 2 : 1;
-    constexpr int NO = CNT + (SELF ? 1 : 0);          // outputs
-    __shared__ double sh[(kRedThreads / 32) * (CNT + 1)];
-    double acc[CNT + 1];
+// State of the device-side rotations (see k_givens_step); H = NULL: none.
+struct Givens {
+    int j, m;
+    const double *h1, *h2;
+    double *H, *cs, *sn, *g, *hist, *par;
+    int *state;
+    cudaGraphConditionalHandle next;
+    int has_next;
+};
+
+// Step j's rotations, by one block: h1, h2 the two passes' coefficients of column j, w2
+// and hn2 the squared norms of w before and after; par: stop threshold, history
+// scale, 1 / h(j+1,j) (output), steps allowed; state: steps taken, stop reason (0 none,
+// 1 criterion met, 2 NaN or Inf).  An FP64 operation takes a whole warp 64 cycles or
+// more, so what can run beside the recurrence does, in other lanes (the products with
+// the column's entries) and other warps (the square root of w2, 1 / hn), and a step of
+// the recurrence is one FMA.  As one thread's loop over global memory it took 5.6 us
+// (j = 0) to 14 us (j = 29).
+constexpr int kGivensMax = 64;
+__device__ __noinline__ void givens_step(const Givens &G, double w2, double hn2) {
+    // t[i]: column entry i after rotations 0 .. i - 1; u[i], v[i]: c_i, s_i times entry i + 1
+    __shared__ double c[kGivensMax], sn[kGivensMax], t[kGivensMax], u[kGivensMax], v[kGivensMax], w0;
+    const int j = G.j, m = G.m, x = threadIdx.x;
+    int bad = 0;
+    if (x <= j) {
+        const double h = G.h1[x] + G.h2[x];
+        bad = !isfinite(h);
+        if (x == 0) t[0] = h;
+        else {
+            c[x - 1] = G.cs[x - 1];
+            sn[x - 1] = G.sn[x - 1];
+            u[x - 1] = c[x - 1] * h;
+            v[x - 1] = sn[x - 1] * h;
+        }
+    }
+    double r = 0.0;
+    if (x == 64) {
+        w0 = r = sqrt(w2);
+    } else if (x == 96) {
+        r = sqrt(hn2);
+        G.par[2] = 1.0 / r;
+    }
+    bad = __syncthreads_or(bad || !isfinite(r));
+    if (x == 0) {
+        int stop = 2;
+        if (!bad) {
+            const double hn = sqrt(hn2);
+            double a = t[0];
+            for (int i = 0; i < j; ++i) {
+                a = fma(-sn[i], a, u[i]);
+                t[i + 1] = a;
+            }
+            const double den = hypot(a, hn), cj = a / den, sj = hn / den, gj = G.g[j], gn = -sj * gj;
+            G.cs[j] = cj;
+            G.sn[j] = sj;
+            G.g[j + 1] = gn;
+            G.g[j] = cj * gj;
+            G.hist[j] = fabs(gn) * G.par[1];
+            G.H[(size_t)j * m + j] = den;
+            const bool happy = hn <= 1e-14 * w0;
+            stop = happy || fabs(gn) <= G.par[0] || (double)(j + 1) >= G.par[3] ? 1 : 0;
+        }
+        G.state[0] = j + 1;
+        G.state[1] = stop;
+        if (G.has_next) cudaGraphSetConditional(G.next, stop ? 0u : 1u);
+    }
+    __syncthreads();
+    if (x < j) G.H[(size_t)x * m + j] = fma(c[x], t[x], v[x]);
+    if (x == j + 1) G.H[(size_t)x * m + j] = 0.0;
+}
+
+// One sweep over w and CNT basis vectors V (contiguous, n apart):
+//   kDots        out[i] = V_i . w, out[CNT] = w . w
+//   kUpdateDots  w -= sum_i h_i V_i, then out[i] = V_i . w with the same loaded V
+//   kUpdateNorm  w -= sum_i h_i V_i, out[0] = w . w, and the rotations that need it
+// The count is a template parameter: a predicated-off FP64 FMA still takes its pipe
+// slot, so the loop issues exactly the FMAs it needs.  U elements per thread and
+// iteration keep several loads in flight where CNT is small.  Bound by the FP64 pipe
+// from about eight vectors on (one FMA per loaded value, two in kUpdateDots), by
+// memory below.  Measured on 128 x 128 cells, N = 60 (1.03 M elements): with dots,
+// update, dots and update as four sweeps and 5 additions per value and warp in the
+// reductions, the 163 steps of a Newton step (16 vectors on average) took 31.3 ms, now
+// 23.6 ms, the rotations included; 18.2 ms are FP64 pipe time.
+enum { kDots, kUpdateDots, kUpdateNorm };
+
+constexpr int pow2_at_least(int n) { return n <= 1 ? 1 : n <= 2 ? 2 : n <= 4 ? 4 : n <= 8 ? 8 : n <= 16 ? 16 : 32; }
+
+template <int CNT, int MODE>
+__global__ void __launch_bounds__(kRedThreads, CNT <= kTwoBlocks ? 2 : 1)
+    k_orth(double *w, const double *V, long long n, const double *hcoef, double *partial, double *out,
+           int n_out, unsigned int *ticket, Givens G) {
+    constexpr int U = CNT + 1 <= 3 ? 4 : CNT + 1 <= (MODE == kUpdateNorm ? kTwoBlocks : 7) ? 2 : 1, C1 = CNT > 0 ? CNT : 1;
+    // the same tree in both modes that return dots, so that they return the same bits
+    constexpr int NO = MODE == kUpdateNorm ? 1 : CNT + 1, NV = pow2_at_least(NO);
+    __shared__ double h[C1];
+    pdl_wait();
+    pdl_trigger();
+    if (MODE != kDots) {
+        if (threadIdx.x < CNT) h[threadIdx.x] = __ldcg(hcoef + threadIdx.x);
+        __syncthreads();
+    }
+    double acc[NV];
 #pragma unroll
-    for (int i = 0; i <= CNT; ++i) acc[i] = 0.0;
+    for (int i = 0; i < NV; ++i) acc[i] = 0.0;
     const long long stride = (long long)gridDim.x * blockDim.x;
+    auto step = [&](double we, const double (&v)[C1], long long e) {
+        if (MODE != kDots) {
+#pragma unroll
+            for (int i = 0; i < CNT; ++i) we = fma(-h[i], v[i], we);
+            w[e] = we;
+        }
+        if (MODE != kUpdateNorm) {
+#pragma unroll
+            for (int i = 0; i < CNT; ++i) acc[i] = fma(v[i], we, acc[i]);
+        }
+        if (MODE != kUpdateDots) acc[NO - 1] = fma(we, we, acc[NO - 1]);
+    };
     long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     for (; e + (U - 1) * stride < n; e += U * stride) {
-        double we[U], vv[U][CNT > 0 ? CNT : 1];
+        double we[U], v[U][C1];
 #pragma unroll
         for (int u = 0; u < U; ++u) we[u] = w[e + u * stride];
 #pragma unroll
         for (int u = 0; u < U; ++u)
 #pragma unroll
-            for (int i = 0; i < CNT; ++i) vv[u][i] = V[(size_t)(i0 + i) * n + e + u * stride];
+            for (int i = 0; i < CNT; ++i) v[u][i] = __ldg(V + (size_t)i * n + e + u * stride);
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-#pragma unroll
-            for (int i = 0; i < CNT; ++i) acc[i] = fma(vv[u][i], we[u], acc[i]);
-            if (SELF) acc[CNT] = fma(we[u], we[u], acc[CNT]);
-        }
+        for (int u = 0; u < U; ++u) step(we[u], v[u], e + u * stride);
     }
     for (; e < n; e += stride) {
-        const double we = w[e];
+        double v[C1];
 #pragma unroll
-        for (int i = 0; i < CNT; ++i) acc[i] = fma(V[(size_t)(i0 + i) * n + e], we, acc[i]);
-        if (SELF) acc[CNT] = fma(we, we, acc[CNT]);
+        for (int i = 0; i < CNT; ++i) v[i] = __ldg(V + (size_t)i * n + e);
+        step(w[e], v, e);
     }
-    block_partials<NO>(acc, partial + (size_t)blockIdx.x * ld + i0, sh);
-    last_block_reduce(partial, ld, i0, NO, out, ticket);
+    const bool last = grid_totals<NV>(acc, n_out, partial, out, ticket);
+    if (MODE == kUpdateNorm && last && G.H) givens_step(G, G.h1[G.j + 1], out[0]);
 }
 
-template <int CNT>
-void mdot_launch(const double *V, long long n, int i0, const double *w, double *partial, int ld, bool self,
-                 double *out, unsigned int *ticket, cudaStream_t st) {
-    if (self) k_mdot<CNT, true><<<kRedBlocks, kRedThreads, 0, st>>>(V, n, i0, w, partial, ld, out, ticket);
-    else k_mdot<CNT, false><<<kRedBlocks, kRedThreads, 0, st>>>(V, n, i0, w, partial, ld, out, ticket);
+using OrthKernel = void (*)(double *, const double *, long long, const double *, double *, double *, int,
+                            unsigned int *, Givens);
+template <int MODE, int... I>
+OrthKernel orth_kernel(int cnt, std::integer_sequence<int, I...>) {
+    static const OrthKernel k[] = {k_orth<I, MODE>...};
+    return k[cnt];
 }
 
-// cnt in 0..kDotChunk (cnt = 0 only with self: w . w alone)
-void mdot_dispatch(int cnt, const double *V, long long n, int i0, const double *w, double *partial, int ld,
-                   bool self, double *out, unsigned int *ticket, cudaStream_t st) {
-    static_assert(kDotChunk == 16, "one case per count");
-    switch (cnt) {
-        case 0: mdot_launch<0>(V, n, i0, w, partial, ld, self, out, ticket, st); break;
-        case 1: mdot_launch<1>(V, n, i0, w, partial, ld, self, out, ticket, st); break;
-        case 2: mdot_launch<2>(V, n, i0, w, partial, ld, self, out, ticket, st); break;
-        case 3: mdot_launch<3>(V, n, i0, w, partial, ld, self, out, ticket, st); break;
-        case 4: mdot_launch<4>(V, n, i0, w, partial, ld, self, out, ticket, st); break;
-        case 5: mdot_launch<5>(V, n, i0, w, partial, ld, self, out, ticket, st); break;
-        case 6: mdot_launch<6>(V, n, i0, w, partial, ld, self, out, ticket, st); break;
-        case 7: mdot_launch<7>(V, n, i0, w, partial, ld, self, out, ticket, st); break;
-        case 8: mdot_launch<8>(V, n, i0, w, partial, ld, self, out, ticket, st); break;
-        case 9: mdot_launch<9>(V, n, i0, w, partial, ld, self, out, ticket, st); break;
-        case 10: mdot_launch<10>(V, n, i0, w, partial, ld, self, out, ticket, st); break;
-        case 11: mdot_launch<11>(V, n, i0, w, partial, ld, self, out, ticket, st); break;
-        case 12: mdot_launch<12>(V, n, i0, w, partial, ld, self, out, ticket, st); break;
-        case 13: mdot_launch<13>(V, n, i0, w, partial, ld, self, out, ticket, st); break;
-        case 14: mdot_launch<14>(V, n, i0, w, partial, ld, self, out, ticket, st); break;
-        case 15: mdot_launch<15>(V, n, i0, w, partial, ld, self, out, ticket, st); break;
-        default: mdot_launch<16>(V, n, i0, w, partial, ld, self, out, ticket, st); break;
-    }
-}
-
-// w -= sum_{i<CNT} h_{i0+i} V_{i0+i}; with NORM also out[0] = ||w||^2 after the
-// update (accumulated in the same sweep, reduced by the last block).  CNT is a
-// template parameter for the same reason as in k_mdot.
-template <int CNT, bool NORM>
-__global__ void __launch_bounds__(kRedThreads) k_update(double *w, const double *V, long long n,
-                                                        const double *hcoef, int i0, double *partial,
-                                                        double *out, unsigned int *ticket) {
-    constexpr int U = CNT + 1 <= 3 ? 4 : CNT + 1 <= 7 ? 2 : 1;
-    __shared__ double sh[kRedThreads / 32];
-    double h[CNT > 0 ? CNT : 1];
-#pragma unroll
-    for (int i = 0; i < CNT; ++i) h[i] = __ldg(hcoef + i0 + i);
-    double acc = 0.0;
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    for (; e + (U - 1) * stride < n; e += U * stride) {
-        double v[U], vv[U][CNT > 0 ? CNT : 1];
-#pragma unroll
-        for (int u = 0; u < U; ++u) v[u] = w[e + u * stride];
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-#pragma unroll
-            for (int i = 0; i < CNT; ++i) vv[u][i] = V[(size_t)(i0 + i) * n + e + u * stride];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-#pragma unroll
-            for (int i = 0; i < CNT; ++i) v[u] = fma(-h[i], vv[u][i], v[u]);
-            w[e + u * stride] = v[u];
-            if (NORM) acc = fma(v[u], v[u], acc);
-        }
-    }
-    for (; e < n; e += stride) {
-        double v = w[e];
-#pragma unroll
-        for (int i = 0; i < CNT; ++i) v = fma(-h[i], V[(size_t)(i0 + i) * n + e], v);
-        w[e] = v;
-        if (NORM) acc = fma(v, v, acc);
-    }
-    if (NORM) {
-        double a1[1] = {acc};
-        block_partials<1>(a1, partial + blockIdx.x, sh);
-        last_block_reduce(partial, 1, 0, 1, out, ticket);
-    }
-}
-
-template <int CNT>
-void update_launch(double *w, const double *V, long long n, const double *hcoef, int i0, bool norm,
-                   double *partial, double *out, unsigned int *ticket, cudaStream_t st) {
-    if (norm) k_update<CNT, true><<<kRedBlocks, kRedThreads, 0, st>>>(w, V, n, hcoef, i0, partial, out, ticket);
-    else k_update<CNT, false><<<kRedBlocks, kRedThreads, 0, st>>>(w, V, n, hcoef, i0, partial, out, ticket);
-}
-
-// cnt in 1..kDotChunk
-void update_dispatch(int cnt, double *w, const double *V, long long n, const double *hcoef, int i0, bool norm,
-                     double *partial, double *out, unsigned int *ticket, cudaStream_t st) {
-    switch (cnt) {
-        case 1: update_launch<1>(w, V, n, hcoef, i0, norm, partial, out, ticket, st); break;
-        case 2: update_launch<2>(w, V, n, hcoef, i0, norm, partial, out, ticket, st); break;
-        case 3: update_launch<3>(w, V, n, hcoef, i0, norm, partial, out, ticket, st); break;
-        case 4: update_launch<4>(w, V, n, hcoef, i0, norm, partial, out, ticket, st); break;
-        case 5: update_launch<5>(w, V, n, hcoef, i0, norm, partial, out, ticket, st); break;
-        case 6: update_launch<6>(w, V, n, hcoef, i0, norm, partial, out, ticket, st); break;
-        case 7: update_launch<7>(w, V, n, hcoef, i0, norm, partial, out, ticket, st); break;
-        case 8: update_launch<8>(w, V, n, hcoef, i0, norm, partial, out, ticket, st); break;
-        case 9: update_launch<9>(w, V, n, hcoef, i0, norm, partial, out, ticket, st); break;
-        case 10: update_launch<10>(w, V, n, hcoef, i0, norm, partial, out, ticket, st); break;
-        case 11: update_launch<11>(w, V, n, hcoef, i0, norm, partial, out, ticket, st); break;
-        case 12: update_launch<12>(w, V, n, hcoef, i0, norm, partial, out, ticket, st); break;
-        case 13: update_launch<13>(w, V, n, hcoef, i0, norm, partial, out, ticket, st); break;
-        case 14: update_launch<14>(w, V, n, hcoef, i0, norm, partial, out, ticket, st); break;
-        case 15: update_launch<15>(w, V, n, hcoef, i0, norm, partial, out, ticket, st); break;
-        default: update_launch<16>(w, V, n, hcoef, i0, norm, partial, out, ticket, st); break;
-    }
-}
-
-__global__ void __launch_bounds__(kRedThreads) k_norm2(const double *v, long long n, double *partial, double *out,
-                                                       unsigned int *ticket) {
-    __shared__ double sh[kRedThreads / 32];
-    double acc = 0.0;
-    for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < n;
-         e += (long long)gridDim.x * blockDim.x)
-        acc = fma(v[e], v[e], acc);
-    double a1[1] = {acc};
-    block_partials<1>(a1, partial + blockIdx.x, sh);
-    last_block_reduce(partial, 1, 0, 1, out, ticket);
+sts_status orth_launch(int mode, int cnt, double *w, const double *V, long long n, const double *hcoef,
+                       double *partial, double *out, int n_out, unsigned int *ticket, cudaStream_t st,
+                       const Givens &G = {}) {
+    using All = std::make_integer_sequence<int, kOrthChunk + 1>;
+    const OrthKernel k = mode == kDots ? orth_kernel<kDots>(cnt, All{})
+                         : mode == kUpdateDots ? orth_kernel<kUpdateDots>(cnt, All{}) : orth_kernel<kUpdateNorm>(cnt, All{});
+    const int blocks = orth_blocks(n, cnt);
+    if (early_start(blocks))
+        STS_CK(launch_pdl(k, dim3(blocks), dim3(kRedThreads), 0, st, w, V, n, hcoef, partial, out, n_out, ticket, G));
+    else
+        k<<<blocks, kRedThreads, 0, st>>>(w, V, n, hcoef, partial, out, n_out, ticket, G);
+    STS_LAUNCHED();
+    return STS_OK;
 }
 
 __global__ void k_sub(double *r, const double *b, const double *y, long long n) {
@@ -300,29 +338,35 @@ struct Red {
     // kernel's last block (h->kry.ticket)
     sts_status dots(const double *V, int k, const double *w, int self, double *out) {
         Krylov &K = h->kry;
-        const int ld = K.m + 2;
-        for (int i0 = 0; i0 < k; i0 += kDotChunk) {
-            const int cnt = std::min(kDotChunk, k - i0);
-            const int sf = self && (i0 + cnt == k);
-            mdot_dispatch(cnt, V, n, i0, w, K.partial, ld, sf != 0, out, K.ticket, h->stream);
-            STS_LAUNCHED();
+        for (int i0 = 0; i0 < k; i0 += kOrthChunk) {
+            const int cnt = std::min(kOrthChunk, k - i0);
+            STS_TRY(orth_launch(kDots, cnt, const_cast<double *>(w), V + (size_t)i0 * n, n, nullptr, K.partial,
+                                out + i0, cnt + (self && i0 + cnt == k ? 1 : 0), K.ticket, h->stream));
         }
         return STS_OK;
     }
-    sts_status update(double *w, const double *V, int k, const double *hcoef, int norm, double *out) {
+    // the squared norm goes to out[0] (norm = 1) and, with G.H, on to the rotations
+    sts_status update(double *w, const double *V, int k, const double *hcoef, int norm, double *out,
+                      const Givens &G = {}) {
         Krylov &K = h->kry;
-        for (int i0 = 0; i0 < k; i0 += kDotChunk) {
-            const int cnt = std::min(kDotChunk, k - i0);
-            update_dispatch(cnt, w, V, n, hcoef, i0, norm && i0 + cnt == k, K.partial, out, K.ticket, h->stream);
-            STS_LAUNCHED();
+        for (int i0 = 0; i0 < k; i0 += kOrthChunk) {
+            const int cnt = std::min(kOrthChunk, k - i0), fin = norm && i0 + cnt == k;
+            STS_TRY(orth_launch(kUpdateNorm, cnt, w, V + (size_t)i0 * n, n, hcoef + i0, K.partial, out, fin, K.ticket,
+                                h->stream, fin ? G : Givens{}));
         }
         return STS_OK;
+    }
+    // update with hcoef, then the dots of the result
+    sts_status update_dots(double *w, const double *V, int k, const double *hcoef, double *out) {
+        Krylov &K = h->kry;
+        if (k <= kOrthChunk)
+            return orth_launch(kUpdateDots, k, w, V, n, hcoef, K.partial, out, k, K.ticket, h->stream);
+        STS_TRY(update(w, V, k, hcoef, 0, nullptr));
+        return dots(V, k, w, 0, out);
     }
     sts_status norm2(const double *v, double *out) {
         Krylov &K = h->kry;
-        k_norm2<<<kRedBlocks, kRedThreads, 0, h->stream>>>(v, n, K.partial, out, K.ticket);
-        STS_LAUNCHED();
-        return STS_OK;
+        return orth_launch(kDots, 0, const_cast<double *>(v), v, n, nullptr, K.partial, out, 1, K.ticket, h->stream);
     }
 };
 
@@ -357,7 +401,7 @@ sts_status ensure_workspace(sts_jac_s *h, int m, bool mixed) {
         K.m = 0;
         STS_TRY(dalloc(h, &K.V, (size_t)(m + 1) * n));
         STS_TRY(dalloc(h, &K.Z, (size_t)m * n));
-        STS_TRY(dalloc(h, &K.partial, (size_t)kRedBlocks * (m + 2)));
+        STS_TRY(dalloc(h, &K.partial, (size_t)kRedMax * 32));
         STS_TRY(dalloc(h, &K.red, (size_t)3 * (m + 2)));
         if (!K.ticket) {
             STS_TRY(dalloc(h, &K.ticket, 1));
@@ -389,56 +433,15 @@ sts_status ensure_workspace(sts_jac_s *h, int m, bool mixed) {
 // One Arnoldi cycle as a CUDA graph.  Step j of the cycle is the body of a
 // conditional (IF) node, nested in step j - 1's body: z_j = M v_j, w = A z_j,
 // the two Gram-Schmidt passes,
-// then k_givens, which folds the new Hessenberg column into the rotations on
+// of which the last folds the new Hessenberg column into the rotations on
 // the device (the host loop's arithmetic, in the same order), records the
 // rotated residual, and switches step j + 1 on or off, and finally v_{j+1} =
 // w / h(j+1, j).  The host launches the graph once per cycle and reads the
 // rotated system back once, instead of synchronising after every step.
 
-// Step j's rotations (one thread).  red: h1 at red[0..], h2 at red[ld..], the
-// squared norm at red[2 ld]; par: stop threshold, history scale, 1 / h(j+1,j)
-// (output), steps allowed; state: steps taken, stop reason (0 none, 1
-// criterion met, 2 NaN or Inf).
-__global__ void k_givens(int j, int m, const double *red, int ld, double *H, double *cs, double *sn, double *g,
-                         double *hist, double *par, int *state, cudaGraphConditionalHandle next, int has_next) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    const double *h1 = red, *h2 = red + ld;
-    const double w0 = sqrt(h1[j + 1]);
-    const double hn = sqrt(red[2 * ld]);
-    bool bad = !isfinite(w0) || !isfinite(hn);
-    for (int i = 0; i <= j; ++i) {
-        H[(size_t)i * m + j] = h1[i] + h2[i];
-        bad = bad || !isfinite(H[(size_t)i * m + j]);
-    }
-    int stop = 0;
-    if (bad) {
-        stop = 2;
-    } else {
-        H[(size_t)(j + 1) * m + j] = hn;
-        for (int i = 0; i < j; ++i) {
-            const double a = H[(size_t)i * m + j], c = H[(size_t)(i + 1) * m + j];
-            H[(size_t)i * m + j] = cs[i] * a + sn[i] * c;
-            H[(size_t)(i + 1) * m + j] = -sn[i] * a + cs[i] * c;
-        }
-        const double hjj = H[(size_t)j * m + j];
-        const double den = hypot(hjj, hn);
-        cs[j] = hjj / den;
-        sn[j] = hn / den;
-        H[(size_t)j * m + j] = den;
-        H[(size_t)(j + 1) * m + j] = 0.0;
-        g[j + 1] = -sn[j] * g[j];
-        g[j] = cs[j] * g[j];
-        hist[j] = fabs(g[j + 1]) * par[1];
-        const bool happy = hn <= 1e-14 * w0;
-        if (happy || fabs(g[j + 1]) <= par[0] || (double)(j + 1) >= par[3]) stop = 1;
-        par[2] = 1.0 / hn;
-    }
-    state[0] = j + 1;
-    state[1] = stop;
-    if (has_next) cudaGraphSetConditional(next, stop ? 0u : 1u);
-}
-
 __global__ void k_scale_dev(double *out, const double *in, const double *s, long long n) {
+    pdl_wait();
+    pdl_trigger();
     const double f = *s;
     for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < n;
          e += (long long)gridDim.x * blockDim.x)
@@ -466,7 +469,7 @@ sts_status cycle_graph(sts_jac_s *h, int m, int dir, bool pre) {
         STS_CK(cudaMallocHost(&K.g_pinned, sizeof(double) * ((M + 1) * M + (M + 1) + M + 8)));
     }
     const long long n = (long long)h->b * h->ncp;
-    const int ld = m + 2;
+    const int ld = m + 2, nb = grid_for(n, 256);
     cudaGraph_t graph = nullptr;
     STS_CK(cudaGraphCreate(&graph, 0));
     cudaStream_t cs = nullptr;
@@ -504,16 +507,16 @@ sts_status cycle_graph(sts_jac_s *h, int m, int dir, bool pre) {
             else STS_CK(cudaMemcpyAsync(zj, vj, n * sizeof(double), cudaMemcpyDeviceToDevice, cs));
             STS_TRY(opA64(h, dir, zj, K.w));
             double *h1 = K.red, *h2 = K.red + ld, *nr = K.red + 2 * ld;
-            STS_TRY(R.dots(K.V, j + 1, K.w, 1, h1));
-            STS_TRY(R.update(K.w, K.V, j + 1, h1, 0, nullptr));
-            STS_TRY(R.dots(K.V, j + 1, K.w, 0, h2));
-            STS_TRY(R.update(K.w, K.V, j + 1, h2, 1, nr));
             const int has_next = j + 1 < m ? 1 : 0;
-            k_givens<<<1, 32, 0, cs>>>(j, m, K.red, ld, K.gH, K.gcs, K.gsn, K.gg, K.ghist, K.gpar, K.gstate,
-                                       has_next ? hd[j + 1] : hd[j], has_next);
-            STS_LAUNCHED();
+            const Givens G{j, m, h1, h2, K.gH, K.gcs, K.gsn, K.gg, K.ghist, K.gpar, K.gstate,
+                           has_next ? hd[j + 1] : hd[j], has_next};
+            STS_TRY(R.dots(K.V, j + 1, K.w, 1, h1));
+            STS_TRY(R.update_dots(K.w, K.V, j + 1, h1, h2));
+            STS_TRY(R.update(K.w, K.V, j + 1, h2, 1, nr, G));
             if (has_next) {
-                k_scale_dev<<<grid_for(n, 256), 256, 0, cs>>>(K.V + (size_t)(j + 1) * n, K.w, K.gpar + 2, n);
+                double *vn = K.V + (size_t)(j + 1) * n;
+                if (early_start(nb)) STS_CK(launch_pdl(k_scale_dev, dim3(nb), dim3(256), 0, cs, vn, K.w, K.gpar + 2, n));
+                else k_scale_dev<<<nb, 256, 0, cs>>>(vn, K.w, K.gpar + 2, n);
                 STS_LAUNCHED();
             }
             return STS_OK;
@@ -758,8 +761,7 @@ sts_status gmres(sts_jac_s *h, const double *b_pub, double *x_pub, const sts_gmr
                 // CGS2: h1 = V^T w (+ w.w), w -= V h1; h2 = V^T w, w -= V h2, ||w||^2
                 double *h1 = K.red, *h2 = K.red + (m + 2), *nr = K.red + 2 * (m + 2);
                 STS_TRY(R.dots(K.V, j + 1, K.w, 1, h1));
-                STS_TRY(R.update(K.w, K.V, j + 1, h1, 0, nullptr));
-                STS_TRY(R.dots(K.V, j + 1, K.w, 0, h2));
+                STS_TRY(R.update_dots(K.w, K.V, j + 1, h1, h2));
                 STS_TRY(R.update(K.w, K.V, j + 1, h2, 1, nr));
                 STS_CK(cudaMemcpyAsync(hp, K.red, sizeof(double) * 3 * (m + 2), cudaMemcpyDeviceToHost, h->stream));
                 STS_CK(cudaStreamSynchronize(h->stream));
