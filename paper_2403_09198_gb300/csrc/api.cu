@@ -281,8 +281,10 @@ sts_status build_plan(sts_jac_s *h, int dir, bool with_streams) {
             maxlen = std::max(maxlen, row_off[p + 1] - start);
         }
         P.tile_len = row_off[b];
-        // row groups: contiguous rows, balanced by stream length
-        const long long target = std::max(maxlen, (P.tile_len + 15) / 16);
+        // row groups: contiguous rows, balanced by stream length: 16 per tile, or on small
+        // meshes as many as give every SM 16 warps, down to single rows
+        const long long ng = std::max(16, (16 * h->nsm + nt - 1) / nt);
+        const long long target = std::max(maxlen, (P.tile_len + ng - 1) / ng);
         long long cur = 0;
         for (int p = 0; p < b; ++p) {
             const long long len = row_off[p + 1] - row_off[p];
@@ -303,8 +305,12 @@ sts_status build_plan(sts_jac_s *h, int dir, bool with_streams) {
         }
     }
     P.n_dtasks = (int)dtask_slot.size();
-    P.h_grp_rows = grp;
-    P.h_row_off = row_off;
+    std::vector<int4> groups;
+    if (!P.structured)
+        for (int g = 0; g < P.n_groups; ++g) {
+            const long long q0 = row_off[grp[g]];
+            groups.push_back(make_int4(grp[g], (int)(row_off[grp[g + 1]] - q0), (int)(q0 & 0xffffffffll), (int)(q0 >> 32)));
+        }
     P.h_pslot_slot = pslot_slot;
     P.h_blk = blk;
     std::vector<int> pat_ptr(2 * (b + 1)), pat_idx;
@@ -315,8 +321,7 @@ sts_status build_plan(sts_jac_s *h, int dir, bool with_streams) {
     STS_TRY(upload(h, &P.nbr, nbr));
     STS_TRY(upload(h, &P.blk, blk));
     STS_TRY(upload(h, &P.slot_mask, mask));
-    STS_TRY(upload(h, &P.grp_rows, grp));
-    STS_TRY(upload(h, &P.row_off, row_off));
+    STS_TRY(upload(h, &P.grp, groups));
     STS_TRY(upload(h, &P.dtask_slot, dtask_slot));
     STS_TRY(upload(h, &P.pat_ptr, pat_ptr));
     STS_TRY(upload(h, &P.pat_idx, pat_idx));
@@ -581,19 +586,35 @@ sts_status create_impl(const sts_jac_desc *d, sts_jac_t *out) {
     return STS_OK;
 }
 
-// Run an operator on public-layout vectors through the internal layout.  With
-// the component-major layout and no padding cells the kernels work in place.
+// Run an operator on public-layout vectors: in place where the kernels can take them
+// (any_layout), else through the internal layout.  In place are component-major vectors,
+// whose 32 cells of a component are contiguous (aligned or not), and cell-major ones of
+// up to direct_max values.  A lane's component of a cell-major vector is a sector of its
+// own, but two transposes per call, each a launch, are saved.  Measured on cell-major
+// vectors, us per call through the internal layout and in place:
+//   apply, 2 to 1152 tiles of 32 cells, N = 10: 18.6 and 10.5 (30.9 and 19.9 at 1152 tiles);
+//     N = 60: 51.4 and 42.3 at 2 tiles, 57.5 and 46.3 at 512, 104.8 and 90.0 at 1152: always;
+//   matvec, which reads x about 25 times, N = 10: 21.8 and 12.8 at 2 tiles, 70.2 and 60.7 at
+//     1152 (479 K values); N = 60: 47.0 and 43.6 at 128 tiles (258 K values), 74.6 and 77.9 at
+//     288 (581 K), 113.4 and 113.6 at 512.
+constexpr long long kMatvecDirect = 1 << 19, kApplyDirect = 1LL << 62;
+
 template <typename T, typename F>
-sts_status with_layout(sts_jac_s *h, const T *x, T *y, T *bin, T *bout, F op) {
-    if (h->layout == STS_LAYOUT_COMPONENT_MAJOR && h->nc == h->ncp) return op(x, y);
+sts_status with_layout(sts_jac_s *h, bool any_layout, long long direct_max, const T *x, T *y, T *bin, T *bout, F op) {
+    const bool comp = h->layout == STS_LAYOUT_COMPONENT_MAJOR;
+    if (any_layout && (comp || (long long)h->nc * h->b <= direct_max)) {
+        const long long sc = comp ? 1 : h->b, sq = comp ? h->nc : 1;
+        return op(Vec<T>{const_cast<T *>(x), sc, sq, h->nc, bout}, Vec<T>{y, sc, sq, h->nc, bout});
+    }
+    if (comp && h->nc == h->ncp) return op(internal_vec(h, x), internal_vec(h, y));
     if constexpr (sizeof(T) == 8) {
-        STS_TRY(to_internal64(h, reinterpret_cast<const double *>(x), reinterpret_cast<double *>(bin)));
-        STS_TRY(op(bin, bout));
-        return from_internal64(h, reinterpret_cast<const double *>(bout), reinterpret_cast<double *>(y));
+        STS_TRY(to_internal64(h, x, bin));
+        STS_TRY(op(internal_vec(h, bin), internal_vec(h, bout)));
+        return from_internal64(h, bout, y);
     } else {
-        STS_TRY(to_internal32(h, reinterpret_cast<const float *>(x), reinterpret_cast<float *>(bin)));
-        STS_TRY(op(bin, bout));
-        return from_internal32(h, reinterpret_cast<const float *>(bout), reinterpret_cast<float *>(y));
+        STS_TRY(to_internal32(h, x, bin));
+        STS_TRY(op(internal_vec(h, bin), internal_vec(h, bout)));
+        return from_internal32(h, bout, y);
     }
 }
 
@@ -672,8 +693,9 @@ sts_status sts_jac_matvec(sts_jac_t h, const double *x, double *y, int trans) {
     if (trans && (!h->has_T || h->rep != STS_REP_FACTORED))
         return set_error(STS_ERR_INVALID_ARG, "sts_jac_matvec: trans = 1 needs a factored handle with enable_transpose");
     const int dir = trans ? 1 : 0;
-    STS_GUARD(return with_layout<double>(h, x, y, h->vin, h->vout, [&](const double *a, double *b) {
-        return op_matvec64(h, dir, a, b);
+    STS_GUARD(return with_layout<double>(h, h->rep == STS_REP_FACTORED, kMatvecDirect, x, y, h->vin, h->vout,
+                                         [&](const Vec<double> &a, const Vec<double> &b) {
+        return h->rep == STS_REP_FACTORED ? mv_apply64(h, dir, a, b, h->c64) : op_matvec64(h, dir, a.p, b.p);
     });)
 }
 
@@ -685,7 +707,8 @@ sts_status sts_jac_matvec_noalloc(sts_jac_t h, const double *x, double *y, int t
     if (trans && !h->has_T)
         return set_error(STS_ERR_INVALID_ARG, "sts_jac_matvec_noalloc: trans = 1 needs enable_transpose");
     const int dir = trans ? 1 : 0;
-    STS_GUARD(return with_layout<double>(h, x, y, h->vin, h->vout, [&](const double *a, double *b) {
+    STS_GUARD(return with_layout<double>(h, true, kMatvecDirect, x, y, h->vin, h->vout,
+                                         [&](const Vec<double> &a, const Vec<double> &b) {
         return mv_apply64_noalloc(h, dir, a, b);
     });)
 }
@@ -696,7 +719,8 @@ sts_status sts_jac_matvec_f32(sts_jac_t h, const float *x, float *y, int trans) 
     if (h->dtype != STS_MIXED) return set_error(STS_ERR_INVALID_ARG, "sts_jac_matvec_f32: handle has no FP32 operators");
     if (trans && !h->has_T) return set_error(STS_ERR_INVALID_ARG, "sts_jac_matvec_f32: no transposed operators");
     const int dir = trans ? 1 : 0;
-    STS_GUARD(return with_layout<float>(h, x, y, h->vin32, h->vout32, [&](const float *a, float *b) {
+    STS_GUARD(return with_layout<float>(h, true, kMatvecDirect, x, y, h->vin32, h->vout32,
+                                        [&](const Vec<float> &a, const Vec<float> &b) {
         return mv_apply32(h, dir, a, b, h->c32);
     });)
 }
@@ -716,8 +740,10 @@ sts_status sts_jac_bjacobi_apply(sts_jac_t h, const double *x, double *z, int tr
     if (trans && (!h->has_T || h->rep != STS_REP_FACTORED))
         return set_error(STS_ERR_INVALID_ARG, "sts_jac_bjacobi_apply: trans = 1 needs enable_transpose");
     const int dir = trans ? 1 : 0;
-    STS_GUARD(return with_layout<double>(h, x, z, h->vin, h->vout, [&](const double *a, double *b) {
-        return op_apply64(h, dir, a, b);
+    const bool fact = h->rep == STS_REP_FACTORED;
+    STS_GUARD(return with_layout<double>(h, fact && smw_apply_any_layout(h, 8), kApplyDirect, x, z, h->vin, h->vout,
+                                         [&](const Vec<double> &a, const Vec<double> &b) {
+        return fact ? smw_apply64(h, dir, a, b) : op_apply64(h, dir, a.p, b.p);
     });)
 }
 
@@ -728,7 +754,8 @@ sts_status sts_jac_bjacobi_apply_f32(sts_jac_t h, const float *x, float *z, int 
     if (!h->smw.ready) return set_error(STS_ERR_NOT_SETUP, "sts_jac_bjacobi_apply_f32: call sts_jac_bjacobi_setup first");
     if (trans && !h->has_T) return set_error(STS_ERR_INVALID_ARG, "sts_jac_bjacobi_apply_f32: no transposed operators");
     const int dir = trans ? 1 : 0;
-    STS_GUARD(return with_layout<float>(h, x, z, h->vin32, h->vout32, [&](const float *a, float *b) {
+    STS_GUARD(return with_layout<float>(h, smw_apply_any_layout(h, 4), kApplyDirect, x, z, h->vin32, h->vout32,
+                                        [&](const Vec<float> &a, const Vec<float> &b) {
         return smw_apply32(h, dir, a, b);
     });)
 }

@@ -324,11 +324,11 @@ inline int grid_for(long long n, int block) {
 // Operators shared with the public entry points.
 sts_status opA64(sts_jac_s *h, int dir, const double *x, double *y) {
     if (h->rep == STS_REP_DENSE_BSR) return dense_matvec(h, x, y);
-    return mv_apply64(h, dir, x, y, h->c64);
+    return mv_apply64(h, dir, internal_vec(h, x), internal_vec(h, y), h->c64);
 }
 sts_status opM64(sts_jac_s *h, int dir, const double *x, double *z) {
     if (h->rep == STS_REP_DENSE_BSR) return dense_apply(h, x, z);
-    return smw_apply64(h, dir, x, z);
+    return smw_apply64(h, dir, internal_vec(h, x), internal_vec(h, z));
 }
 
 struct Red {
@@ -753,8 +753,8 @@ sts_status gmres(sts_jac_s *h, const double *b_pub, double *x_pub, const sts_gmr
                     float *zj = K.Z32 + (size_t)j * n;
                     k_convert<float, double><<<nb, 256, 0, h->stream>>>(pre ? K.t32a : zj, vj, n);
                     STS_LAUNCHED();
-                    if (pre) STS_TRY(smw_apply32(h, dir, K.t32a, zj));
-                    STS_TRY(mv_apply32(h, dir, zj, K.t32b, h->c32));
+                    if (pre) STS_TRY(smw_apply32(h, dir, internal_vec(h, K.t32a), internal_vec(h, zj)));
+                    STS_TRY(mv_apply32(h, dir, internal_vec(h, zj), internal_vec(h, K.t32b), h->c32));
                     k_convert<double, float><<<nb, 256, 0, h->stream>>>(K.w, K.t32b, n);
                     STS_LAUNCHED();
                 }

@@ -29,16 +29,14 @@ template <typename T>
 struct MvArgs {
     const T *main;          // [n_tiles][tile_len][32]
     const T *dotv;          // [n_tiles][n_dtasks][Lp][32]
-    const T *x;             // [b][ncp]
-    T *y;                   // [b][ncp]
+    Vec<T> x, y;
     T *c;                   // [n_tiles][n_dtasks][32]
     int *err;               // set when a bounded wait gave up
     unsigned *sched;        // [2] pass-2 item counter and finished warps, zero between launches
     int pre;                // the coefficient streams may be read before the grid-dependency wait
     const int *nbr;         // [n_tiles][n_slots][32]
     const unsigned *slot_mask;
-    const int *grp_rows;
-    const long long *row_off;
+    const int4 *grp;        // [n_groups] generic main pass: first row, positions, first position
     const int *dtask_slot;  // [n_dtasks]
     const int *pat_ptr;     // [2][b+1]
     const int *pat_idx;
@@ -107,21 +105,21 @@ __global__ void __launch_bounds__(128) k_dots(MvArgs<T> a) {
     T acc = T(0);
     if (present) {
         // an absent neighbour reads the lane's own cell: its coefficients are zero
-        const T *__restrict__ xj = a.x + (j >= 0 ? j : t * kTile + lane);
+        const T *__restrict__ xj = a.x.at(j >= 0 ? j : t * kTile + lane);
         const int bm1 = a.b - 1;
-        const size_t ncp = a.ncp;
+        const size_t sq = (size_t)a.x.sq;
         if (!a.pre) {
 #pragma unroll
             for (int i = 0; i < NV; ++i) va[i] = __ldcs(dv + i * kTile);
         }
 #pragma unroll
-        for (int i = 0; i < CH; ++i) xa[i] = __ldg(xj + (size_t)min(i, bm1) * ncp);
+        for (int i = 0; i < CH; ++i) xa[i] = __ldg(xj + (size_t)min(i, bm1) * sq);
         for (int base = 0; base < a.Lp; base += 2 * CH) {
             if (base + CH < a.Lp) {
 #pragma unroll
                 for (int i = 0; i < NV; ++i) vb[i] = __ldcs(dv + ((base + CH) / VEC + i) * kTile);
 #pragma unroll
-                for (int i = 0; i < CH; ++i) xb[i] = __ldg(xj + (size_t)min(base + CH + i, bm1) * ncp);
+                for (int i = 0; i < CH; ++i) xb[i] = __ldg(xj + (size_t)min(base + CH + i, bm1) * sq);
             }
 #pragma unroll
             for (int i = 0; i < CH; ++i) acc = fma(dot_el(va[i / VEC], i % VEC), xa[i], acc);
@@ -130,7 +128,7 @@ __global__ void __launch_bounds__(128) k_dots(MvArgs<T> a) {
 #pragma unroll
                 for (int i = 0; i < NV; ++i) va[i] = __ldcs(dv + ((base + 2 * CH) / VEC + i) * kTile);
 #pragma unroll
-                for (int i = 0; i < CH; ++i) xa[i] = __ldg(xj + (size_t)min(base + 2 * CH + i, bm1) * ncp);
+                for (int i = 0; i < CH; ++i) xa[i] = __ldg(xj + (size_t)min(base + 2 * CH + i, bm1) * sq);
             }
 #pragma unroll
             for (int i = 0; i < CH; ++i) acc = fma(dot_el(vb[i / VEC], i % VEC), xb[i], acc);
@@ -143,57 +141,84 @@ __global__ void __launch_bounds__(128) k_dots(MvArgs<T> a) {
 // group's stream positions are consumed in order under a flat program (one
 // descriptor per position: column and block slot of an S entry, or the pair
 // slot of a pair term, plus an end-of-row flag); each row is accumulated
-// serially.  Stream values are double-buffered in registers one chunk ahead.
+// serially.  A chunk's values and operands are loaded one chunk ahead: an operand's
+// address comes out of its descriptor, so a load at its use is two memory latencies
+// per position.  With few tiles a group is one row and a warp's own instructions set
+// the time (41 x 37 cells, b = 33, 15% filled: 22 us, now 10).
 template <typename T>
 __global__ void __launch_bounds__(128) k_mv_main(MvArgs<T> a) {
-    constexpr int CH = Chunk<T>::CH;
+    constexpr int CH = 8;
     __shared__ int snb[4][kMaxSlots][kTile];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const long long wid = (long long)blockIdx.x * (blockDim.x >> 5) + wib;
     if (wid >= (long long)a.n_tiles * a.n_groups) return;
     const int t = (int)(wid / a.n_groups), g = (int)(wid % a.n_groups);
-    for (int s = 0; s < a.n_slots; ++s) snb[wib][s][lane] = a.nbr[((size_t)t * a.n_slots + s) * kTile + lane];
-    __syncwarp();
-    const int p0 = a.grp_rows[g], p1 = a.grp_rows[g + 1];
-    const long long q0 = a.row_off[p0];
-    const int L = (int)(a.row_off[p1] - q0);
+    const int4 grp = __ldg(a.grp + g);          // first row, positions, first position (low, high)
+    const int p0 = grp.x, L = grp.y;
+    const long long q0 = (long long)(unsigned)grp.z | ((long long)grp.w << 32);
     const T *__restrict__ sv = a.main + ((size_t)t * a.tile_len + q0) * kTile + lane;
+    if (lane == 0) prefetch_l2_bulk(sv, (unsigned)L * kTile * (unsigned)sizeof(T));
+    const int *__restrict__ nb = a.nbr + (size_t)t * a.n_slots * kTile + lane;
+    // offset of a slot's cell in x; complemented where the neighbour is absent, whose own cell
+    // is read and not used.  Offsets fit 32 bits: a vector has fewer than 2^31 values
+    const int own = min(t * kTile + lane, a.x.cells - 1), xc = (int)a.x.sc, xq = (int)a.x.sq;
+#pragma unroll 8
+    for (int s = 0; s < a.n_slots; ++s) {
+        const int j = __ldg(nb + s * kTile);
+        snb[wib][s][lane] = j >= 0 ? j * xc : ~(own * xc);
+    }
+    __syncwarp();
     const unsigned *__restrict__ dd = a.desc + q0;
-    const T *__restrict__ xp = a.x;
+    const T *__restrict__ xp = a.x.p;
     const T *__restrict__ cc = a.c + (size_t)t * a.n_dtasks * kTile + lane;
-    T *__restrict__ yp = a.y + (size_t)p0 * a.ncp + (size_t)t * kTile + lane;
-    T cur[CH], nxt[CH];
+    long long ystep;
+    T *__restrict__ yp = a.y.out(t * kTile + lane, ystep);
+    yp += p0 * ystep;
+    T v[CH], o[CH], vn[CH], on[CH];
+    unsigned d[CH], dn[CH], df[CH], gone = 0, gone_n = 0;     // of this chunk, the next one, and the one after
+    // past the end of the group the last position is read again, and not used; no branch
+    // stands between the loads of a chunk, so all of them are in flight together
+    auto fetch_desc = [&](int base) {
 #pragma unroll
-    for (int i = 0; i < CH; ++i) cur[i] = i < L ? __ldg(sv + (size_t)i * kTile) : T(0);
+        for (int i = 0; i < CH; ++i) df[i] = __ldg(dd + min(base + i, L - 1));
+    };
+    auto fetch = [&](int base) {
+#pragma unroll
+        for (int i = 0; i < CH; ++i) dn[i] = df[i];
+#pragma unroll
+        for (int i = 0; i < CH; ++i) vn[i] = __ldg(sv + min(base + i, L - 1) * kTile);
+        gone_n = 0;
+#pragma unroll
+        for (int i = 0; i < CH; ++i) {
+            const int k = (int)(dn[i] & 0xffffu), off = snb[wib][(dn[i] >> 16) & 0x1fu][lane];
+            const bool pair = dn[i] & kDescPair;
+            gone_n |= !pair && off < 0 ? 1u << i : 0u;
+            on[i] = __ldg((pair ? cc : xp) + (pair ? (unsigned)(k * kTile) : (unsigned)k * (unsigned)xq + (unsigned)(off >= 0 ? off : ~off)));
+        }
+        fetch_desc(base + CH);
+    };
+    fetch_desc(0);
+    fetch(0);
     T acc = T(0);
     for (int base = 0; base < L; base += CH) {
 #pragma unroll
         for (int i = 0; i < CH; ++i) {
-            const int pp = base + CH + i;
-            nxt[i] = pp < L ? __ldg(sv + (size_t)pp * kTile) : T(0);
+            v[i] = vn[i];
+            o[i] = on[i];
+            d[i] = dn[i];
         }
+        gone = gone_n;
+        if (base + CH < L) fetch(base + CH);
 #pragma unroll
         for (int i = 0; i < CH; ++i) {
-            const int pp = base + i;
-            if (pp < L) {
-                const unsigned d = __ldg(dd + pp);
-                T opnd;
-                if (d & kDescPair) {
-                    opnd = __ldg(cc + (size_t)(d & 0xffffu) * kTile);
-                } else {
-                    const int j = snb[wib][(d >> 16) & 0x1fu][lane];
-                    opnd = j >= 0 ? __ldg(xp + (size_t)(d & 0xffffu) * a.ncp + j) : T(0);
-                }
-                acc = fma(cur[i], opnd, acc);
-                if (d & kDescEnd) {
-                    *yp = acc;
-                    yp += a.ncp;
-                    acc = T(0);
-                }
+            if (base + i >= L) break;
+            acc = fma(v[i], gone >> i & 1u ? T(0) : o[i], acc);
+            if (d[i] & kDescEnd) {
+                *yp = acc;
+                yp += ystep;
+                acc = T(0);
             }
         }
-#pragma unroll
-        for (int i = 0; i < CH; ++i) cur[i] = nxt[i];
     }
 }
 
@@ -232,7 +257,7 @@ __global__ void __launch_bounds__(64) k_mv_struct(MvArgs<T> a) {
     constexpr int BANDW = 2 * WD + 1;
     const int lane = threadIdx.x & 31;
     const int ns = a.n_slots, nps = a.n_pslots, N = a.sN;
-    const size_t ncp = a.ncp;
+    const size_t sq = (size_t)a.x.sq;
     const int RL = a.s_rl;
     const uint32_t row_bytes = (uint32_t)RL * kTile * (uint32_t)sizeof(T);
     extern __shared__ __align__(128) unsigned char mv_smem[];
@@ -277,7 +302,9 @@ __global__ void __launch_bounds__(64) k_mv_struct(MvArgs<T> a) {
     for (long long wid = wid0; wid < n_items; wid = wstep + (long long)__shfl_sync(0xffffffffu, ticket, 0)) {
     if (lane == 0) ticket = atomicAdd(a.sched, 1u);
     const int t = (int)(wid / a.n_groups), g = (int)(wid % a.n_groups);
-    const size_t cell = (size_t)t * kTile + lane;
+    const int cell = t * kTile + lane;
+    long long ystep;
+    T *const ycell = a.y.out(cell, ystep);
     const T *__restrict__ cc = a.c + (size_t)t * a.n_dtasks * kTile + lane;
     if (g == a.n_lgroups) {
         const T *__restrict__ su = a.main + ((size_t)t * a.tile_len + (size_t)N * RL) * kTile + lane;
@@ -287,7 +314,7 @@ __global__ void __launch_bounds__(64) k_mv_struct(MvArgs<T> a) {
             for (int s = 0; s < ns; ++s) acc += __ldg(cc + (size_t)(nps + f * ns + s) * kTile);
             for (int k = 0; k < nps; ++k)
                 acc = fma(__ldg(su + (size_t)(f * nps + k) * kTile), __ldg(cc + (size_t)k * kTile), acc);
-            a.y[(size_t)(N + f) * ncp + cell] = acc;
+            ycell[(N + f) * ystep] = acc;
         }
         continue;
     }
@@ -312,9 +339,9 @@ __global__ void __launch_bounds__(64) k_mv_struct(MvArgs<T> a) {
     for (int s = 0; s < NS; ++s) {
         const int j = s < ns ? a.nbr[((size_t)t * ns + s) * kTile + lane] : -1;
         // an absent neighbour reads the lane's own cell: its coefficients are zero
-        xs[s] = a.x + (j >= 0 ? (size_t)j : cell);
+        xs[s] = a.x.at(j >= 0 ? j : cell);
 #pragma unroll
-        for (int f = 0; f < NF; ++f) xf[s][f] = s < ns ? __ldg(xs[s] + (size_t)(N + f) * ncp) : T(0);
+        for (int f = 0; f < NF; ++f) xf[s][f] = s < ns ? __ldg(xs[s] + (size_t)(N + f) * sq) : T(0);
     }
     // pair dots in registers (see above): an optional block of RB = 16, then the
     // last m terms aligned to the end of the D switch slots
@@ -330,12 +357,12 @@ __global__ void __launch_bounds__(64) k_mv_struct(MvArgs<T> a) {
     // band window: xb[k] = x_own[p - WD + k] (clipped; clipped entries carry zero coefficients)
     T xb[BANDW];
 #pragma unroll
-    for (int k = 0; k + 1 < BANDW; ++k) xb[k + 1] = __ldg(xs[0] + (size_t)min(max(p0 - WD + k, 0), N - 1) * ncp);
-    T xbn = __ldg(xs[0] + (size_t)min(p0 + WD, N - 1) * ncp);
+    for (int k = 0; k + 1 < BANDW; ++k) xb[k + 1] = __ldg(xs[0] + (size_t)min(max(p0 - WD + k, 0), N - 1) * sq);
+    T xbn = __ldg(xs[0] + (size_t)min(p0 + WD, N - 1) * sq);
     T xn[NS];
 #pragma unroll
-    for (int s = 1; s < NS; ++s) xn[s] = s < ns ? __ldg(xs[s] + (size_t)p0 * ncp) : T(0);
-    T *yp = a.y + (size_t)p0 * ncp + cell;
+    for (int s = 1; s < NS; ++s) xn[s] = s < ns ? __ldg(xs[s] + (size_t)p0 * sq) : T(0);
+    T *yp = ycell + p0 * ystep;
     T ylag = T(0);          // row p-1's result, stored during row p (its FMA has long completed)
     for (int p = p0; p < p1; ++p) {
         const int sg = (p - p0) & 1;
@@ -356,10 +383,10 @@ __global__ void __launch_bounds__(64) k_mv_struct(MvArgs<T> a) {
 #pragma unroll
         for (int s = 1; s < NS; ++s) xc[s] = xn[s];
         if (p + 1 < p1) {
-            xbn = __ldg(xs[0] + (size_t)min(p + 1 + WD, N - 1) * ncp);
+            xbn = __ldg(xs[0] + (size_t)min(p + 1 + WD, N - 1) * sq);
 #pragma unroll
             for (int s = 1; s < NS; ++s)
-                if (s < ns) xn[s] = __ldg(xs[s] + (size_t)(p + 1) * ncp);
+                if (s < ns) xn[s] = __ldg(xs[s] + (size_t)(p + 1) * sq);
         }
         const T *v = stage0 + (size_t)sg * RL * kTile + lane;
         T acc = T(0);
@@ -422,7 +449,7 @@ __global__ void __launch_bounds__(64) k_mv_struct(MvArgs<T> a) {
         }
         if (p > p0) {
             *yp = ylag;
-            yp += ncp;
+            yp += ystep;
         }
         ylag = acc;
         __syncwarp();     // every lane is done with the stage before it is refilled
@@ -505,7 +532,7 @@ inline int grid_for(long long n, int block) {
 }
 
 template <typename T>
-MvArgs<T> make_args(sts_jac_s *h, int dir, const T *main, const T *dotv, const T *x, T *y, T *c) {
+MvArgs<T> make_args(sts_jac_s *h, int dir, const T *main, const T *dotv, const Vec<T> &x, const Vec<T> &y, T *c) {
     const MvPlan &P = h->mv[dir];
     MvArgs<T> a;
     a.main = main;
@@ -518,8 +545,7 @@ MvArgs<T> make_args(sts_jac_s *h, int dir, const T *main, const T *dotv, const T
     a.pre = h->streams_dirty ? 0 : 1;
     a.nbr = P.nbr;
     a.slot_mask = P.slot_mask;
-    a.grp_rows = P.grp_rows;
-    a.row_off = P.row_off;
+    a.grp = P.grp;
     a.dtask_slot = P.dtask_slot;
     a.pat_ptr = P.pat_ptr;
     a.pat_idx = P.pat_idx;
@@ -571,8 +597,13 @@ void (*mv_struct_kernel(int nreg))(MvArgs<T>) {
 inline int pass2_group_rows(int N, int n_tiles, long long W, int s_plan, int s_rl) {
     const long long items = (long long)n_tiles * ((N + s_plan - 1) / s_plan + 1);
     if (W <= 0 || items >= 8 * W) return s_plan;
-    const int s = (int)std::lround(3.8 * std::sqrt((double)N / std::max(s_rl, 1)));
-    return std::max(1, std::min({N, 8, std::max(4, s)}));
+    const int s = std::max(1, std::min({N, 8, std::max(4, (int)std::lround(3.8 * std::sqrt((double)N / std::max(s_rl, 1))))}));
+    // small meshes: the fewest rows that still give every item a warp of its own, so that
+    // a warp's serial rows, not the number of items, set the time (whole products, cell-major
+    // in place, us: N = 10, 32 tiles 22.1 -> 14.6, 128 tiles 26.0 -> 16.7; N = 60, 32 tiles
+    // 36.3 -> 21.9, 128 tiles 43.6 -> 39.9)
+    const long long per_tile = W / n_tiles - 1;
+    return per_tile > 0 ? (int)std::min<long long>(s, (N + per_tile - 1) / per_tile) : s;
 }
 
 template <typename T>
@@ -626,14 +657,14 @@ sts_status mv_launch(sts_jac_s *h, const MvArgs<T> &args) {
 
 }  // namespace
 
-sts_status mv_apply64(sts_jac_s *h, int dir, const double *x, double *y, double *c) {
+sts_status mv_apply64(sts_jac_s *h, int dir, const Vec<double> &x, const Vec<double> &y, double *c) {
     const MvPlan &P = h->mv[dir];
     return mv_launch<double>(h, make_args<double>(h, dir, P.main64, P.dotv64, x, y, c));
 }
 
 sts_status mv_dots64(sts_jac_s *h, int dir, const double *x, double *c) {
     const MvPlan &P = h->mv[dir];
-    return dots_launch<double>(h, make_args<double>(h, dir, P.main64, P.dotv64, x, nullptr, c));
+    return dots_launch<double>(h, make_args<double>(h, dir, P.main64, P.dotv64, internal_vec(h, x), Vec<double>{}, c));
 }
 
 // ---------------------------------------------------------------------------
@@ -654,7 +685,7 @@ constexpr int kNoAllocMaxDevices = 64;
 double *g_noalloc_ptr[kNoAllocMaxDevices] = {};
 }  // namespace
 
-sts_status mv_apply64_noalloc(sts_jac_s *h, int dir, const double *x, double *y) {
+sts_status mv_apply64_noalloc(sts_jac_s *h, int dir, const Vec<double> &x, const Vec<double> &y) {
     const MvPlan &P = h->mv[dir];
     const size_t need = (size_t)h->n_tiles * P.n_dtasks * kTile;
     if (need > kNoAllocScratch)
@@ -687,7 +718,7 @@ sts_status mv_apply64_noalloc(sts_jac_s *h, int dir, const double *x, double *y)
     return mv_launch<double>(h, make_args<double>(h, dir, P.main64, P.dotv64, x, y, c));
 }
 
-sts_status mv_apply32(sts_jac_s *h, int dir, const float *x, float *y, float *c) {
+sts_status mv_apply32(sts_jac_s *h, int dir, const Vec<float> &x, const Vec<float> &y, float *c) {
     const MvPlan &P = h->mv[dir];
     return mv_launch<float>(h, make_args<float>(h, dir, P.main32, P.dotv32, x, y, c));
 }

@@ -24,62 +24,131 @@ namespace {
 
 template <typename T>
 struct ApplyArgs {
-    const T *st;            // [len][ncp] stream
-    const unsigned *desc;   // [len] apply program
+    const T *st;            // [kGenWarps][wlen][ncp] coefficients of every warp, in its order
+    const short *row;       // [kGenWarps][wlen] row that a coefficient updates, -1: none
+    const int *n_fwd, *n_bwd;   // [b] coefficients of every warp for column j, forward and backward
     const T *dv;            // [r][b][ncp] dot vectors (V for N, U for T)
     const T *W;             // [r][b][ncp] (W for N, Wt for T)
     const double *Cinv;     // [r][r][ncp]
-    const T *x;
-    T *y;
-    int len, b, r, ncp, trans;
+    Vec<T> x, y;
+    int wlen, b, r, ncp, trans;
 };
 
-constexpr int kApStage = 32;    // stream positions per shared-memory stage
-constexpr int kApStages = 3;    // stages in flight (two ahead of the one consumed)
 
-// One warp per 32 cells, one lane per cell.  The tile's apply stream is
-// copied into a ring of shared-memory stages with cp.async two stages ahead of
-// its use; the working vector lives in shared memory [q][lane]; the triangular
-// sweeps run a flat program (one descriptor per stream position).
+// Any pattern: one block of four warps per 32 cells, one lane per cell.  The working
+// vector lives in shared memory [q][lane]; the sweeps go column by column, and the rows
+// that a column updates are dealt to the warps, so that four FP64 pipes share a tile's
+// work with one barrier per column.  Forward updates reach a row in ascending column
+// order, the order of a serial sweep over the rows.  Each warp's coefficients are one
+// sequence, loaded a batch of four ahead of its use and brought into L2 well before.
+//
+// As one warp's serial program over the rows a tile took 85 us for 33 x 33 blocks (41 x 37
+// cells, 15% filled before the factorisation), mostly one dependent step after
+// another; now 32 us.  Rings of bulk or cp.async stages in front of the batches took 39 us:
+// with one block on most SMs a warp's instructions per coefficient set the time.
+constexpr int kGenAhead = 4;        // coefficients of a batch; padding behind every warp's sequence
+constexpr int kGenPrefetch = 64;    // coefficients between one used and one brought into L2
+constexpr int kGenSum = 8;          // pairs whose partial sums are added at once
+
 template <typename T, int RMAX>
-__global__ void __launch_bounds__(32) k_smw_apply(ApplyArgs<T> a) {
+__global__ void __launch_bounds__(kGenWarps * kTile) k_smw_apply(ApplyArgs<T> a) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    T *stg = reinterpret_cast<T *>(smem_raw);                  // [kApStages][kApStage][32]
-    T *w = stg + kApStages * kApStage * kTile;                  // [b][32]
-    const int lane = threadIdx.x;
-    const int tile = blockIdx.x;
-    const int cell = tile * kTile + lane;
+    constexpr int U = kGenAhead, KC = RMAX < kGenSum ? RMAX : kGenSum;
+    T *part = reinterpret_cast<T *>(smem_raw);                     // [kGenWarps][KC][32]
+    T *w = part + kGenWarps * KC * kTile;                           // [b][32]
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int cell = blockIdx.x * kTile + lane, b = a.b;
     const size_t P = a.ncp;
-    const T *__restrict__ x = a.x;
-    Ring<T, kApStage, kApStages> R;
-    R.start(stg, a.st + (size_t)tile * kTile, P, a.len, lane);
-    for (int i = 0; i < a.b; ++i) w[i * kTile + lane] = __ldg(x + i * P + cell);
-    const unsigned *__restrict__ dd = a.desc;
-    T acc = T(0);
-    for (int i = 0; i < a.len; ++i) {
-        const unsigned d = __ldg(dd + i);
-        const T v = R.next();
-        const int row = (d >> 12) & 0xfffu, col = d & 0xfffu;
-        if (d & kApScale) {
-            acc = v * w[row * kTile + lane];
-        } else {
-            if (d & kApBegin) acc = w[row * kTile + lane];
-            acc = fma(-v, w[col * kTile + lane], acc);
+    const T *__restrict__ x = a.x.at(cell);
+    const T *__restrict__ st = a.st + (size_t)warp * a.wlen * P + cell;
+    const short *__restrict__ row = a.row + (size_t)warp * a.wlen;
+    // the next batch; the sequences end in U padding positions, there to be read
+    T vn[U];
+    int rn[U], left = a.wlen;
+    auto advance = [&](int n) {
+        st += (size_t)n * P;
+        row += n;
+        left -= n;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            vn[u] = __ldg(st + (size_t)u * P);
+            rn[u] = __ldg(row + u);
+            if (u < n && kGenPrefetch + u < left) prefetch_l2(st + (size_t)(kGenPrefetch + u) * P);
         }
-        if (d & kApEnd) w[row * kTile + lane] = acc;
+    };
+    for (int k = 0; k < min(kGenPrefetch + U, a.wlen); ++k) prefetch_l2(st + (size_t)k * P);
+    advance(0);
+    for (int i = warp; i < b; i += kGenWarps) w[i * kTile + lane] = __ldg(x + i * a.x.sq);
+    __syncthreads();
+    // n updates w[row] -= coefficient * xj: the rows of one column are distinct
+    auto column = [&](T xj, int n) {
+        for (int s = 0; s < n; s += U) {
+            T v[U], c[U];
+            int r[U];
+            const int m = min(U, n - s);
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                v[u] = vn[u];
+                r[u] = u < m ? rn[u] : -1;
+            }
+            advance(m);
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (r[u] >= 0) c[u] = w[r[u] * kTile + lane];
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (r[u] >= 0) w[r[u] * kTile + lane] = fma(-v[u], xj, c[u]);
+        }
+    };
+    for (int j = 0; j < b; ++j) {
+        const int n = __ldg(a.n_fwd + j);
+        if (n == 0) continue;
+        column(w[j * kTile + lane], n);
+        __syncthreads();
     }
-    R.finish();
-    // t = dv^T x0, z = C^-1 t (FP64), x = x0 - W z
+    // pivot inverses: ceil(b / kGenWarps) positions of every warp, the last one padding where
+    // the warps are too many
+    for (int i = warp; i < b; i += kGenWarps) {
+        const T v = vn[0];
+        advance(1);
+        w[i * kTile + lane] *= v;
+    }
+    if (b % kGenWarps && warp >= b % kGenWarps) advance(1);
+    __syncthreads();
+    for (int j = b - 1; j >= 0; --j) {
+        const int n = __ldg(a.n_bwd + j);
+        if (n == 0) continue;
+        column(w[j * kTile + lane], n);
+        __syncthreads();
+    }
+    // t = dv^T x0 over the warps' rows, z = C^-1 t (FP64), x = x0 - W z
     T t[RMAX];
 #pragma unroll
     for (int k = 0; k < RMAX; ++k) t[k] = T(0);
     const T *__restrict__ dv = a.dv + cell;
 #pragma unroll 4
-    for (int q = 0; q < a.b; ++q) {
+    for (int q = warp; q < b; q += kGenWarps) {
         const T xq = w[q * kTile + lane];
 #pragma unroll
         for (int k = 0; k < RMAX; ++k)
-            if (k < a.r) t[k] = fma(__ldg(dv + ((size_t)k * a.b + q) * P), xq, t[k]);
+            if (k < a.r) t[k] = fma(__ldg(dv + ((size_t)k * b + q) * P), xq, t[k]);
+    }
+#pragma unroll
+    for (int k0 = 0; k0 < RMAX; k0 += KC) {
+        if (k0 >= a.r) break;
+#pragma unroll
+        for (int k = 0; k < KC; ++k)
+            if (k0 + k < a.r) part[(warp * KC + k) * kTile + lane] = t[k0 + k];
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < KC; ++k)
+            if (k0 + k < a.r) {
+                T s = part[k * kTile + lane];
+#pragma unroll
+                for (int v = 1; v < kGenWarps; ++v) s += part[(v * KC + k) * kTile + lane];
+                t[k0 + k] = s;
+            }
+        __syncthreads();
     }
     T z[RMAX];
 #pragma unroll
@@ -97,13 +166,15 @@ __global__ void __launch_bounds__(32) k_smw_apply(ApplyArgs<T> a) {
         z[k] = (T)s;
     }
     const T *__restrict__ Wp = a.W + cell;
+    long long ystep;
+    T *__restrict__ y = a.y.out(cell, ystep);
 #pragma unroll 4
-    for (int q = 0; q < a.b; ++q) {
+    for (int q = warp; q < b; q += kGenWarps) {
         T v = w[q * kTile + lane];
 #pragma unroll
         for (int k = 0; k < RMAX; ++k)
-            if (k < a.r) v = fma(-__ldg(Wp + ((size_t)k * a.b + q) * P), z[k], v);
-        a.y[q * P + cell] = v;
+            if (k < a.r) v = fma(-__ldg(Wp + ((size_t)k * b + q) * P), z[k], v);
+        y[q * ystep] = v;
     }
 }
 
@@ -148,12 +219,12 @@ template <typename T>
 struct SApplyArgs {
     const T *st;            // [n_tiles][Lt / VEC][32][VEC]
     const double *Cinv;     // [r][r][ncp] (instances that do not fold only)
-    const T *x;
-    T *y;
+    Vec<T> x, y;            // internal layout where the working vector lives in y
     int *err;               // set when a bounded wait gave up
     int Lt, b, N, r, ncp, trans, n_tiles;
     int pre;                // the stream and C^-1 may be read before the grid-dependency wait
     int evict_first;        // the stream of one call is larger than L2
+    int bulk;               // FP64: 32 cells of a component of x are one aligned run
 };
 
 constexpr int kApWarps = 4;              // consumer warps per block of the structured apply (one per sub-partition)
@@ -311,25 +382,27 @@ __global__ void __launch_bounds__((kApWarps + 1) * 32) k_smw_sapply(SApplyArgs<T
     // against 12.9 us on 128 x 128 cells, N = 60).
     constexpr bool XBULK = !GW && sizeof(T) == 8;
     const uint32_t xbar = full + 8u * (2 * kSApStages);
-    if constexpr (XBULK) {
+    const bool bulk = XBULK && a.bulk;
+    if (bulk) {
         if (lane == 0) mbar_expect_tx(xbar, (uint32_t)((size_t)b * kTile * sizeof(T)));
         __syncwarp();
         for (int i = lane; i < b; i += kTile)
-            bulk_copy_g2s(smem_addr(wl - lane + (size_t)i * kTile), a.x + (size_t)i * P + (size_t)gw * kTile,
+            bulk_copy_g2s(smem_addr(wl - lane + (size_t)i * kTile), a.x.p + (size_t)i * P + (size_t)gw * kTile,
                           (uint32_t)(kTile * sizeof(T)), xbar);
     } else if constexpr (!GW) {
-        for (int i = 0; i < b; ++i) cp_async_elem(wl + i * kTile, a.x + (size_t)i * P + (size_t)gw * kTile + lane);
+        const T *x0 = a.x.at(gw * kTile + lane);
+        for (int i = 0; i < b; ++i) cp_async_elem(wl + i * kTile, x0 + (size_t)i * (size_t)a.x.sq);
         cp_async_commit();
     }
     for (int k = 0; k < my; ++k) {
         const int cell = (gw + k * nw) * kTile + lane;
         // row j of the working vector, and row j of this tile's x
         auto wv = [&](int j) -> T & {
-            if constexpr (GW) return a.y[(size_t)j * P + cell];
+            if constexpr (GW) return a.y.p[(size_t)j * P + cell];
             else return wl[j * kTile];
         };
         auto xin = [&](int j) -> T {
-            if constexpr (GW) return a.x[(size_t)j * P + cell];
+            if constexpr (GW) return a.x.p[(size_t)j * P + cell];
             else return wl[j * kTile];
         };
         double cz[FOLD ? 1 : RMAX * RMAX];      // C^-1 (transposed for A^T), zero outside r x r
@@ -343,7 +416,7 @@ __global__ void __launch_bounds__((kApWarps + 1) * 32) k_smw_sapply(SApplyArgs<T
                                          : 0.0;
         }
         if constexpr (!GW) {
-            if (XBULK && k == 0) {
+            if (bulk && k == 0) {
                 if (!mbar_wait_bounded(xbar, 0)) goto fail;
             } else {
                 cp_async_wait<0>();             // copied in by the previous tile's tail (or, FP32, before it)
@@ -452,8 +525,10 @@ __global__ void __launch_bounds__((kApWarps + 1) * 32) k_smw_sapply(SApplyArgs<T
                     z[i] = (T)sacc;
                 }
             }
-            const T *xn = a.x + (size_t)cell + (size_t)nw * kTile;
-            T *y = a.y + cell;
+            const T *xn = a.x.at(cell + nw * kTile);
+            const size_t xq = (size_t)a.x.sq;
+            long long yq;
+            T *y = a.y.out(cell, yq);
             // the next tile's x is copied in one group of rows at a time, at
             // the group's last row (all its rows have been read by then): a
             // test of the runtime flag on every row measured about 25 cycles
@@ -468,15 +543,15 @@ __global__ void __launch_bounds__((kApWarps + 1) * 32) k_smw_sapply(SApplyArgs<T
                         if (u == UT - 1 && more) {
 #pragma unroll
                             for (int q = 0; q < UT; ++q)
-                                cp_async_elem(wl + (j - q) * kTile, xn + (size_t)(j - q) * P);
+                                cp_async_elem(wl + (j - q) * kTile, xn + (size_t)(j - q) * xq);
                         }
                     }
                     return val;
                 },
-                [&](int j, T v) { y[(size_t)j * P] = v; });
+                [&](int j, T v) { y[j * yq] = v; });
             if constexpr (!GW) {
                 if (more) {
-                    for (int j = b / UT * UT; j < b; ++j) cp_async_elem(wl + j * kTile, xn + (size_t)j * P);  // ragged last group
+                    for (int j = b / UT * UT; j < b; ++j) cp_async_elem(wl + j * kTile, xn + (size_t)j * xq);  // ragged last group
                     cp_async_commit();
                 }
             }
@@ -489,7 +564,7 @@ fail:
     // the producer waits (bounded) for every copy it issued before it exits;
     // this warp waits (bounded) for its own copies of the first tile's x
     if (lane == 0) atomicExch(a.err, 1);
-    if constexpr (XBULK) mbar_wait_bounded(xbar, 0);
+    if (bulk) mbar_wait_bounded(xbar, 0);
     cp_async_wait<0>();
 }
 
@@ -526,6 +601,8 @@ sts_status smw_build(sts_jac_s *h) {
         M.h_lu_ptr[i + 1] = (int)M.h_lu_idx.size();
     }
     M.nnz_lu = (int)M.h_lu_idx.size();
+    const int sw = struct_band(b, h->dptr, h->didx);
+    M.structured = sw >= 0 && sap_rmax(h->r_diag, sw) > 0 && M.nnz_lu == h->nnz_d;
     M.h_src_slot.assign(h->nnz_d, 0);
     for (int p = 0; p < b; ++p)
         for (int e = h->dptr[p]; e < h->dptr[p + 1]; ++e) M.h_src_slot[e] = slot[(size_t)p * b + h->didx[e]];
@@ -574,55 +651,60 @@ sts_status smw_build(sts_jac_s *h) {
             }
             bptr[r + 1] = (int)bcol.size();
         }
-        M.n_fwd[dir] = (int)fcol.size();
-        M.n_bwd[dir] = (int)bcol.size();
-        // pack tables: stream = forward entries, then per backward row [dinv_i, entries...]
-        std::vector<int> pk_slot, pk_scale;
-        for (size_t e = 0; e < fcol.size(); ++e) {
-            pk_slot.push_back(fslot[e]);
-            pk_scale.push_back(fscale[e]);
-        }
-        for (int r = 0; r < b; ++r) {
-            const int i = b - 1 - r;
-            pk_slot.push_back(-1);
-            pk_scale.push_back(i);
-            for (int e = bptr[r]; e < bptr[r + 1]; ++e) {
-                pk_slot.push_back(bslot[e]);
-                pk_scale.push_back(bscale[e]);
-            }
-        }
         STS_TRY(upload(h, &M.ap_fwd_ptr[dir], fptr));
         STS_TRY(upload(h, &M.ap_fwd_col[dir], fcol));
         STS_TRY(upload(h, &M.ap_fwd_slot[dir], fslot));
         STS_TRY(upload(h, &M.ap_bwd_ptr[dir], bptr));
         STS_TRY(upload(h, &M.ap_bwd_col[dir], bcol));
         STS_TRY(upload(h, &M.ap_bwd_slot[dir], bslot));
-        STS_TRY(upload(h, &M.pk_slot[dir], pk_slot));
-        STS_TRY(upload(h, &M.pk_scale[dir], pk_scale));
-        // apply program, same position order as the pack tables
-        std::vector<unsigned> desc;
+        // apply program of any other pattern (k_smw_apply): columns forward, the pivot
+        // inverses, columns backward, every column's rows dealt to the warps
+        if (M.structured) continue;
+        struct Entry {
+            int row, slot, scale;
+        };
+        std::vector<std::vector<Entry>> fc(b), bc(b);
         for (int i = 0; i < b; ++i)
-            for (int e = fptr[i]; e < fptr[i + 1]; ++e) {
-                unsigned d = (unsigned)fcol[e] | ((unsigned)i << 12);
-                if (e == fptr[i]) d |= kApBegin;
-                if (e == fptr[i + 1] - 1) d |= kApEnd;
-                desc.push_back(d);
+            for (int e = fptr[i]; e < fptr[i + 1]; ++e) fc[fcol[e]].push_back({i, fslot[e], fscale[e]});
+        for (int r = 0; r < b; ++r)
+            for (int e = bptr[r]; e < bptr[r + 1]; ++e) bc[bcol[e]].push_back({b - 1 - r, bslot[e], bscale[e]});
+        std::vector<int> nf(b), nb(b), pk_slot[kGenWarps], pk_scale[kGenWarps];
+        std::vector<short> row[kGenWarps];
+        auto deal = [&](const std::vector<Entry> &col) {
+            const int n = ((int)col.size() + kGenWarps - 1) / kGenWarps;
+            for (int k = 0; k < n * kGenWarps; ++k) {
+                const bool on = k < (int)col.size();
+                row[k % kGenWarps].push_back(on ? (short)col[k].row : (short)-1);
+                pk_slot[k % kGenWarps].push_back(on ? col[k].slot : -2);
+                pk_scale[k % kGenWarps].push_back(on ? col[k].scale : -1);
             }
-        for (int r = 0; r < b; ++r) {
-            const int i = b - 1 - r;
-            desc.push_back(((unsigned)i << 12) | kApScale | (bptr[r + 1] == bptr[r] ? kApEnd : 0u));
-            for (int e = bptr[r]; e < bptr[r + 1]; ++e) {
-                unsigned d = (unsigned)bcol[e] | ((unsigned)i << 12);
-                if (e == bptr[r + 1] - 1) d |= kApEnd;
-                desc.push_back(d);
-            }
+            return n;
+        };
+        for (int j = 0; j < b; ++j) nf[j] = deal(fc[j]);
+        std::vector<Entry> piv(b);
+        for (int i = 0; i < b; ++i) piv[i] = {i, -1, i};
+        deal(piv);
+        for (int j = b - 1; j >= 0; --j) nb[j] = deal(bc[j]);
+        for (int v = 0; v < kGenWarps; ++v) {
+            row[v].insert(row[v].end(), kGenAhead, (short)-1);
+            pk_slot[v].insert(pk_slot[v].end(), kGenAhead, -2);
+            pk_scale[v].insert(pk_scale[v].end(), kGenAhead, -1);
         }
-        if (desc.size() != pk_slot.size()) return set_error(STS_ERR_INVALID_ARG, "internal: apply program size");
-        STS_TRY(upload(h, &M.ap_desc[dir], desc));
+        M.g_wlen[dir] = (int)row[0].size();
+        std::vector<int> all_slot, all_scale;
+        std::vector<short> all_row;
+        for (int v = 0; v < kGenWarps; ++v) {
+            all_slot.insert(all_slot.end(), pk_slot[v].begin(), pk_slot[v].end());
+            all_scale.insert(all_scale.end(), pk_scale[v].begin(), pk_scale[v].end());
+            all_row.insert(all_row.end(), row[v].begin(), row[v].end());
+        }
+        STS_TRY(upload(h, &M.pk_slot[dir], all_slot));
+        STS_TRY(upload(h, &M.pk_scale[dir], all_scale));
+        STS_TRY(upload(h, &M.g_row[dir], all_row));
+        STS_TRY(upload(h, &M.g_nf[dir], nf));
+        STS_TRY(upload(h, &M.g_nb[dir], nb));
     }
     // structured apply tables (both directions; FP64 and, for mixed handles, FP32)
-    const int sw = struct_band(b, h->dptr, h->didx);
-    M.structured = sw >= 0 && sap_rmax(h->r_diag, sw) > 0 && M.nnz_lu == h->nnz_d;
     if (M.structured) {
         const int NF = kStructNF, N = b - NF, r = h->r_diag;
         M.s_w = sw;
@@ -781,7 +863,7 @@ sts_status smw_build(sts_jac_s *h) {
     STS_TRY(dalloc(h, &M.Cinv, (size_t)std::max(r * r, 1) * P));
     for (int dir = 0; dir < 2; ++dir) {
         if (dir == 1 && !h->has_T) continue;
-        const size_t len = M.structured ? (size_t)M.s_lt[0] : (size_t)M.n_fwd[dir] + M.n_bwd[dir] + b;
+        const size_t len = M.structured ? (size_t)M.s_lt[0] : (size_t)kGenWarps * M.g_wlen[dir];
         const size_t len32 = M.structured ? (size_t)M.s_lt[1] : len;
         // the structured streams' zero padding is written here and never again
         STS_TRY(dalloc_zero(h, &M.ap64[dir], len * P));
@@ -796,17 +878,19 @@ sts_status smw_build(sts_jac_s *h) {
 }
 
 template <typename T>
-static sts_status smw_apply_t(sts_jac_s *h, int dir, const T *st, const T *dv, const T *W, const T *x,
-                              T *z) {
+static sts_status smw_apply_t(sts_jac_s *h, int dir, const T *st, const T *dv, const T *W, const Vec<T> &x,
+                              const Vec<T> &z) {
     const SmwPlan &M = h->smw;
     ApplyArgs<T> a;
-    a.st = st; a.desc = M.ap_desc[dir]; a.dv = dv; a.W = W; a.Cinv = M.Cinv; a.x = x; a.y = z;
-    a.len = M.n_fwd[dir] + M.n_bwd[dir] + h->b; a.b = h->b; a.r = h->r_diag; a.ncp = h->ncp; a.trans = dir;
-    const size_t smem = ((size_t)kApStages * kApStage + h->b) * kTile * sizeof(T);
-    auto kern = a.r <= 2 ? k_smw_apply<T, 2> : a.r <= 4 ? k_smw_apply<T, 4> : k_smw_apply<T, kMaxPairsDiag>;
+    a.st = st; a.row = M.g_row[dir]; a.n_fwd = M.g_nf[dir]; a.n_bwd = M.g_nb[dir];
+    a.dv = dv; a.W = W; a.Cinv = M.Cinv; a.x = x; a.y = z;
+    a.wlen = M.g_wlen[dir]; a.b = h->b; a.r = h->r_diag; a.ncp = h->ncp; a.trans = dir;
+    const int rmax = a.r <= 2 ? 2 : a.r <= 4 ? 4 : kMaxPairsDiag;
+    const size_t smem = ((size_t)kGenWarps * std::min(rmax, kGenSum) + h->b) * kTile * sizeof(T);
+    auto kern = rmax == 2 ? k_smw_apply<T, 2> : rmax == 4 ? k_smw_apply<T, 4> : k_smw_apply<T, kMaxPairsDiag>;
     if (smem > 48 * 1024)
         STS_CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    kern<<<h->n_tiles, kTile, smem, h->stream>>>(a);
+    kern<<<h->n_tiles, kGenWarps * kTile, smem, h->stream>>>(a);
     STS_LAUNCHED();
     return STS_OK;
 }
@@ -821,8 +905,13 @@ static void (*sap_kernel(int rmax, bool gw))(SApplyArgs<T>) {
     return gw ? sap_kernel_gw<T, W, true>(rmax) : sap_kernel_gw<T, W, false>(rmax);
 }
 
+// The working vector moves to y where b rows per warp would leave fewer than kApWarps
+// consumers per SM.
+static bool sap_in_y(int b, int elem) { return (size_t)(227 * 1024) / sap_warp_bytes(b, elem) < (size_t)kApWarps; }
+bool smw_apply_any_layout(const sts_jac_s *h, int elem) { return !h->smw.structured || !sap_in_y(h->b, elem); }
+
 template <typename T>
-static sts_status smw_sapply_t(sts_jac_s *h, int dir, const T *st, const T *x, T *z) {
+static sts_status smw_sapply_t(sts_jac_s *h, int dir, const T *st, const Vec<T> &x, const Vec<T> &z) {
     const SmwPlan &M = h->smw;
     SApplyArgs<T> a;
     a.st = st; a.Cinv = M.Cinv; a.x = x; a.y = z; a.err = h->d_err;
@@ -830,9 +919,8 @@ static sts_status smw_sapply_t(sts_jac_s *h, int dir, const T *st, const T *x, T
     a.trans = dir; a.n_tiles = h->n_tiles;
     a.pre = h->streams_dirty ? 0 : 1;
     a.evict_first = (double)a.n_tiles * a.Lt * kTile * sizeof(T) > (double)h->l2_bytes ? 1 : 0;
-    // the working vector moves to y where b rows per warp would leave fewer
-    // than kApWarps consumers per SM
-    const bool gw = (size_t)(227 * 1024) / sap_warp_bytes(h->b, (int)sizeof(T)) < (size_t)kApWarps;
+    const bool gw = sap_in_y(h->b, (int)sizeof(T));
+    a.bulk = x.sc == 1 && x.cells == h->ncp && reinterpret_cast<uintptr_t>(x.p) % 16 == 0 ? 1 : 0;
     const size_t per_warp = sap_warp_bytes(gw ? 0 : h->b, (int)sizeof(T));
     const int wpb = (int)std::min<size_t>(kApWarps, (size_t)(227 * 1024) / per_warp);
     if (wpb < 1)
@@ -858,13 +946,13 @@ static sts_status smw_sapply_t(sts_jac_s *h, int dir, const T *st, const T *x, T
     return STS_OK;
 }
 
-sts_status smw_apply64(sts_jac_s *h, int dir, const double *x, double *z) {
+sts_status smw_apply64(sts_jac_s *h, int dir, const Vec<double> &x, const Vec<double> &z) {
     const SmwPlan &M = h->smw;
     if (M.structured) return smw_sapply_t<double>(h, dir, M.ap64[dir], x, z);
     return smw_apply_t<double>(h, dir, M.ap64[dir], dir == 0 ? M.Vd : M.Ud, dir == 0 ? M.W : M.Wt, x, z);
 }
 
-sts_status smw_apply32(sts_jac_s *h, int dir, const float *x, float *z) {
+sts_status smw_apply32(sts_jac_s *h, int dir, const Vec<float> &x, const Vec<float> &z) {
     const SmwPlan &M = h->smw;
     if (M.structured) return smw_sapply_t<float>(h, dir, M.ap32[dir], x, z);
     return smw_apply_t<float>(h, dir, M.ap32[dir], M.DV32[dir], M.W32[dir], x, z);

@@ -603,9 +603,8 @@ __global__ void __launch_bounds__(kTile) k_smw_cinv_sh(SetupArgs a) {
     if (!ok) atomicMin(a.err_cell, cell);
 }
 
-// Write the apply streams: forward coefficients, then per backward row its
-// pivot inverse followed by its coefficients (scaled by the row's dinv where the
-// program asks for it).
+// Write the general apply's streams from the packing tables (SmwPlan); the zeros of the
+// padding were written when they were allocated.
 template <typename T>
 __global__ void k_smw_pack(T *out, const double *lu, const double *dinv, const int *pk_slot,
                            const int *pk_scale, int len, int ncp) {
@@ -615,6 +614,7 @@ __global__ void k_smw_pack(T *out, const double *lu, const double *dinv, const i
         const int cell = (int)(i % ncp), pos = (int)(i / ncp);
         const int sl = pk_slot[pos], sc = pk_scale[pos];
         double v;
+        if (sl < -1) continue;
         if (sl >= 0) {
             v = lu[(size_t)sl * ncp + cell];
             if (sc >= 0) v *= dinv[(size_t)sc * ncp + cell];
@@ -824,7 +824,7 @@ sts_status smw_setup(sts_jac_s *h) {
             }
             continue;
         }
-        const int len = M.n_fwd[dir] + M.n_bwd[dir] + b;
+        const int len = kGenWarps * M.g_wlen[dir];
         const long long n = (long long)len * P;
         k_smw_pack<double><<<grid_for(n, 256), 256, 0, h->stream>>>(M.ap64[dir], M.lu, M.dinv, M.pk_slot[dir],
                                                                      M.pk_scale[dir], len, h->ncp);

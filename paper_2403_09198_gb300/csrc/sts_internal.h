@@ -47,14 +47,7 @@ constexpr int kStructMaxW = 4;
 constexpr int kStructMaxSlots = 5;
 constexpr unsigned kDescEnd = 1u << 31;
 
-// SMW apply program descriptor (one per stream position):
-//   bits 0-11 column j, bits 12-23 row i
-//   kApBegin  acc = w_i before this entry (first forward entry of row i)
-//   kApScale  acc = value * w_i (the pivot inverse opening backward row i)
-//   kApEnd    w_i = acc after this position
-constexpr unsigned kApBegin = 1u << 28;
-constexpr unsigned kApScale = 1u << 29;
-constexpr unsigned kApEnd = 1u << 31;
+constexpr int kGenWarps = 4;       // warps per tile of the general block-Jacobi apply
 
 sts_status set_error(sts_status s, const char *fmt, ...);
 
@@ -111,6 +104,24 @@ inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, siz
         if (s_ != STS_OK) return s_;     \
     } while (0)
 
+// Where the kernels find component q of cell c of a vector: p[c * sc + q * sq].  The
+// internal layout is (1, ncp) over ncp cells; a public vector may be read and written in
+// place (see with_layout), over its nc cells only: `junk` takes the results of the
+// padding lanes then, and reads of a padding lane go to the last cell.
+template <typename T>
+struct Vec {
+    T *p;
+    long long sc, sq;
+    int cells;
+    T *junk;
+    __device__ __forceinline__ T *at(int c) const { return p + (long long)min(c, cells - 1) * sc; }
+    // for writing: the cell's first component and the step to the next one
+    __device__ __forceinline__ T *out(int c, long long &step) const {
+        step = c < cells ? sq : 0;
+        return c < cells ? p + (long long)c * sc : junk + (c & (kTile - 1));
+    }
+};
+
 // Device allocation tracked by the handle.
 struct DevBuf {
     void *p = nullptr;
@@ -132,16 +143,13 @@ struct MvPlan {
     int n_slots = 0, n_pslots = 0, n_groups = 0;
     int n_dtasks = 0, Lp = 0;                // pass-1 dot tasks per tile, padded dot length
     long long tile_len = 0;                  // main-stream elements per lane per tile
-    std::vector<int> h_grp_rows;             // [n_groups+1]
-    std::vector<long long> h_row_off;        // [b+1] start of row p in the tile stream
     std::vector<int> h_pslot_slot;           // [n_pslots]
     std::vector<int> h_blk;                  // host copy of blk
     // device copies
     int *nbr = nullptr;                      // [n_tiles][n_slots][32]: input cell or -1
     int *blk = nullptr;                      // [n_tiles][n_slots][32]: public block id or -1
     unsigned *slot_mask = nullptr;           // [n_tiles]: bit s set if any lane has slot s
-    int *grp_rows = nullptr;                 // [n_groups+1]
-    long long *row_off = nullptr;            // [b+1]
+    int4 *grp = nullptr;                     // [n_groups] generic pass 2: first row, positions, first position (two words)
     int *pat_ptr = nullptr;                  // [2][b+1] pattern rows (kind 0 diag, 1 off), this direction
     int *pat_idx = nullptr;                  // [nnz_d + nnz_o] column indices (kind 1 after kind 0)
     int *dtask_slot = nullptr;               // [n_dtasks]: block slot whose x a dot task reads
@@ -185,11 +193,14 @@ struct SmwPlan {
     int *ap_fwd_ptr[2] = {nullptr, nullptr}, *ap_fwd_col[2] = {nullptr, nullptr};
     int *ap_bwd_ptr[2] = {nullptr, nullptr}, *ap_bwd_col[2] = {nullptr, nullptr};
     int *ap_fwd_slot[2] = {nullptr, nullptr}, *ap_bwd_slot[2] = {nullptr, nullptr};
-    // Stream packing per direction, one entry per stream position: LU slot (or
-    // -1 for a pivot inverse) and the row whose pivot inverse scales it (-1: none).
+    // General apply per direction (see k_smw_apply): coefficients of the kGenWarps warps one
+    // after another, g_wlen each; the row each one updates (-1: padding), the
+    // coefficients per warp of every column; and for packing the LU slot (-1: a pivot
+    // inverse, -2: padding) and the row whose pivot inverse it is or is scaled by (-1: none).
+    int g_wlen[2] = {0, 0};
+    short *g_row[2] = {nullptr, nullptr};
+    int *g_nf[2] = {nullptr, nullptr}, *g_nb[2] = {nullptr, nullptr};
     int *pk_slot[2] = {nullptr, nullptr}, *pk_scale[2] = {nullptr, nullptr};
-    unsigned *ap_desc[2] = {nullptr, nullptr};   // apply program (see kApBegin)
-    int n_fwd[2] = {0, 0}, n_bwd[2] = {0, 0};
     // per-cell data
     double *Sd = nullptr;        // [nnz_d][ncp] diagonal-block S values
     double *Ud = nullptr;        // [r][b][ncp]
@@ -199,7 +210,7 @@ struct SmwPlan {
     double *W = nullptr;         // [r][b][ncp]   S^-1 U
     double *Wt = nullptr;        // [r][b][ncp]   S^-T V
     double *Cinv = nullptr;      // [r][r][ncp]   (I + V^T S^-1 U)^-1
-    double *ap64[2] = {nullptr, nullptr};   // [n_fwd+n_bwd+b][ncp] apply streams
+    double *ap64[2] = {nullptr, nullptr};   // apply streams ([kGenWarps * g_wlen][ncp], or structured)
     float *ap32[2] = {nullptr, nullptr};
     float *W32[2] = {nullptr, nullptr};     // W, Wt rounded
     float *DV32[2] = {nullptr, nullptr};    // Vd, Ud rounded (dot vectors of the two directions)
@@ -336,10 +347,14 @@ sts_status values_plan(sts_jac_s *h, MvPlan &P, const std::vector<int> &pk, cons
 sts_status values_load(sts_jac_s *h, int dir, const double *S, const double *U, const double *V);
 
 // kernels_matvec.cu
-sts_status mv_apply64(sts_jac_s *h, int dir, const double *x, double *y, double *c);
-sts_status mv_apply32(sts_jac_s *h, int dir, const float *x, float *y, float *c);
+template <typename T>
+Vec<T> internal_vec(const sts_jac_s *h, const T *p) {
+    return Vec<T>{const_cast<T *>(p), 1, h->ncp, h->ncp, nullptr};
+}
+sts_status mv_apply64(sts_jac_s *h, int dir, const Vec<double> &x, const Vec<double> &y, double *c);
+sts_status mv_apply32(sts_jac_s *h, int dir, const Vec<float> &x, const Vec<float> &y, float *c);
 sts_status mv_dots64(sts_jac_s *h, int dir, const double *x, double *c);   // pass 1 only
-sts_status mv_apply64_noalloc(sts_jac_s *h, int dir, const double *x, double *y);
+sts_status mv_apply64_noalloc(sts_jac_s *h, int dir, const Vec<double> &x, const Vec<double> &y);
 sts_status to_internal64(sts_jac_s *h, const double *x, double *xi);
 sts_status from_internal64(sts_jac_s *h, const double *xi, double *x);
 sts_status to_internal32(sts_jac_s *h, const float *x, float *xi);
@@ -349,8 +364,9 @@ sts_status from_internal32(sts_jac_s *h, const float *xi, float *x);
 sts_status smw_build(sts_jac_s *h);                       // host schedule + device tables
 sts_status smw_setup(sts_jac_s *h);
 sts_status check_device(sts_jac_s *h);                   // STS_ERR_TIMEOUT if a bounded device wait gave up
-sts_status smw_apply64(sts_jac_s *h, int dir, const double *x, double *z);
-sts_status smw_apply32(sts_jac_s *h, int dir, const float *x, float *z);
+sts_status smw_apply64(sts_jac_s *h, int dir, const Vec<double> &x, const Vec<double> &z);
+sts_status smw_apply32(sts_jac_s *h, int dir, const Vec<float> &x, const Vec<float> &z);
+bool smw_apply_any_layout(const sts_jac_s *h, int elem);     // whether the apply takes any Vec, not the internal layout only
 
 // kernels_dense.cu
 sts_status dense_build(sts_jac_s *h, const double *S, const double *U, const double *V);
