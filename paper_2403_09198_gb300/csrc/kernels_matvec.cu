@@ -78,7 +78,9 @@ template <> struct DotVec<float> {
 __device__ __forceinline__ double dot_el(double v, int) { return v; }
 __device__ __forceinline__ float dot_el(const float4 &v, int i) { return vel(v, i); }
 
-template <typename T>
+// INT: x is in the internal layout, the common case: its addresses then cost a warp,
+// whose 63 FMAs at N = 60 are soon done, about 1% less.
+template <typename T, bool INT>
 __global__ void __launch_bounds__(128) k_dots(MvArgs<T> a) {
     using V = typename DotVec<T>::type;
     constexpr int CH = Chunk<T>::CH;
@@ -105,9 +107,9 @@ __global__ void __launch_bounds__(128) k_dots(MvArgs<T> a) {
     T acc = T(0);
     if (present) {
         // an absent neighbour reads the lane's own cell: its coefficients are zero
-        const T *__restrict__ xj = a.x.at(j >= 0 ? j : t * kTile + lane);
+        const T *__restrict__ xj = a.x.template cell<INT>(j >= 0 ? j : t * kTile + lane);
         const int bm1 = a.b - 1;
-        const size_t sq = (size_t)a.x.sq;
+        const size_t sq = INT ? (size_t)a.ncp : (size_t)a.x.sq;
         if (!a.pre) {
 #pragma unroll
             for (int i = 0; i < NV; ++i) va[i] = __ldcs(dv + i * kTile);
@@ -249,7 +251,7 @@ __host__ __device__ inline size_t mv_struct_warp_bytes(int rl, int elem) {
     return 128 + 2 * (size_t)rl * kTile * elem;     // two mbarriers (padded), two row stages
 }
 
-template <typename T, int WD, int NREG>
+template <typename T, int WD, int NREG, bool INT>
 __global__ void __launch_bounds__(64) k_mv_struct(MvArgs<T> a) {
     static_assert(NREG == 0 || NREG == 8 || NREG == 2 * kStructDuff, "register pair slots");
     constexpr int NF = kStructNF;
@@ -257,7 +259,7 @@ __global__ void __launch_bounds__(64) k_mv_struct(MvArgs<T> a) {
     constexpr int BANDW = 2 * WD + 1;
     const int lane = threadIdx.x & 31;
     const int ns = a.n_slots, nps = a.n_pslots, N = a.sN;
-    const size_t sq = (size_t)a.x.sq;
+    const size_t sq = INT ? (size_t)a.ncp : (size_t)a.x.sq;
     const int RL = a.s_rl;
     const uint32_t row_bytes = (uint32_t)RL * kTile * (uint32_t)sizeof(T);
     extern __shared__ __align__(128) unsigned char mv_smem[];
@@ -303,8 +305,6 @@ __global__ void __launch_bounds__(64) k_mv_struct(MvArgs<T> a) {
     if (lane == 0) ticket = atomicAdd(a.sched, 1u);
     const int t = (int)(wid / a.n_groups), g = (int)(wid % a.n_groups);
     const int cell = t * kTile + lane;
-    long long ystep;
-    T *const ycell = a.y.out(cell, ystep);
     const T *__restrict__ cc = a.c + (size_t)t * a.n_dtasks * kTile + lane;
     if (g == a.n_lgroups) {
         const T *__restrict__ su = a.main + ((size_t)t * a.tile_len + (size_t)N * RL) * kTile + lane;
@@ -314,7 +314,7 @@ __global__ void __launch_bounds__(64) k_mv_struct(MvArgs<T> a) {
             for (int s = 0; s < ns; ++s) acc += __ldg(cc + (size_t)(nps + f * ns + s) * kTile);
             for (int k = 0; k < nps; ++k)
                 acc = fma(__ldg(su + (size_t)(f * nps + k) * kTile), __ldg(cc + (size_t)k * kTile), acc);
-            ycell[(N + f) * ystep] = acc;
+            if (INT || cell < a.y.cells) a.y.template cell<INT>(cell)[(size_t)(N + f) * sq] = acc;
         }
         continue;
     }
@@ -339,7 +339,7 @@ __global__ void __launch_bounds__(64) k_mv_struct(MvArgs<T> a) {
     for (int s = 0; s < NS; ++s) {
         const int j = s < ns ? a.nbr[((size_t)t * ns + s) * kTile + lane] : -1;
         // an absent neighbour reads the lane's own cell: its coefficients are zero
-        xs[s] = a.x.at(j >= 0 ? j : cell);
+        xs[s] = a.x.template cell<INT>(j >= 0 ? j : cell);
 #pragma unroll
         for (int f = 0; f < NF; ++f) xf[s][f] = s < ns ? __ldg(xs[s] + (size_t)(N + f) * sq) : T(0);
     }
@@ -362,7 +362,8 @@ __global__ void __launch_bounds__(64) k_mv_struct(MvArgs<T> a) {
     T xn[NS];
 #pragma unroll
     for (int s = 1; s < NS; ++s) xn[s] = s < ns ? __ldg(xs[s] + (size_t)p0 * sq) : T(0);
-    T *yp = ycell + p0 * ystep;
+    T *yp = a.y.template cell<INT>(cell) + (size_t)p0 * sq;      // y has x's strides
+    const bool on = INT || cell < a.y.cells;
     T ylag = T(0);          // row p-1's result, stored during row p (its FMA has long completed)
     for (int p = p0; p < p1; ++p) {
         const int sg = (p - p0) & 1;
@@ -448,14 +449,14 @@ __global__ void __launch_bounds__(64) k_mv_struct(MvArgs<T> a) {
             for (int k = 0; k < nps; ++k) acc = fma(vu[k * kTile], __ldg(cc + (size_t)k * kTile), acc);
         }
         if (p > p0) {
-            *yp = ylag;
-            yp += ystep;
+            if (on) *yp = ylag;
+            yp += sq;
         }
         ylag = acc;
         __syncwarp();     // every lane is done with the stage before it is refilled
         if (p + 2 < p1) issue(p + 2);
     }
-    if (p1 > p0) *yp = ylag;
+    if (on && p1 > p0) *yp = ylag;
     }
 done:
     // The last warp to finish resets the counters for the next launch.  A
@@ -573,15 +574,21 @@ template <typename T>
 sts_status dots_launch(sts_jac_s *h, const MvArgs<T> &a) {
     if (a.n_dtasks == 0) return STS_OK;
     const long long warps = (long long)a.n_tiles * a.n_dtasks;
-    k_dots<T><<<(unsigned)((warps + 3) / 4), 128, 0, h->stream>>>(a);
+    const auto kern = a.x.internal(a.ncp) ? k_dots<T, true> : k_dots<T, false>;
+    kern<<<(unsigned)((warps + 3) / 4), 128, 0, h->stream>>>(a);
     STS_LAUNCHED();
     h->streams_dirty = false;
     return STS_OK;
 }
 
+template <typename T, int WD, bool INT>
+void (*mv_struct_kernel_of(int nreg))(MvArgs<T>) {
+    return nreg == 8 ? k_mv_struct<T, WD, 8, INT> : nreg ? k_mv_struct<T, WD, 2 * kStructDuff, INT>
+                                                          : k_mv_struct<T, WD, 0, INT>;
+}
 template <typename T, int WD>
-void (*mv_struct_kernel(int nreg))(MvArgs<T>) {
-    return nreg == 8 ? k_mv_struct<T, WD, 8> : nreg ? k_mv_struct<T, WD, 2 * kStructDuff> : k_mv_struct<T, WD, 0>;
+void (*mv_struct_kernel(int nreg, bool internal))(MvArgs<T>) {
+    return internal ? mv_struct_kernel_of<T, WD, true>(nreg) : mv_struct_kernel_of<T, WD, false>(nreg);
 }
 
 // Level rows per pass-2 item.  The persistent grid runs n_tiles x (groups + 1)
@@ -617,12 +624,13 @@ sts_status mv_launch(sts_jac_s *h, const MvArgs<T> &args) {
         const size_t smem = (size_t)kWarpsPerBlock * mv_struct_warp_bytes(a.s_rl, (int)sizeof(T));
         void (*kern)(MvArgs<T>) = nullptr;
         const int nreg = a.n_pslots <= 8 ? 8 : a.n_pslots <= 2 * kStructDuff ? 2 * kStructDuff : 0;
+        const bool in = a.x.internal(a.ncp);
         switch (a.wd) {
-            case 0: kern = mv_struct_kernel<T, 0>(nreg); break;
-            case 1: kern = mv_struct_kernel<T, 1>(nreg); break;
-            case 2: kern = mv_struct_kernel<T, 2>(nreg); break;
-            case 3: kern = mv_struct_kernel<T, 3>(nreg); break;
-            default: kern = mv_struct_kernel<T, 4>(nreg); break;
+            case 0: kern = mv_struct_kernel<T, 0>(nreg, in); break;
+            case 1: kern = mv_struct_kernel<T, 1>(nreg, in); break;
+            case 2: kern = mv_struct_kernel<T, 2>(nreg, in); break;
+            case 3: kern = mv_struct_kernel<T, 3>(nreg, in); break;
+            default: kern = mv_struct_kernel<T, 4>(nreg, in); break;
         }
         // blocks resident at once, found once per kernel instance and shared-memory
         // size: the instance (pair slots) and the row length differ between the
@@ -662,9 +670,9 @@ sts_status mv_apply64(sts_jac_s *h, int dir, const Vec<double> &x, const Vec<dou
     return mv_launch<double>(h, make_args<double>(h, dir, P.main64, P.dotv64, x, y, c));
 }
 
-sts_status mv_dots64(sts_jac_s *h, int dir, const double *x, double *c) {
+sts_status mv_dots64(sts_jac_s *h, int dir, const Vec<double> &x, double *c) {
     const MvPlan &P = h->mv[dir];
-    return dots_launch<double>(h, make_args<double>(h, dir, P.main64, P.dotv64, internal_vec(h, x), Vec<double>{}, c));
+    return dots_launch<double>(h, make_args<double>(h, dir, P.main64, P.dotv64, x, Vec<double>{}, c));
 }
 
 // ---------------------------------------------------------------------------
@@ -748,6 +756,14 @@ static sts_status from_internal(sts_jac_s *h, const T *xi, T *x) {
         k_comp_unpad<T><<<grid_for(n, 256), 256, 0, h->stream>>>(xi, x, h->nc, h->b, h->ncp);
         STS_LAUNCHED();
     }
+    return STS_OK;
+}
+
+// component-major [b][nc] to cell-major
+sts_status comp_to_cell64(sts_jac_s *h, const double *x, double *xc) {
+    k_comp_to_cell<double><<<dim3((h->nc + 31) / 32, (h->b + 31) / 32), dim3(32, 8), 0, h->stream>>>(x, xc, h->nc, h->b,
+                                                                                                    h->nc);
+    STS_LAUNCHED();
     return STS_OK;
 }
 

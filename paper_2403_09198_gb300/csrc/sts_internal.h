@@ -115,6 +115,10 @@ struct Vec {
     int cells;
     T *junk;
     __device__ __forceinline__ T *at(int c) const { return p + (long long)min(c, cells - 1) * sc; }
+    // the same; INT: the layout is known to be the internal one
+    template <bool INT>
+    __device__ __forceinline__ T *cell(int c) const { return INT ? p + c : at(c); }
+    bool internal(int ncp) const { return sc == 1 && sq == ncp && cells == ncp; }
     // for writing: the cell's first component and the step to the next one
     __device__ __forceinline__ T *out(int c, long long &step) const {
         step = c < cells ? sq : 0;
@@ -353,8 +357,9 @@ Vec<T> internal_vec(const sts_jac_s *h, const T *p) {
 }
 sts_status mv_apply64(sts_jac_s *h, int dir, const Vec<double> &x, const Vec<double> &y, double *c);
 sts_status mv_apply32(sts_jac_s *h, int dir, const Vec<float> &x, const Vec<float> &y, float *c);
-sts_status mv_dots64(sts_jac_s *h, int dir, const double *x, double *c);   // pass 1 only
+sts_status mv_dots64(sts_jac_s *h, int dir, const Vec<double> &x, double *c);   // pass 1 only
 sts_status mv_apply64_noalloc(sts_jac_s *h, int dir, const Vec<double> &x, const Vec<double> &y);
+sts_status comp_to_cell64(sts_jac_s *h, const double *x, double *xc);
 sts_status to_internal64(sts_jac_s *h, const double *x, double *xi);
 sts_status from_internal64(sts_jac_s *h, const double *xi, double *x);
 sts_status to_internal32(sts_jac_s *h, const float *x, float *xi);
