@@ -764,8 +764,10 @@ sts_status sts_gmres_solve(sts_jac_t h, const double *b, double *x, const sts_gm
                            sts_gmres_info *info) {
     NvtxRange nvtx_range("sts_gmres_solve");
     STS_TRY(check_handle(h, b, x, "sts_gmres_solve"));
-    STS_GUARD(const sts_status st = gmres(h, b, x, opts, info);
-              if (st == STS_OK || st == STS_ERR_NOT_CONVERGED || st == STS_ERR_NUMERIC) STS_TRY(check_device(h));
+    STS_GUARD(bool checked = false;
+              const sts_status st = gmres(h, b, x, opts, info, &checked);
+              if (!checked && (st == STS_OK || st == STS_ERR_NOT_CONVERGED || st == STS_ERR_NUMERIC))
+                  STS_TRY(check_device(h));
               return st;)
 }
 

@@ -251,19 +251,23 @@ struct Krylov {
     double *w = nullptr, *r = nullptr, *xb = nullptr, *bb = nullptr, *tmp = nullptr;  // [n]
     double *partial = nullptr;   // [kRedBlocks][m+2]
     double *red = nullptr;       // [3][m+2] reduced dots and norms
-    unsigned int *ticket = nullptr;   // finished-block counter of the last-block reductions (0 between launches)
+    unsigned int *ticket = nullptr;   // [2] finished-block counters of the last-block reductions (0 between launches)
     double *h_pinned = nullptr;  // host pinned [m+2]
     double *c = nullptr;         // pair dots scratch [n_tiles*n_pslots*32]
     float *c32 = nullptr;
     // A cycle's Arnoldi steps as one CUDA graph (sts_gmres_opts.arnoldi): the
     // Givens state lives on the device, sized for m
-    double *gH = nullptr;        // [(m+1) * m] Hessenberg matrix, rotated in place
-    double *gcs = nullptr, *gsn = nullptr;   // [m] rotations
-    double *gg = nullptr;        // [m+1] rotated right-hand side
-    double *ghist = nullptr;     // [m] rotated residual / ||b|| per step
+    double *gbuf = nullptr;      // holds the following
     double *gpar = nullptr;      // [4] stop threshold, history scale, 1 / h(j+1,j), steps allowed
     int *gstate = nullptr;       // [2] steps taken, stop reason (1 criterion met, 2 NaN or Inf)
-    double *g_pinned = nullptr;  // host pinned copy of the above
+    double *grn = nullptr;       // squared norm of the residual after the cycle
+    int *gerr = nullptr;         // the handle's error flag after the cycle
+    double *gg = nullptr;        // [m+1] rotated right-hand side
+    double *ghist = nullptr;     // [m] rotated residual / ||b|| per step
+    double *gH = nullptr;        // [(m+1) * m] Hessenberg matrix, rotated in place
+    double *gcs = nullptr, *gsn = nullptr;   // [m] rotations
+    double *gy = nullptr;        // [m] coefficients of the correction
+    double *g_pinned = nullptr;  // host pinned copy of gbuf up to ghist
     cudaGraphExec_t gexec[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};   // [direction][preconditioned]
     int g_m[2][2] = {{0, 0}, {0, 0}};
     cudaStream_t g_stream[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};
@@ -293,7 +297,7 @@ struct sts_jac_s {
         int blocks;
     };
     std::vector<Resident> mvs_resident;
-    bool sap_attr[2] = {false, false};  // shared-memory limit of the structured apply set
+    bool sap_attr[2][2] = {{false, false}, {false, false}};  // shared-memory limit of the structured apply set [precision][internal layout]
     // host copies of the structure
     std::vector<int> bptr, bidx, dptr, didx, optr, oidx;
     std::vector<long long> soff;    // [nnzb+1]
@@ -371,6 +375,7 @@ sts_status smw_setup(sts_jac_s *h);
 sts_status check_device(sts_jac_s *h);                   // STS_ERR_TIMEOUT if a bounded device wait gave up
 sts_status smw_apply64(sts_jac_s *h, int dir, const Vec<double> &x, const Vec<double> &z);
 sts_status smw_apply32(sts_jac_s *h, int dir, const Vec<float> &x, const Vec<float> &z);
+sts_status smw_sapply32(sts_jac_s *h, int dir, const Vec<float> &x, const Vec<float> &z);     // kernels_smw32.cu
 bool smw_apply_any_layout(const sts_jac_s *h, int elem);     // whether the apply takes any Vec, not the internal layout only
 
 // kernels_dense.cu
@@ -382,7 +387,8 @@ sts_status dense_apply(sts_jac_s *h, const double *x, double *z);
 // kernels_krylov.cu
 sts_status op_matvec64(sts_jac_s *h, int dir, const double *x, double *y);
 sts_status op_apply64(sts_jac_s *h, int dir, const double *x, double *z);
-sts_status gmres(sts_jac_s *h, const double *b, double *x, const sts_gmres_opts *o, sts_gmres_info *info);
+sts_status gmres(sts_jac_s *h, const double *b, double *x, const sts_gmres_opts *o, sts_gmres_info *info,
+                 bool *checked);
 sts_status kry_reserve(sts_jac_s *h, int m);
 sts_status kry_dots(sts_jac_s *h, const double *V, int k, const double *w, int self, double *out_dev);
 sts_status kry_update(sts_jac_s *h, double *w, const double *V, int k, const double *hcoef_dev, int norm,
