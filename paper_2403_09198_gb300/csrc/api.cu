@@ -553,7 +553,7 @@ sts_status create_impl(const sts_jac_desc *d, sts_jac_t *out) {
         const size_t n = (size_t)b * h->ncp;
         if ((st = dalloc(h, &h->vin, n)) != STS_OK) break;
         if ((st = dalloc(h, &h->vout, n)) != STS_OK) break;
-        if ((st = dalloc(h, &h->d_err, 1)) != STS_OK) break;
+        if ((st = dalloc(h, &h->d_err, 2)) != STS_OK) break;
         if ((st = dalloc(h, &h->d_sched, 2)) != STS_OK) break;
         if (cudaMemsetAsync(h->d_sched, 0, 2 * sizeof(unsigned), h->stream) != cudaSuccess ||
             cudaMemsetAsync(h->d_err, 0, sizeof(int), h->stream) != cudaSuccess) {
@@ -646,6 +646,11 @@ sts_status check_device(sts_jac_s *h) {
     int flag = 0;
     STS_CK(cudaMemcpyAsync(&flag, h->d_err, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
     STS_CK(cudaStreamSynchronize(h->stream));
+    return report_wait(h, flag);
+}
+
+// The same with the flag's value in hand.
+sts_status report_wait(sts_jac_s *h, int flag) {
     if (!flag) return STS_OK;
     STS_CK(cudaMemsetAsync(h->d_err, 0, sizeof(int), h->stream));
     if (h->d_sched) STS_CK(cudaMemsetAsync(h->d_sched, 0, 2 * sizeof(unsigned), h->stream));
@@ -728,8 +733,9 @@ sts_status sts_jac_matvec_f32(sts_jac_t h, const float *x, float *y, int trans) 
 sts_status sts_jac_bjacobi_setup(sts_jac_t h) {
     NvtxRange nvtx_range("sts_jac_bjacobi_setup");
     if (!h) return set_error(STS_ERR_INVALID_ARG, "sts_jac_bjacobi_setup: handle is NULL");
-    STS_GUARD(STS_TRY(check_device(h));
-              return h->rep == STS_REP_FACTORED ? smw_setup(h) : dense_setup(h);)
+    STS_GUARD(if (h->rep == STS_REP_FACTORED) return smw_setup(h);      // checks the device with its own flag
+              STS_TRY(check_device(h));
+              return dense_setup(h);)
 }
 
 sts_status sts_jac_bjacobi_apply(sts_jac_t h, const double *x, double *z, int trans) {

@@ -18,7 +18,7 @@
 //
 // Measured on 128 x 128 cells, N = 60 (band 2): Jacobian (571 MB written) 1326 us with the
 // scalars formed by every warp and every entry on its own, now 27 + 28 + 238 us (scalars
-// of cells, of faces, entries); residual 540 us, now 33 + 12 + 47.  The entries keep the
+// of cells, of faces, entries); residual 540 us, now 26 + 12 + 47.  The entries keep the
 // FP64 pipe 63% busy (134 of the 238 us are pipe time); more warps per SM or four faces
 // at once without branches between them left the time as it was.
 #include <cuda_runtime.h>
@@ -26,6 +26,7 @@
 #include <algorithm>
 #include <cmath>
 #include <new>
+#include <type_traits>
 #include <vector>
 
 #include "sts_internal.h"
@@ -100,17 +101,23 @@ __global__ void __launch_bounds__(128) k_flow_mix(FlowDev F, const double *Q, co
     __syncthreads();
     const double *q = rows + min(lane, n - 1) * st;
     double s[4][5] = {};
-    for (int k = warp; k < N; k += 16) {
+    // Qn gives the conserved variables only: its sums of r and beta are left out
+    auto sums = [&](auto all) {
+        for (int k = warp; k < N; k += 16) {
 #pragma unroll
-        for (int h = 0; h < 4; ++h) {
-            const int kk = k + 4 * h;
-            if (kk >= N) break;
-            const double x = q[kk];
-            s[h][0] += x;
+            for (int h = 0; h < 4; ++h) {
+                const int kk = k + 4 * h;
+                if (kk >= N) break;
+                const double x = q[kk];
+                s[h][0] += x;
 #pragma unroll
-            for (int j = 0; j < 4; ++j) s[h][j + 1] = fma(x, cst[4 * kk + j], s[h][j + 1]);
+                for (int j = 0; j < 4; ++j)
+                    if (decltype(all)::value || j == 1 || j == 2) s[h][j + 1] = fma(x, cst[4 * kk + j], s[h][j + 1]);
+            }
         }
-    }
+    };
+    if (blockIdx.y) sums(std::false_type{});
+    else sums(std::true_type{});
 #pragma unroll
     for (int j = 0; j < 5; ++j) part[warp][j][lane] = (s[0][j] + s[1][j]) + (s[2][j] + s[3][j]);
     __syncthreads();
@@ -120,11 +127,10 @@ __global__ void __launch_bounds__(128) k_flow_mix(FlowDev F, const double *Q, co
     double *M = F.mix + (size_t)blockIdx.y * kMixFields * F.nc + c0 + lane;
     const size_t P = F.nc;
     // the scalars' dependent chains on a warp each
-    if (warp == 0) {
+    if (warp == 0 && blockIdx.y == 0) {
         const double rho = total(0), R = total(1), C = total(2);
         const double g = (C + R) * R / (rho * C), a = sqrt(g * T);
         M[mA * P] = a;
-        if (blockIdx.y) return;                  // Qn gives the conserved variables only
         const double cga = T / (2.0 * a * rho * C);
         M[mG0 * P] = -cga * ((C + R) * R / rho);
         M[mG1 * P] = -cga * (R * R / C);
@@ -142,7 +148,7 @@ __global__ void __launch_bounds__(128) k_flow_mix(FlowDev F, const double *Q, co
         M[mKe * P] = ke;
         M[mP * P] = R * T;
         M[mE * P] = total(3) + C * T + rho * ke;
-    } else if (warp == 2) {
+    } else if (warp == 2 && blockIdx.y == 0) {
         M[mKap * P] = F.A * exp(-F.theta / T);
         M[mSb * P] = total(4);
     }

@@ -483,7 +483,7 @@ sts_status smw_build(sts_jac_s *h) {
             STS_TRY(dalloc(h, &M.DV32[dir], (size_t)std::max(r, 1) * b * P));
         }
     }
-    STS_TRY(dalloc(h, &M.err_cell, 1));
+    M.err_cell = h->d_err + 1;
     return STS_OK;
 }
 

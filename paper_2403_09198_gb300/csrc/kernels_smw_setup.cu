@@ -10,7 +10,6 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
-#include <climits>
 #include <cmath>
 #include <type_traits>
 
@@ -750,8 +749,8 @@ sts_status smw_setup(sts_jac_s *h) {
     a.err_cell = M.err_cell;
     a.nc = h->nc; a.ncp = h->ncp; a.b = h->b; a.r = h->r_diag; a.nnz_lu = M.nnz_lu;
     a.nnz_d = h->nnz_d; a.with_T = h->has_T ? 1 : 0;
-    const int big = INT_MAX;
-    STS_CK(cudaMemcpyAsync(M.err_cell, &big, sizeof(int), cudaMemcpyHostToDevice, h->stream));
+    constexpr int kNone = 0x7f7f7f7f;       // above any cell
+    STS_CK(cudaMemsetAsync(M.err_cell, 0x7f, sizeof(int), h->stream));
     if (M.structured) {
         auto lu = M.s_w == 0 ? k_smw_lu_arrow<0> : M.s_w == 1 ? k_smw_lu_arrow<1> : M.s_w == 2 ? k_smw_lu_arrow<2>
                   : M.s_w == 3 ? k_smw_lu_arrow<3> : k_smw_lu_arrow<4>;
@@ -781,13 +780,6 @@ sts_status smw_setup(sts_jac_s *h) {
         else k_smw_cinv<<<(h->ncp + 63) / 64, 64, 0, h->stream>>>(a);      // more than any structured instance holds
         STS_LAUNCHED();
     }
-    int bad = INT_MAX;
-    STS_CK(cudaMemcpyAsync(&bad, M.err_cell, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
-    STS_CK(cudaStreamSynchronize(h->stream));
-    if (bad != INT_MAX)
-        return set_error(STS_ERR_SINGULAR,
-                         "block-Jacobi setup: cell %d has a pivot below 1e-14 x its row maximum "
-                         "(static pivot order) or a singular capacitance matrix C_k", bad);
     const size_t P = h->ncp;
     const int b = h->b, r = h->r_diag;
     for (int dir = 0; dir < 2; ++dir) {
@@ -842,9 +834,20 @@ sts_status smw_setup(sts_jac_s *h) {
             }
         }
     }
-    M.ready = true;
+    // one look at the device for the whole setup, after the packing (which a failed cell
+    // makes useless, not wrong): the wait flag and, beside it, the first failing cell
     h->streams_dirty = true;
-    return STS_OK;
+    int flags[2] = {0, kNone};
+    STS_CK(cudaMemcpyAsync(flags, h->d_err, sizeof(flags), cudaMemcpyDeviceToHost, h->stream));
+    STS_CK(cudaStreamSynchronize(h->stream));
+    if (flags[1] != kNone) {
+        STS_TRY(report_wait(h, flags[0]));
+        return set_error(STS_ERR_SINGULAR,
+                         "block-Jacobi setup: cell %d has a pivot below 1e-14 x its row maximum "
+                         "(static pivot order) or a singular capacitance matrix C_k", flags[1]);
+    }
+    M.ready = true;
+    return report_wait(h, flags[0]);
 }
 
 }  // namespace sts

@@ -218,7 +218,7 @@ struct SmwPlan {
     float *ap32[2] = {nullptr, nullptr};
     float *W32[2] = {nullptr, nullptr};     // W, Wt rounded
     float *DV32[2] = {nullptr, nullptr};    // Vd, Ud rounded (dot vectors of the two directions)
-    int *err_cell = nullptr;     // device: first failing cell (INT_MAX if none)
+    int *err_cell = nullptr;     // device: first failing cell of a setup, beside the handle's wait flag
     bool ready = false;
     // Structured apply (diagonal pattern of the paper's family, no fill): one
     // coefficient stream per direction and precision in ap64 / ap32, s_lt[prec]
@@ -313,7 +313,7 @@ struct sts_jac_s {
     double *staging = nullptr;                  // device copy of host values (first host update on)
     float *vin32 = nullptr, *vout32 = nullptr;
     double *c64 = nullptr;                      // matvec pair dots [n_tiles*n_pslots_max*32]
-    int *d_err = nullptr;                       // device: set when a bounded device wait gave up
+    int *d_err = nullptr;                       // device: [0] set when a bounded device wait gave up, [1] SmwPlan::err_cell
     unsigned *d_sched = nullptr;                // device: matvec pass-2 item counter, finished warps
     float *c32 = nullptr;
     double *g_c = nullptr;                      // adjoint: pair dots of the T direction
@@ -373,6 +373,7 @@ sts_status from_internal32(sts_jac_s *h, const float *xi, float *x);
 sts_status smw_build(sts_jac_s *h);                       // host schedule + device tables
 sts_status smw_setup(sts_jac_s *h);
 sts_status check_device(sts_jac_s *h);                   // STS_ERR_TIMEOUT if a bounded device wait gave up
+sts_status report_wait(sts_jac_s *h, int flag);
 sts_status smw_apply64(sts_jac_s *h, int dir, const Vec<double> &x, const Vec<double> &z);
 sts_status smw_apply32(sts_jac_s *h, int dir, const Vec<float> &x, const Vec<float> &z);
 sts_status smw_sapply32(sts_jac_s *h, int dir, const Vec<float> &x, const Vec<float> &z);     // kernels_smw32.cu
