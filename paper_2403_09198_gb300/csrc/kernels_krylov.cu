@@ -30,16 +30,18 @@ namespace sts {
 namespace {
 
 constexpr int kRedThreads = 256;
-constexpr int kRedMax = 304;        // blocks of a reduction at most: two per SM
+constexpr int kRedMax = 304;        // blocks of a reduction with several totals at most: two per SM
 constexpr int kOrthChunk = 31;      // vectors per sweep: their dots and w . w fill a warp's 32 lanes
 
 // Blocks of the sweeps over n elements and cnt vectors, one element per thread at
 // least.  The sums depend on this number: it is a function of n and cnt alone, so that
 // every caller gets the same bits.  Above kTwoBlocks vectors the accumulators leave
-// room for one block per SM.
+// room for one block per SM; the last sweep has none, and four blocks per SM hide its
+// serial FMA chains (128 x 128 cells, N = 60, 28 / 30 vectors: 86 / 94 -> 71 / 75 us;
+// 24 and fewer are faster in two blocks: 61 against 63 us, 2 vectors 15.5 against 16.9).
 constexpr int kTwoBlocks = 24;
-inline int orth_blocks(long long n, int cnt) {
-    const long long most = cnt <= kTwoBlocks ? kRedMax : kRedMax / 2;
+inline int orth_blocks(long long n, int cnt, bool norm_only = false) {
+    const long long most = cnt <= kTwoBlocks ? kRedMax : norm_only ? 2 * kRedMax : kRedMax / 2;
     return (int)std::max(1LL, std::min(most, (n + kRedThreads - 1) / kRedThreads));
 }
 
@@ -212,7 +214,7 @@ enum { kDots, kDotsOnly, kUpdateDots, kUpdateNorm };
 constexpr int pow2_at_least(int n) { return n <= 1 ? 1 : n <= 2 ? 2 : n <= 4 ? 4 : n <= 8 ? 8 : n <= 16 ? 16 : 32; }
 
 template <int CNT, int MODE>
-__global__ void __launch_bounds__(kRedThreads, CNT <= kTwoBlocks ? 2 : 1)
+__global__ void __launch_bounds__(kRedThreads, CNT <= kTwoBlocks ? 2 : MODE == kUpdateNorm ? 4 : 1)
     k_orth(double *w, const double *V, long long n, const double *hcoef, double *partial, double *out,
            int n_out, unsigned int *ticket, Givens G) {
     constexpr int U = CNT <= 1 ? 8 : CNT <= 3 ? 4 : CNT <= (MODE == kUpdateNorm ? kTwoBlocks - 1 : 6) ? 2 : 1;
@@ -280,7 +282,7 @@ sts_status orth_launch(int mode, int cnt, double *w, const double *V, long long 
     const OrthKernel k = mode == kDots ? orth_kernel<kDots>(cnt, All{})
                          : mode == kDotsOnly ? orth_kernel<kDotsOnly>(cnt, All{})
                          : mode == kUpdateDots ? orth_kernel<kUpdateDots>(cnt, All{}) : orth_kernel<kUpdateNorm>(cnt, All{});
-    const int blocks = orth_blocks(n, cnt);
+    const int blocks = orth_blocks(n, cnt, mode == kUpdateNorm);
     if (early_start(blocks))
         STS_CK(launch_pdl(k, dim3(blocks), dim3(kRedThreads), 0, st, w, V, n, hcoef, partial, out, n_out, ticket, G));
     else
