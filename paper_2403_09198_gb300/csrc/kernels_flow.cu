@@ -645,8 +645,7 @@ sts_status flow_alloc(sts_flow_s *f, double **p, size_t n) {
 sts_status flow_mix(sts_flow_s *f, const double *Q, const double *Qn) {
     const int b = f->dev.b;
     const size_t smem = (32 * (size_t)(b | 1) + 4 * (size_t)f->dev.N + 4 * 5 * 32) * sizeof(double);
-    if (smem > 48 * 1024)
-        STS_CK(cudaFuncSetAttribute(k_flow_mix, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (smem > 48 * 1024) STS_CK(allow_all_smem(k_flow_mix));
     k_flow_mix<<<dim3((f->dev.nc + kMixCells - 1) / kMixCells, Qn ? 2 : 1), 128, smem, f->stream>>>(f->dev, Q, Qn);
     STS_LAUNCHED();
     return STS_OK;

@@ -639,8 +639,7 @@ sts_status mv_launch(sts_jac_s *h, const MvArgs<T> &args) {
         for (const auto &e : h->mvs_resident)
             if (e.kern == reinterpret_cast<const void *>(kern) && e.smem == smem) resident = e.blocks;
         if (!resident) {
-            if (smem > 48 * 1024)
-                STS_CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            if (smem > 48 * 1024) STS_CK(allow_all_smem(kern));
             int per_sm = 0;
             STS_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kWarpsPerBlock * kTile, smem));
             resident = std::max(per_sm, 1) * h->nsm;

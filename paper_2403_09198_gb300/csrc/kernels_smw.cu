@@ -498,8 +498,7 @@ static sts_status smw_apply_t(sts_jac_s *h, int dir, const T *st, const T *dv, c
     const int rmax = a.r <= 2 ? 2 : a.r <= 4 ? 4 : kMaxPairsDiag;
     const size_t smem = ((size_t)kGenWarps * std::min(rmax, kGenSum) + h->b) * kTile * sizeof(T);
     auto kern = rmax == 2 ? k_smw_apply<T, 2> : rmax == 4 ? k_smw_apply<T, 4> : k_smw_apply<T, kMaxPairsDiag>;
-    if (smem > 48 * 1024)
-        STS_CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (smem > 48 * 1024) STS_CK(allow_all_smem(kern));
     kern<<<h->n_tiles, kGenWarps * kTile, smem, h->stream>>>(a);
     STS_LAUNCHED();
     return STS_OK;

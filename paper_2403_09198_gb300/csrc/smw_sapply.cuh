@@ -454,8 +454,7 @@ sts_status smw_sapply_t(sts_jac_s *h, int dir, const T *st, const Vec<T> &x, con
         default: kern = sap_kernel<T, 4>(rm, gw, in); break;
     }
     bool &attr = h->sap_attr[sizeof(T) == 8 ? 0 : 1][in ? 1 : 0];
-    if (!attr && smem > 48 * 1024)
-        STS_CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (!attr && smem > 48 * 1024) STS_CK(allow_all_smem(kern));
     attr = true;
     const int blocks = std::max(1, std::min(h->nsm, (h->n_tiles + wpb - 1) / wpb));
     STS_CK(launch_pdl(kern, dim3(blocks), dim3((wpb + 1) * kTile), smem, h->stream, a));

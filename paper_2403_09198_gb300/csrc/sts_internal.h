@@ -92,6 +92,17 @@ inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, siz
     return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
 }
 
+// Let a kernel take all the shared memory a block can have.  The limit belongs to the
+// kernel, not to a launch: set to one handle's size, it would refuse the launch of
+// another handle that needs more.
+template <typename... KArgs>
+inline cudaError_t allow_all_smem(void (*kern)(KArgs...)) {
+    cudaFuncAttributes at;
+    const cudaError_t e = cudaFuncGetAttributes(&at, kern);
+    return e != cudaSuccess ? e : cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                       227 * 1024 - (int)at.sharedSizeBytes);
+}
+
 #define STS_LAUNCHED()                                                    \
     do {                                                                  \
         ::sts::g_launches.fetch_add(1, std::memory_order_relaxed);        \

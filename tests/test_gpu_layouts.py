@@ -103,3 +103,19 @@ def test_absent_neighbours_add_nothing_in_general_patterns():
     y = host(jac.matvec(dev(x.ravel()))).reshape(3, w.b)
     assert np.isinf(y[0, 0]) and np.isfinite(y[0, 1:]).all() and np.isinf(y[1]).all() and np.isfinite(y[2]).all()
     jac.close()
+
+
+def test_block_sizes_take_turns():
+    """Handles whose launches of one kernel instance need different shared memory, applied
+    in turn: the larger one's launches stay possible after the smaller one's.  Applies on
+    a pattern of one cell solve with the block itself, so J M b = b; the rounding of a
+    block of 63 with entries below 1 on a diagonal above 1000 is far below TOL64."""
+    jacs = []
+    for N in (60, 10):
+        w = inputs.make_workload(1, 1, N=N, w=2, r_diag=2, r_off=0, seed=5)
+        jacs.append((StsJacobian(w, dev(w.S), dev(w.U), dev(w.V)), w))
+        jacs[-1][0].bjacobi_setup()
+    for j, w in jacs + jacs:
+        assert rel_err(host(j.matvec(j.bjacobi_apply(dev(w.rhs)))), w.rhs) <= TOL64
+    for j, _ in jacs:
+        j.close()
