@@ -118,7 +118,7 @@ __device__ __forceinline__ bool grid_totals(double (&v)[NV], int used, double *p
     return true;
 }
 
-// State of the device-side rotations (see k_givens_step); H = NULL: none.
+// State of the device-side rotations (see givens_step); H = NULL: none.
 struct Givens {
     int j, m;
     const double *h1, *h2;
@@ -208,7 +208,7 @@ __device__ __noinline__ void givens_step(const Givens &G, double hn2) {
 // memory below.  Measured on 128 x 128 cells, N = 60 (1.03 M elements): with dots,
 // update, dots and update as four sweeps and 5 additions per value and warp in the
 // reductions, the 163 steps of a Newton step (16 vectors on average) took 31.3 ms, now
-// 23.6 ms, the rotations included; 18.2 ms are FP64 pipe time.
+// 22.4 ms, the rotations included; 18.2 ms are FP64 pipe time.
 enum { kDots, kDotsOnly, kUpdateDots, kUpdateNorm };
 
 constexpr int pow2_at_least(int n) { return n <= 1 ? 1 : n <= 2 ? 2 : n <= 4 ? 4 : n <= 8 ? 8 : n <= 16 ? 16 : 32; }
