@@ -435,11 +435,14 @@ sts_status smw_build(sts_jac_s *h) {
                 // vectors to pack: those that scale an entry first; none for all zeros or folded tails
                 std::vector<int> list, plain;
                 for (int v = 0; v < (int)src.size() / vec; ++v) {
-                    bool any = false, scaled = false;
+                    bool any = false, scaled = false, folded = false;
                     for (int e = v * vec; e < (v + 1) * vec; ++e) {
                         any = any || src[e] > -4;
                         scaled = scaled || (src[e] >= 0 && arg[e] >= 0);
+                        folded = folded || src[e] == -5;
                     }
+                    // a packed vector is written whole, beside the kernel's folding blocks
+                    if (any && folded) return set_error(STS_ERR_INVALID_ARG, "internal: structured apply vector");
                     if (any) (scaled ? list : plain).push_back(v);
                 }
                 M.spk_scaled[prec][dir] = (int)list.size();

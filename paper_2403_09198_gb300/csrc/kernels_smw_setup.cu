@@ -642,38 +642,44 @@ __global__ void k_round(T *out, const double *in, long long n) {
 // need a product with a pivot inverse first: a product that a predicate switches
 // off still takes its FP64 pipe slot, so the others run a loop without one.  The
 // zeros of the other vectors were written when the stream was allocated.
-// Measured on 128 x 128 cells, N = 60: two pairs 68 -> 51 us per direction; nine pairs,
-// the fold included, 280 -> 68 + 173 us.
+// Measured on 128 x 128 cells, N = 60: two pairs 68 -> 51 us per direction.
 constexpr int kPackWarps = 4;
 template <typename T> struct PackVec;
 template <> struct PackVec<double> { using type = double2; };
 template <> struct PackVec<float> { using type = float4; };
 
 template <typename T>
-__global__ void __launch_bounds__(kPackWarps * kTile) k_smw_spack(T *out, const double *lu, const double *dinv,
-                                                                  const double *DV, const double *WW, const int *src,
-                                                                  const int *arg, const int *list, int n_scaled,
-                                                                  int n_list, int Lt, int ncp) {
+struct PackArgs {
+    T *out;
+    const double *lu, *dinv, *DV, *WW;
+    const int *src, *arg, *list;
+    int n_scaled, n_list, Lt, ncp;
+};
+
+// Part `part` of `parts` of the tile blockIdx.x.
+template <typename T>
+__device__ __forceinline__ void pack_part(const PackArgs<T> &A, int part, int parts) {
     constexpr int VEC = 16 / (int)sizeof(T);
     using V = typename PackVec<T>::type;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const size_t cell = (size_t)blockIdx.x * kTile + lane;
-    T *o = out + ((size_t)blockIdx.x * Lt) * kTile + (size_t)lane * VEC;
-    const int step = gridDim.y * kPackWarps;
+    const size_t ncp = A.ncp;
+    T *o = A.out + ((size_t)blockIdx.x * A.Lt) * kTile + (size_t)lane * VEC;
+    const int step = parts * kPackWarps;
     auto run = [&](auto scaled, int i0, int i1) {
 #pragma unroll 4
         for (int i = i0; i < i1; i += step) {
-            const int pv = __ldg(list + i);
+            const int pv = __ldg(A.list + i);
             alignas(16) T v[VEC];
 #pragma unroll
             for (int j = 0; j < VEC; ++j) {
                 // loads without branches, so that the unrolled vectors' loads are in flight together
-                const int sv = __ldg(src + pv * VEC + j), ag = __ldg(arg + pv * VEC + j);
-                const double *s = sv >= 0 ? lu : sv == -2 ? DV : sv == -3 ? WW : dinv;
+                const int sv = __ldg(A.src + pv * VEC + j), ag = __ldg(A.arg + pv * VEC + j);
+                const double *s = sv >= 0 ? A.lu : sv == -2 ? A.DV : sv == -3 ? A.WW : A.dinv;
                 double e = __ldg(s + (size_t)(sv >= 0 ? sv : sv > -4 ? ag : 0) * ncp + cell);
                 if constexpr (decltype(scaled)::value) {
                     const bool on = sv >= 0 && ag >= 0;
-                    const double d = __ldg(dinv + (size_t)(on ? ag : 0) * ncp + cell);
+                    const double d = __ldg(A.dinv + (size_t)(on ? ag : 0) * ncp + cell);
                     e *= on ? d : 1.0;
                 }
                 v[j] = sv > -4 ? (T)e : T(0);
@@ -681,31 +687,47 @@ __global__ void __launch_bounds__(kPackWarps * kTile) k_smw_spack(T *out, const 
             *reinterpret_cast<V *>(o + (size_t)pv * kTile * VEC) = *reinterpret_cast<V *>(v);
         }
     };
-    const int w = blockIdx.y * kPackWarps + warp;
-    run(std::true_type{}, w, n_scaled);
-    run(std::false_type{}, n_scaled + w, n_list);
+    const int w = part * kPackWarps + warp;
+    run(std::true_type{}, w, A.n_scaled);
+    run(std::false_type{}, A.n_scaled + w, A.n_list);
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kPackWarps * kTile) k_smw_spack(PackArgs<T> A) {
+    pack_part(A, blockIdx.y, gridDim.y);
 }
 
 // Folded tail entries (W C^-1)[q][a] = sum_l W[l][q] C^-1[l][a] (transposed: W'
 // and C^-T), in FP64, into their stream positions tp[a * b + q] of the FP64
 // stream and, where there is one, the FP32 stream.  One warp per tile and rows
 // q; the r entries of W are read once for the r sums, C^-1 sits in shared
-// memory.  r^2 FMAs a row: bound by the FP64 pipe (133 of the 173 us of nine pairs on
-// 128 x 128 cells, N = 60).
+// memory.  r^2 FMAs a row: bound by the FP64 pipe.  The rest of the FP64 stream, bound
+// by memory, is packed beside it by `parts` of the blocks of every tile, which alternate
+// with the folding ones as far as they go.  Nine pairs on 128 x 128 cells, N = 60:
+// 280 us in one kernel that formed a fold entry per position, 68 + 173 us as two kernels
+// (133 us of FP64 pipe time), 216 us here.
 constexpr int kFoldWarps = 4;
 
 template <int R>
-__global__ void __launch_bounds__(kFoldWarps * kTile) k_smw_fold(double *out64, float *out32, const int *tp64,
-                                                                 const int *tp32, int Lt64, int Lt32,
-                                                                 const double *WW, const double *Cinv, int b, int ncp,
-                                                                 int trans) {
+__global__ void __launch_bounds__(kFoldWarps * kTile) k_smw_fold(PackArgs<double> A, int parts, float *out32,
+                                                                 const int *tp64, const int *tp32, int Lt32,
+                                                                 const double *Cinv, int b, int trans) {
     __shared__ double sc[R * R][kTile];
+    const int y = blockIdx.y, folds = gridDim.y - parts, both = min(parts, folds);
+    const int part = y < 2 * both ? y >> 1 : y - both;
+    if (y < 2 * both ? !(y & 1) : parts > folds) {
+        pack_part(A, part, parts);
+        return;
+    }
+    double *out64 = A.out;
+    const double *WW = A.WW;
+    const int Lt64 = A.Lt, ncp = A.ncp;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const size_t tile = blockIdx.x, cell = tile * kTile + lane;
     for (int i = warp; i < R * R; i += kFoldWarps)           // sc[l * R + a]
         sc[i][lane] = __ldg(Cinv + (size_t)(trans ? (i % R) * R + i / R : i) * ncp + cell);
     __syncthreads();
-    for (int q = blockIdx.y * kFoldWarps + warp; q < b; q += gridDim.y * kFoldWarps) {
+    for (int q = part * kFoldWarps + warp; q < b; q += folds * kFoldWarps) {
         double w[R];
 #pragma unroll
         for (int l = 0; l < R; ++l) w[l] = __ldg(WW + ((size_t)l * b + q) * ncp + cell);
@@ -792,28 +814,27 @@ sts_status smw_setup(sts_jac_s *h) {
                 return (unsigned)std::max(1, std::min((work + 4 * kPackWarps - 1) / (4 * kPackWarps),
                                                       (h->nsm * 64 + nt * kPackWarps - 1) / (nt * kPackWarps)));
             };
-            k_smw_spack<double><<<dim3(nt, ysplit(M.spk_n[0][dir])), kPackWarps * kTile, 0, h->stream>>>(
-                M.ap64[dir], M.lu, M.dinv, DV, WW, M.spk_src[0][dir], M.spk_arg[0][dir], M.spk_list[0][dir],
-                M.spk_scaled[0][dir], M.spk_n[0][dir], M.s_lt[0], h->ncp);
-            STS_LAUNCHED();
+            const PackArgs<double> p64{M.ap64[dir], M.lu, M.dinv, DV, WW, M.spk_src[0][dir], M.spk_arg[0][dir],
+                                       M.spk_list[0][dir], M.spk_scaled[0][dir], M.spk_n[0][dir], M.s_lt[0], h->ncp};
+            const unsigned parts = ysplit(M.spk_n[0][dir]);
             if (M.ap32[dir]) {
-                k_smw_spack<float><<<dim3(nt, ysplit(M.spk_n[1][dir])), kPackWarps * kTile, 0, h->stream>>>(
-                    M.ap32[dir], M.lu, M.dinv, DV, WW, M.spk_src[1][dir], M.spk_arg[1][dir], M.spk_list[1][dir],
-                    M.spk_scaled[1][dir], M.spk_n[1][dir], M.s_lt[1], h->ncp);
+                const PackArgs<float> p32{M.ap32[dir], M.lu, M.dinv, DV, WW, M.spk_src[1][dir], M.spk_arg[1][dir],
+                                          M.spk_list[1][dir], M.spk_scaled[1][dir], M.spk_n[1][dir], M.s_lt[1], h->ncp};
+                k_smw_spack<float><<<dim3(nt, ysplit(M.spk_n[1][dir])), kPackWarps * kTile, 0, h->stream>>>(p32);
                 STS_LAUNCHED();
             }
             if (M.tail_pos[0] && r > 0) {
                 static_assert(kPackWarps == kFoldWarps, "one split rule");
-                using Fold = void (*)(double *, float *, const int *, const int *, int, int, const double *,
-                                      const double *, int, int, int);
+                using Fold = void (*)(PackArgs<double>, int, float *, const int *, const int *, int, const double *, int, int);
                 static const Fold fold[11] = {nullptr, k_smw_fold<1>, k_smw_fold<2>, k_smw_fold<3>, k_smw_fold<4>,
                                               k_smw_fold<5>, k_smw_fold<6>, k_smw_fold<7>, k_smw_fold<8>,
                                               k_smw_fold<9>, k_smw_fold<10>};
-                fold[r]<<<dim3(nt, ysplit(b)), kFoldWarps * kTile, 0, h->stream>>>(
-                    M.ap64[dir], M.ap32[dir], M.tail_pos[0], M.tail_pos[1], M.s_lt[0], M.s_lt[1], WW, M.Cinv, b,
-                    h->ncp, dir);
-                STS_LAUNCHED();
+                fold[r]<<<dim3(nt, parts + ysplit(b)), kFoldWarps * kTile, 0, h->stream>>>(
+                    p64, (int)parts, M.ap32[dir], M.tail_pos[0], M.tail_pos[1], M.s_lt[1], M.Cinv, b, dir);
+            } else {
+                k_smw_spack<double><<<dim3(nt, parts), kPackWarps * kTile, 0, h->stream>>>(p64);
             }
+            STS_LAUNCHED();
             continue;
         }
         const int len = kGenWarps * M.g_wlen[dir];
