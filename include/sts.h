@@ -31,8 +31,8 @@
  *   sts_jac_desc.vec_layout: STS_LAYOUT_CELL_MAJOR stores cell c's b values
  *   contiguously (x[c*b + p]); STS_LAYOUT_COMPONENT_MAJOR stores component p of
  *   all cells contiguously (x[p*n_cells + c]), close to the layout the kernels use
- *   internally: it is read and written in place, where large cell-major vectors
- *   take two transposes per product.
+ *   internally: it is read and written in place, where a large cell-major operand
+ *   is transposed first.
  * - "device" pointers are CUDA device (or managed) memory on the current
  *   device; "host" pointers are ordinary host memory.  The library never takes
  *   ownership of caller memory; arguments need to stay valid only for the

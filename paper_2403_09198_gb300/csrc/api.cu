@@ -588,16 +588,20 @@ sts_status create_impl(const sts_jac_desc *d, sts_jac_t *out) {
 
 // Run an operator on public-layout vectors: in place where the kernels can take them
 // (any_layout), else through the internal layout.  In place are component-major vectors,
-// whose 32 cells of a component are contiguous (aligned or not), and cell-major ones of
-// up to direct_max values.  A lane's component of a cell-major vector is a sector of its
-// own, but two transposes per call, each a launch, are saved.  Measured on cell-major
-// vectors, us per call through the internal layout and in place:
-//   apply, 2 to 1152 tiles of 32 cells, N = 10: 18.6 and 10.5 (30.9 and 19.9 at 1152 tiles);
-//     N = 60: 51.4 and 42.3 at 2 tiles, 57.5 and 46.3 at 512, 104.8 and 90.0 at 1152: always;
-//   matvec, which reads x about 25 times, N = 10: 21.8 and 12.8 at 2 tiles, 70.2 and 60.7 at
-//     1152 (479 K values); N = 60: 47.0 and 43.6 at 128 tiles (258 K values), 74.6 and 77.9 at
-//     288 (581 K), 113.4 and 113.6 at 512.
-constexpr long long kMatvecDirect = 1 << 19, kApplyDirect = 1LL << 62;
+// whose 32 cells of a component are contiguous (aligned or not), the result of every
+// cell-major call, and its operand up to direct_max values.  A lane's component of a
+// cell-major vector is a sector of its own: one write per row hides behind the FP64 pipe
+// and merges in L2, but a product reads its operand about 25 times, against the launch
+// that a transpose takes.  Measured on cell-major vectors, us per call:
+//   apply, both vectors transposed and in place, N = 10: 18.6 and 10.5 at 2 tiles of 32
+//     cells, 30.9 and 19.9 at 1152; N = 60: 51.4 and 42.3 at 2, 104.8 and 90.0 at 1152: always;
+//   matvec, both vectors transposed and x alone, N = 60: 112.7 and 106.7 at 512 tiles, 384.3
+//     and 371.9 at 2048; N = 200 at 512 tiles 350.6 and 337.9; FP32 52.8 and 49.4 (N = 60, 512);
+//   matvec, x transposed and in place, FP64: N = 60 20.6 and 14.5 at 4 K values, 39.0 and 39.0
+//     at 258 K, 66.1 and 69.7 at 488 K; N = 20 38.9 and 39.0 at 212 K, 63.4 and 67.2 at 451 K;
+//     N = 10 36.9 and 34.7 at 213 K.  FP32, where no pipe hides the reads: N = 60 14.8 and
+//     12.3 at 16 K, 16.4 and 18.5 at 36 K; N = 20 16.4 and 14.8 at 24 K, 22.8 and 25.7 at 212 K.
+constexpr long long kMatvecDirect = 1 << 18, kMatvecDirect32 = 1 << 15, kApplyDirect = 1LL << 62;
 
 template <typename T, typename F>
 sts_status with_layout(sts_jac_s *h, bool any_layout, long long direct_max, const T *x, T *y, T *bin, T *bout, F op) {
@@ -607,6 +611,11 @@ sts_status with_layout(sts_jac_s *h, bool any_layout, long long direct_max, cons
         return op(Vec<T>{const_cast<T *>(x), sc, sq, h->nc, bout}, Vec<T>{y, sc, sq, h->nc, bout});
     }
     if (comp && h->nc == h->ncp) return op(internal_vec(h, x), internal_vec(h, y));
+    if (any_layout) {       // cell-major: only x is worth a transpose
+        if constexpr (sizeof(T) == 8) STS_TRY(to_internal64(h, x, bin));
+        else STS_TRY(to_internal32(h, x, bin));
+        return op(internal_vec(h, bin), Vec<T>{y, h->b, 1, h->nc, bout});
+    }
     if constexpr (sizeof(T) == 8) {
         STS_TRY(to_internal64(h, x, bin));
         STS_TRY(op(internal_vec(h, bin), internal_vec(h, bout)));
@@ -724,7 +733,7 @@ sts_status sts_jac_matvec_f32(sts_jac_t h, const float *x, float *y, int trans) 
     if (h->dtype != STS_MIXED) return set_error(STS_ERR_INVALID_ARG, "sts_jac_matvec_f32: handle has no FP32 operators");
     if (trans && !h->has_T) return set_error(STS_ERR_INVALID_ARG, "sts_jac_matvec_f32: no transposed operators");
     const int dir = trans ? 1 : 0;
-    STS_GUARD(return with_layout<float>(h, true, kMatvecDirect, x, y, h->vin32, h->vout32,
+    STS_GUARD(return with_layout<float>(h, true, kMatvecDirect32, x, y, h->vin32, h->vout32,
                                         [&](const Vec<float> &a, const Vec<float> &b) {
         return mv_apply32(h, dir, a, b, h->c32);
     });)

@@ -259,7 +259,7 @@ __global__ void __launch_bounds__(64) k_mv_struct(MvArgs<T> a) {
     constexpr int BANDW = 2 * WD + 1;
     const int lane = threadIdx.x & 31;
     const int ns = a.n_slots, nps = a.n_pslots, N = a.sN;
-    const size_t sq = INT ? (size_t)a.ncp : (size_t)a.x.sq;
+    const size_t sq = INT ? (size_t)a.ncp : (size_t)a.x.sq, ysq = INT ? sq : (size_t)a.y.sq;
     const int RL = a.s_rl;
     const uint32_t row_bytes = (uint32_t)RL * kTile * (uint32_t)sizeof(T);
     extern __shared__ __align__(128) unsigned char mv_smem[];
@@ -314,7 +314,7 @@ __global__ void __launch_bounds__(64) k_mv_struct(MvArgs<T> a) {
             for (int s = 0; s < ns; ++s) acc += __ldg(cc + (size_t)(nps + f * ns + s) * kTile);
             for (int k = 0; k < nps; ++k)
                 acc = fma(__ldg(su + (size_t)(f * nps + k) * kTile), __ldg(cc + (size_t)k * kTile), acc);
-            if (INT || cell < a.y.cells) a.y.template cell<INT>(cell)[(size_t)(N + f) * sq] = acc;
+            if (INT || cell < a.y.cells) a.y.template cell<INT>(cell)[(size_t)(N + f) * ysq] = acc;
         }
         continue;
     }
@@ -362,7 +362,7 @@ __global__ void __launch_bounds__(64) k_mv_struct(MvArgs<T> a) {
     T xn[NS];
 #pragma unroll
     for (int s = 1; s < NS; ++s) xn[s] = s < ns ? __ldg(xs[s] + (size_t)p0 * sq) : T(0);
-    T *yp = a.y.template cell<INT>(cell) + (size_t)p0 * sq;      // y has x's strides
+    T *yp = a.y.template cell<INT>(cell) + (size_t)p0 * ysq;
     const bool on = INT || cell < a.y.cells;
     T ylag = T(0);          // row p-1's result, stored during row p (its FMA has long completed)
     for (int p = p0; p < p1; ++p) {
@@ -450,7 +450,7 @@ __global__ void __launch_bounds__(64) k_mv_struct(MvArgs<T> a) {
         }
         if (p > p0) {
             if (on) *yp = ylag;
-            yp += sq;
+            yp += ysq;
         }
         ylag = acc;
         __syncwarp();     // every lane is done with the stage before it is refilled
@@ -624,7 +624,7 @@ sts_status mv_launch(sts_jac_s *h, const MvArgs<T> &args) {
         const size_t smem = (size_t)kWarpsPerBlock * mv_struct_warp_bytes(a.s_rl, (int)sizeof(T));
         void (*kern)(MvArgs<T>) = nullptr;
         const int nreg = a.n_pslots <= 8 ? 8 : a.n_pslots <= 2 * kStructDuff ? 2 * kStructDuff : 0;
-        const bool in = a.x.internal(a.ncp);
+        const bool in = a.x.internal(a.ncp) && a.y.internal(a.ncp);
         switch (a.wd) {
             case 0: kern = mv_struct_kernel<T, 0>(nreg, in); break;
             case 1: kern = mv_struct_kernel<T, 1>(nreg, in); break;

@@ -1,8 +1,8 @@
 """Operators on public vectors in place, and the general kernels' programs.
 
-Small cell-major and all component-major vectors are read and written in place;
-larger cell-major matvecs, and applies whose working vector lives in y, go through the
-internal layout.  Either way the arithmetic is the same, so every layout gives the
+Component-major and small cell-major vectors are read and written in place; larger
+cell-major matvecs transpose x, and applies whose working vector lives in y go through
+the internal layout.  Either way the arithmetic is the same, so every layout gives the
 same bits.
 """
 import numpy as np
@@ -33,11 +33,13 @@ def _calls(jac, x, out):
     return got
 
 
-# ragged and full tiles; 130 x 127 x 33 values are more than the largest in-place
-# cell-major matvec (2^19); b = 143 keeps the apply's working vector in y (FP64)
-@pytest.mark.parametrize("Lx,Ly,N", [(8, 4, 20), (5, 7, 60), (130, 127, 30), (9, 8, 140)])
-def test_layouts_give_the_same_bits(Lx, Ly, N):
-    w = inputs.make_workload(Lx, Ly, N=N, w=2, r_diag=2, r_off=1, seed=70)
+# ragged and full tiles; 130 x 127 x 33 values are more than a cell-major matvec reads
+# in place in FP64 (2^18), 60 x 50 x 33 more than in FP32 (2^15); b = 143 keeps the apply's
+# working vector in y (FP64)
+@pytest.mark.parametrize("Lx,Ly,N,density", [(8, 4, 20, 0.0), (5, 7, 60, 0.0), (60, 50, 30, 0.0), (130, 127, 30, 0.0),
+                                             (9, 8, 140, 0.0), (91, 90, 30, 0.1)])
+def test_layouts_give_the_same_bits(Lx, Ly, N, density):
+    w = inputs.make_workload(Lx, Ly, N=N, w=2, r_diag=2, r_off=1, seed=70, random_density=density)
     x = np.random.default_rng(1).standard_normal(w.n)
     got = {}
     for layout in ("cell", "component"):
