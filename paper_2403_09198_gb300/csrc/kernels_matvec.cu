@@ -146,10 +146,12 @@ __global__ void __launch_bounds__(128) k_dots(MvArgs<T> a) {
 // serially.  A chunk's values and operands are loaded one chunk ahead: an operand's
 // address comes out of its descriptor, so a load at its use is two memory latencies
 // per position.  With few tiles a group is one row and a warp's own instructions set
-// the time (41 x 37 cells, b = 33, 15% filled: 22 us, now 10).
-template <typename T>
+// the time (41 x 37 cells, b = 33, 15% filled: 22 us, now 10).  Chunks of 8 there; FP64
+// grids of more warps than fit beside chunks of 8 take 4 (whole products, 128 / 800
+// tiles: 26 / 91 us, 30 / 98 with longer chunks; the products of 47 tiles 20.5 and 21.7).
+constexpr int kMainWarps = 20;      // resident warps per SM with chunks of 8
+template <typename T, int CH>
 __global__ void __launch_bounds__(128) k_mv_main(MvArgs<T> a) {
-    constexpr int CH = 8;
     __shared__ int snb[4][kMaxSlots][kTile];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const long long wid = (long long)blockIdx.x * (blockDim.x >> 5) + wib;
@@ -601,14 +603,16 @@ void (*mv_struct_kernel(int nreg, bool internal))(MvArgs<T>) {
 // with s_rl = 30, 102.7 / 102.0 / 106.5 / - / -; with the paper's pair counts
 // (s_rl = 41), 145.0 / 144.8 / 147.5 / 148.5 / 148.2.  The constant puts both
 // at 5 rows.
-inline int pass2_group_rows(int N, int n_tiles, long long W, int s_plan, int s_rl) {
+inline int pass2_group_rows(int N, int n_tiles, long long W, int s_plan, int s_rl, bool spread) {
     const long long items = (long long)n_tiles * ((N + s_plan - 1) / s_plan + 1);
     if (W <= 0 || items >= 8 * W) return s_plan;
     const int s = std::max(1, std::min({N, 8, std::max(4, (int)std::lround(3.8 * std::sqrt((double)N / std::max(s_rl, 1))))}));
     // small meshes: the fewest rows that still give every item a warp of its own, so that
     // a warp's serial rows, not the number of items, set the time (whole products, cell-major
     // in place, us: N = 10, 32 tiles 22.1 -> 14.6, 128 tiles 26.0 -> 16.7; N = 60, 32 tiles
-    // 36.3 -> 21.9, 128 tiles 43.6 -> 39.9)
+    // 36.3 -> 21.9, 128 tiles 43.6 -> 39.9).  Not in FP32 (spread = false), whose rows are
+    // short against an item's start: N = 60, 8 / 128 tiles 10.3 / 17.6 us, spread 12.1 / 19.2
+    if (!spread) return s;
     const long long per_tile = W / n_tiles - 1;
     return per_tile > 0 ? (int)std::min<long long>(s, (N + per_tile - 1) / per_tile) : s;
 }
@@ -645,7 +649,8 @@ sts_status mv_launch(sts_jac_s *h, const MvArgs<T> &args) {
             resident = std::max(per_sm, 1) * h->nsm;
             h->mvs_resident.push_back({reinterpret_cast<const void *>(kern), smem, resident});
         }
-        a.s_gl = pass2_group_rows(a.sN, a.n_tiles, (long long)resident * kWarpsPerBlock, a.s_gl, a.s_rl);
+        a.s_gl = pass2_group_rows(a.sN, a.n_tiles, (long long)resident * kWarpsPerBlock, a.s_gl, a.s_rl,
+                                 sizeof(T) == 8);
         a.n_lgroups = (a.sN + a.s_gl - 1) / a.s_gl;
         a.n_groups = a.n_lgroups + 1;
         warps = (long long)a.n_tiles * a.n_groups;
@@ -656,7 +661,8 @@ sts_status mv_launch(sts_jac_s *h, const MvArgs<T> &args) {
         // blocks that start late do not finish late
         STS_CK(launch_pdl(kern, dim3((unsigned)blocks), dim3(kWarpsPerBlock * kTile), smem, h->stream, a));
     } else {
-        k_mv_main<T><<<grid, 128, 0, h->stream>>>(a);
+        const bool full = sizeof(T) == 8 && warps > (long long)kMainWarps * h->nsm;
+        (full ? k_mv_main<T, sizeof(T) == 8 ? 4 : 8> : k_mv_main<T, 8>)<<<grid, 128, 0, h->stream>>>(a);
     }
     STS_LAUNCHED();
     return STS_OK;
