@@ -285,8 +285,8 @@ sts_status sts_jac_bjacobi_apply_f32(sts_jac_t h, const float *x, float *z, int 
  * Mixed mode: FP32 matvec and block-Jacobi, FP64 Krylov basis, Arnoldi,
  * residual refresh and capacitance solves, flexible GMRES.  Convergence is
  * declared on the FP64 true residual only.  Synchronous; info may be NULL.
- * Errors: STS_ERR_NOT_CONVERGED (x valid), STS_ERR_NUMERIC, STS_ERR_NOT_SETUP,
- * STS_ERR_TIMEOUT (see sts_jac_bjacobi_apply).
+ * Errors: STS_ERR_NOT_CONVERGED (x valid), STS_ERR_NUMERIC (x as it was on entry),
+ * STS_ERR_NOT_SETUP, STS_ERR_TIMEOUT (see sts_jac_bjacobi_apply).
  */
 sts_status sts_gmres_solve(sts_jac_t h, const double *b, double *x, const sts_gmres_opts *opts,
                            sts_gmres_info *info);

@@ -297,11 +297,21 @@ __global__ void k_sub(double *r, const double *b, const double *y, long long n) 
         r[e] = b[e] - y[e];
 }
 
-// r = b - y and out[0] = r . r, in the order of a difference followed by a norm; with
-// err_out also a copy of the handle's error flag, for the host to read with the norm.
+// What k_residual leaves beside the norm after a graph cycle (err = NULL: nothing): a copy
+// of the handle's error flag, and whether the solve ends here with a result, as the host
+// will decide it from the same numbers (its square root and quotient round alike): steps
+// that did not break down, a finite norm, and rtol reached or none of the `left` steps left.
+struct CycleEnd {
+    const int *err, *state;
+    double bnorm, rtol;
+    int left;
+    int *err_out, *done;
+};
+
+// r = b - y and out[0] = r . r, in the order of a difference followed by a norm.
 __global__ void __launch_bounds__(kRedThreads, 2) k_residual(double *r, const double *b, const double *y, long long n,
                                                              double *partial, double *out, unsigned int *ticket,
-                                                             const int *err, int *err_out) {
+                                                             CycleEnd E) {
     constexpr int U = 4;
     double acc[1] = {0.0};
     const long long stride = (long long)gridDim.x * blockDim.x;
@@ -321,7 +331,11 @@ __global__ void __launch_bounds__(kRedThreads, 2) k_residual(double *r, const do
         r[e] = v;
         acc[0] = fma(v, v, acc[0]);
     }
-    if (grid_totals<1>(acc, 1, partial, out, ticket) && err_out && threadIdx.x == 0) *err_out = *err;
+    if (grid_totals<1>(acc, 1, partial, out, ticket) && E.err && threadIdx.x == 0) {
+        const double norm = sqrt(out[0]);
+        *E.err_out = *E.err;
+        *E.done = E.state[1] != 2 && isfinite(norm) && (norm / E.bnorm <= E.rtol || E.state[0] >= E.left);
+    }
 }
 
 // out[y] = ||v_y||^2 of the two vectors, blockIdx.y = y, each in the order of its own sweep.
@@ -542,6 +556,7 @@ sts_status cycle_graph(sts_jac_s *h, int m, int dir, bool pre) {
         K.gstate = reinterpret_cast<int *>(K.gbuf + 4);
         K.grn = K.gbuf + 5;
         K.gerr = reinterpret_cast<int *>(K.gbuf + 6);
+        K.gdone = reinterpret_cast<int *>(K.gbuf + 7);
         K.gg = K.gbuf + 8;
         K.ghist = K.gg + (M + 1);
         K.gH = K.gbuf + io;
@@ -733,18 +748,18 @@ sts_status gmres(sts_jac_s *h, const double *b_pub, double *x_pub, const sts_gmr
     if (!std::isfinite(bnorm)) return set_error(STS_ERR_NUMERIC, "gmres: right-hand side has NaN or Inf");
     sts_gmres_info inf{0, 0, 1, 0.0, 0, 0};
     sts_status status = STS_OK;
-    bool written = false;       // x_pub holds the present x, and the error flag has been read
+    bool written = false;       // x_pub holds the result, and the error flag has been read
     if (bnorm == 0.0) {
         STS_CK(cudaMemsetAsync(K.xb, 0, n * sizeof(double), h->stream));
     } else {
         std::vector<double> H((size_t)(m + 1) * m), cs(m), sn(m), g(m + 1), y(m);
         int its = 0;
         // r = b - A x and its squared norm
-        auto residual = [&](double *norm, int *err_out) -> sts_status {
+        auto residual = [&](double *norm, const CycleEnd &end) -> sts_status {
             STS_TRY(opA64(h, dir, K.xb, K.w));
             ++inf.matvecs;
             k_residual<<<orth_blocks(n, 0), kRedThreads, 0, h->stream>>>(K.r, K.bb, K.w, n, K.partial, norm, K.ticket,
-                                                                         h->d_err, err_out);
+                                                                         end);
             STS_LAUNCHED();
             return STS_OK;
         };
@@ -761,7 +776,7 @@ sts_status gmres(sts_jac_s *h, const double *b_pub, double *x_pub, const sts_gmr
                 beta = beta_known;
                 beta_known = -1.0;
             } else {
-                STS_TRY(residual(K.red, nullptr));
+                STS_TRY(residual(K.red, CycleEnd{}));
                 STS_CK(cudaMemcpyAsync(hp, K.red, sizeof(double), cudaMemcpyDeviceToHost, h->stream));
                 STS_CK(cudaStreamSynchronize(h->stream));
                 beta = std::sqrt(hp[0]);
@@ -796,14 +811,16 @@ sts_status gmres(sts_jac_s *h, const double *b_pub, double *x_pub, const sts_gmr
             g[0] = g0;
             int k = 0;
             if (use_graph) {
-                // the whole cycle on the device, then x, its residual and (for device vectors) the
-                // result, so that one synchronisation ends a cycle whether it is the last or not
-                // (it took four; one-cycle solves on 16 x 16 cells, N = 10 338 -> 290 us, with the
-                // shorter rotations)
+                // the whole cycle on the device, then x, its residual and (for device vectors, if
+                // the solve ends here with a result: the caller's x stays as it was after a
+                // failure) the result, so that one synchronisation ends a cycle whether it is the
+                // last or not (it took four; one-cycle solves on 16 x 16 cells, N = 10
+                // 338 -> 290 us, with the shorter rotations)
                 NvtxRange nvtx_graph("gmres cycle graph");
                 STS_TRY(cycle_graph(h, m, dir, pre));
                 double *pp = K.g_pinned, *pg = pp + 8, *ph = pg + (K.m + 1);
                 const int *ps = reinterpret_cast<const int *>(pp + 4), *pe = reinterpret_cast<const int *>(pp + 6);
+                const int *pd = reinterpret_cast<const int *>(pp + 7);
                 pp[0] = stop_abs;
                 pp[1] = hscale;
                 pp[2] = 0.0;
@@ -815,8 +832,8 @@ sts_status gmres(sts_jac_s *h, const double *b_pub, double *x_pub, const sts_gmr
                 STS_LAUNCHED();
                 k_axpy_multi<double><<<nb, 256, 0, h->stream>>>(K.xb, K.Z, n, K.gy, 0, K.gstate);
                 STS_LAUNCHED();
-                STS_TRY(residual(K.grn, K.gerr));
-                if (!d.vectors_on_host) STS_TRY(from_internal64(h, K.xb, x_pub));
+                STS_TRY(residual(K.grn, CycleEnd{h->d_err, K.gstate, bnorm, rtol, max_iters - its, K.gerr, K.gdone}));
+                if (!d.vectors_on_host) STS_TRY(from_internal64(h, K.xb, x_pub, K.gdone));
                 STS_CK(cudaMemcpyAsync(pp, K.gbuf, sizeof(double) * (8 + (K.m + 1) + K.m), cudaMemcpyDeviceToHost,
                                        h->stream));
                 STS_CK(cudaStreamSynchronize(h->stream));
@@ -831,7 +848,7 @@ sts_status gmres(sts_jac_s *h, const double *b_pub, double *x_pub, const sts_gmr
                 inf.matvecs += k;
                 if (pre) inf.applies += k;
                 ++inf.restarts;
-                written = !d.vectors_on_host && *pe == 0;
+                written = !d.vectors_on_host && *pd && *pe == 0;
                 beta_known = std::sqrt(pp[5]);
                 continue;
             }

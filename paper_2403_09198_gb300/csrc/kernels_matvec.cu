@@ -492,9 +492,11 @@ __global__ void k_cell_to_comp(const T *__restrict__ x, T *__restrict__ xi, int 
     }
 }
 
+// go (may be NULL): nothing is written where the device has left it zero.
 template <typename T>
-__global__ void k_comp_to_cell(const T *__restrict__ xi, T *__restrict__ x, int nc, int b, int ncp) {
+__global__ void k_comp_to_cell(const T *__restrict__ xi, T *__restrict__ x, int nc, int b, int ncp, const int *go) {
     __shared__ T tile[32][33];
+    if (go && !*go) return;
     const int c0 = blockIdx.x * 32, q0 = blockIdx.y * 32;
     for (int r = threadIdx.y; r < 32; r += blockDim.y) {
         const int q = q0 + r, c = c0 + threadIdx.x;
@@ -518,7 +520,8 @@ __global__ void k_comp_pad(const T *__restrict__ x, T *__restrict__ xi, int nc, 
 }
 
 template <typename T>
-__global__ void k_comp_unpad(const T *__restrict__ xi, T *__restrict__ x, int nc, int b, int ncp) {
+__global__ void k_comp_unpad(const T *__restrict__ xi, T *__restrict__ x, int nc, int b, int ncp, const int *go) {
+    if (go && !*go) return;
     const long long total = (long long)b * nc;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total;
          i += (long long)gridDim.x * blockDim.x) {
@@ -751,14 +754,14 @@ static sts_status to_internal(sts_jac_s *h, const T *x, T *xi) {
 }
 
 template <typename T>
-static sts_status from_internal(sts_jac_s *h, const T *xi, T *x) {
+static sts_status from_internal(sts_jac_s *h, const T *xi, T *x, const int *go) {
     if (h->layout == STS_LAYOUT_CELL_MAJOR) {
         dim3 grid((h->nc + 31) / 32, (h->b + 31) / 32), block(32, 8);
-        k_comp_to_cell<T><<<grid, block, 0, h->stream>>>(xi, x, h->nc, h->b, h->ncp);
+        k_comp_to_cell<T><<<grid, block, 0, h->stream>>>(xi, x, h->nc, h->b, h->ncp, go);
         STS_LAUNCHED();
     } else {
         const long long n = (long long)h->b * h->nc;
-        k_comp_unpad<T><<<grid_for(n, 256), 256, 0, h->stream>>>(xi, x, h->nc, h->b, h->ncp);
+        k_comp_unpad<T><<<grid_for(n, 256), 256, 0, h->stream>>>(xi, x, h->nc, h->b, h->ncp, go);
         STS_LAUNCHED();
     }
     return STS_OK;
@@ -767,14 +770,16 @@ static sts_status from_internal(sts_jac_s *h, const T *xi, T *x) {
 // component-major [b][nc] to cell-major
 sts_status comp_to_cell64(sts_jac_s *h, const double *x, double *xc) {
     k_comp_to_cell<double><<<dim3((h->nc + 31) / 32, (h->b + 31) / 32), dim3(32, 8), 0, h->stream>>>(x, xc, h->nc, h->b,
-                                                                                                    h->nc);
+                                                                                                    h->nc, nullptr);
     STS_LAUNCHED();
     return STS_OK;
 }
 
 sts_status to_internal64(sts_jac_s *h, const double *x, double *xi) { return to_internal<double>(h, x, xi); }
-sts_status from_internal64(sts_jac_s *h, const double *xi, double *x) { return from_internal<double>(h, xi, x); }
+sts_status from_internal64(sts_jac_s *h, const double *xi, double *x, const int *go) {
+    return from_internal<double>(h, xi, x, go);
+}
 sts_status to_internal32(sts_jac_s *h, const float *x, float *xi) { return to_internal<float>(h, x, xi); }
-sts_status from_internal32(sts_jac_s *h, const float *xi, float *x) { return from_internal<float>(h, xi, x); }
+sts_status from_internal32(sts_jac_s *h, const float *xi, float *x) { return from_internal<float>(h, xi, x, nullptr); }
 
 }  // namespace sts

@@ -273,6 +273,7 @@ struct Krylov {
     int *gstate = nullptr;       // [2] steps taken, stop reason (1 criterion met, 2 NaN or Inf)
     double *grn = nullptr;       // squared norm of the residual after the cycle
     int *gerr = nullptr;         // the handle's error flag after the cycle
+    int *gdone = nullptr;        // the solve ends with this cycle, and x is its result
     double *gg = nullptr;        // [m+1] rotated right-hand side
     double *ghist = nullptr;     // [m] rotated residual / ||b|| per step
     double *gH = nullptr;        // [(m+1) * m] Hessenberg matrix, rotated in place
@@ -376,7 +377,7 @@ sts_status mv_dots64(sts_jac_s *h, int dir, const Vec<double> &x, double *c);   
 sts_status mv_apply64_noalloc(sts_jac_s *h, int dir, const Vec<double> &x, const Vec<double> &y);
 sts_status comp_to_cell64(sts_jac_s *h, const double *x, double *xc);
 sts_status to_internal64(sts_jac_s *h, const double *x, double *xi);
-sts_status from_internal64(sts_jac_s *h, const double *xi, double *x);
+sts_status from_internal64(sts_jac_s *h, const double *xi, double *x, const int *go = nullptr);     // go: device flag, 0: write nothing
 sts_status to_internal32(sts_jac_s *h, const float *x, float *xi);
 sts_status from_internal32(sts_jac_s *h, const float *xi, float *x);
 
