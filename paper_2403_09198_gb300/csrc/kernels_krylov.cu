@@ -159,7 +159,10 @@ __device__ __noinline__ void givens_step(const Givens &G, double hn2) {
         for (int i = x - 64; i <= j; i += 32) q = fma(G.h1[i], G.h1[i], q);
 #pragma unroll
         for (int k = 16; k >= 1; k /= 2) q += __shfl_xor_sync(0xffffffffu, q, k);
-        if (x == 64) w2 = q + hn2;
+        if (x == 64) {
+            w2 = q + hn2;
+            bad = !isfinite(w2);        // it tells a breakdown from an overflow
+        }
     } else if (x == 96) {
         hn = sqrt(hn2);
         G.par[2] = 1.0 / hn;

@@ -60,6 +60,18 @@ def test_x_stays_as_it_was_after_a_breakdown(vals, restart, graph, layout, on_ho
     jac.close()
 
 
+# ||w||^2 overflows where w itself is finite; in the first case w is a multiple of v_0, so
+# that what is left of it after the update is zero, in the second small
+@pytest.mark.parametrize("vals", [[1e200] * 4, [1e155, 1.0000001e155, 1e155, 1e155], [1e200, 2e200, 3e200, 5e200]])
+@pytest.mark.parametrize("graph", [True, False])
+def test_an_overflowing_norm_is_no_breakdown(vals, graph):
+    jac = _diagonal(vals)
+    st, x, info = _solve(jac, dev(np.ones(4)), dev(np.zeros(4)), restart=5, graph=graph)
+    assert st == STS_ERR_NUMERIC and info.iterations == 0
+    assert not x.any()
+    jac.close()
+
+
 @pytest.mark.parametrize("restart,max_iters", [(2, 1), (2, 2), (2, 3), (5, 200)])
 @pytest.mark.parametrize("graph", [True, False])
 def test_x_is_the_last_iterate_when_the_steps_run_out(restart, max_iters, graph):
