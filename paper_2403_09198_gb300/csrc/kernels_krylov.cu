@@ -760,7 +760,6 @@ sts_status gmres(sts_jac_s *h, const double *b_pub, double *x_pub, const sts_gmr
         // r = b - A x and its squared norm
         auto residual = [&](double *norm, const CycleEnd &end) -> sts_status {
             STS_TRY(opA64(h, dir, K.xb, K.w));
-            ++inf.matvecs;
             k_residual<<<orth_blocks(n, 0), kRedThreads, 0, h->stream>>>(K.r, K.bb, K.w, n, K.partial, norm, K.ticket,
                                                                          end);
             STS_LAUNCHED();
@@ -780,6 +779,7 @@ sts_status gmres(sts_jac_s *h, const double *b_pub, double *x_pub, const sts_gmr
                 beta_known = -1.0;
             } else {
                 STS_TRY(residual(K.red, CycleEnd{}));
+                ++inf.matvecs;
                 STS_CK(cudaMemcpyAsync(hp, K.red, sizeof(double), cudaMemcpyDeviceToHost, h->stream));
                 STS_CK(cudaStreamSynchronize(h->stream));
                 beta = std::sqrt(hp[0]);
@@ -848,7 +848,7 @@ sts_status gmres(sts_jac_s *h, const double *b_pub, double *x_pub, const sts_gmr
                 for (int i = 0; i < k; ++i)
                     if (d.history && its + i < max_iters) d.history[its + i] = ph[i];
                 its += k;
-                inf.matvecs += k;
+                inf.matvecs += k + 1;       // the steps' and the residual's
                 if (pre) inf.applies += k;
                 ++inf.restarts;
                 written = !d.vectors_on_host && *pd && *pe == 0;

@@ -72,6 +72,15 @@ def test_an_overflowing_norm_is_no_breakdown(vals, graph):
     jac.close()
 
 
+def test_a_broken_cycle_counts_no_product():
+    """A graph cycle that broke down adds neither steps nor products, the residual queued
+    behind it included."""
+    jac = _diagonal([1e200, 2e200, 3e200, 5e200])
+    st, _, info = _solve(jac, dev(np.ones(4)), dev(np.zeros(4)), restart=5)
+    assert st == STS_ERR_NUMERIC and (info.matvecs, info.iterations, info.restarts) == (0, 0, 0)
+    jac.close()
+
+
 @pytest.mark.parametrize("restart,max_iters", [(2, 1), (2, 2), (2, 3), (5, 200)])
 @pytest.mark.parametrize("graph", [True, False])
 def test_x_is_the_last_iterate_when_the_steps_run_out(restart, max_iters, graph):
