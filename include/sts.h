@@ -251,7 +251,9 @@ sts_status sts_jac_matvec_f32(sts_jac_t h, const float *x, float *y, int trans);
  * representation: per-cell dense LU with partial pivoting.  Synchronous.
  * Errors: STS_ERR_SINGULAR when a pivot fails |p| > 1e-14 * max|row of S_ii|, or
  * C_k is singular; the message names the first failing cell.  STS_ERR_TIMEOUT
- * when an apply since the last check reported a timed-out wait (see below).
+ * when an apply since the last check reported a timed-out wait (see below).  After
+ * either error the preconditioner is not set up (a timeout reported on a handle
+ * that was set up already leaves it so).
  */
 sts_status sts_jac_bjacobi_setup(sts_jac_t h);
 
@@ -324,6 +326,13 @@ sts_status sts_launch_count(unsigned long long *count);
  * stream (NULL: the legacy default stream).
  */
 sts_status sts_selftest_bounded_wait(void *stream);
+
+/*
+ * Self-test of the report (no paper counterpart): set the handle's flag from the
+ * host, as a kernel whose wait gave up sets it, so that the next sts_gmres_solve
+ * or sts_jac_bjacobi_setup reports STS_ERR_TIMEOUT.  Nothing waits.  Asynchronous.
+ */
+sts_status sts_selftest_wait_flag(sts_jac_t h);
 
 /* Destroy a handle and free its device memory.  NULL is accepted. */
 sts_status sts_jac_destroy(sts_jac_t h);

@@ -30,7 +30,7 @@ ABI_FUNCTIONS = ["sts_last_error", "sts_version", "sts_jac_create", "sts_jac_upd
                  "sts_jac_matvec", "sts_jac_matvec_noalloc", "sts_jac_matvec_f32", "sts_jac_bjacobi_setup",
                  "sts_jac_bjacobi_apply", "sts_jac_bjacobi_apply_f32", "sts_gmres_solve",
                  "sts_jac_grad", "sts_jac_memory", "sts_launch_count", "sts_selftest_bounded_wait",
-                 "sts_jac_destroy", "sts_flow_create", "sts_flow_get_sizes", "sts_flow_get_layout",
+                 "sts_selftest_wait_flag", "sts_jac_destroy", "sts_flow_create", "sts_flow_get_sizes", "sts_flow_get_layout",
                  "sts_flow_residual", "sts_flow_jacobian", "sts_flow_newton", "sts_flow_destroy",
                  "sts_dd_plan_create", "sts_dd_plan_sizes", "sts_dd_plan_get", "sts_dd_plan_value_sizes",
                  "sts_dd_plan_gather", "sts_dd_plan_destroy", "sts_dd_create", "sts_dd_matvec",
@@ -165,6 +165,7 @@ def load(path: str = LIB_PATH) -> ctypes.CDLL:
                 "sts_jac_memory": [P, ctypes.POINTER(ctypes.c_size_t)],
                 "sts_launch_count": [ctypes.POINTER(ctypes.c_ulonglong)],
                 "sts_selftest_bounded_wait": [P],
+                "sts_selftest_wait_flag": [P],
                 "sts_jac_destroy": [P],
                 "sts_flow_create": [ctypes.POINTER(sts_flow_desc), ctypes.POINTER(P)],
                 "sts_flow_get_sizes": [P, ctypes.POINTER(sts_flow_sizes)],

@@ -815,6 +815,13 @@ sts_status sts_selftest_bounded_wait(void *stream_) {
     return set_error(STS_ERR_TIMEOUT, "sts_selftest_bounded_wait: the bounded wait gave up as expected");
 }
 
+sts_status sts_selftest_wait_flag(sts_jac_t h) {
+    NvtxRange nvtx_range("sts_selftest_wait_flag");
+    if (!h) return set_error(STS_ERR_INVALID_ARG, "sts_selftest_wait_flag: handle is NULL");
+    STS_CK(cudaMemsetAsync(h->d_err, 1, sizeof(int), h->stream));
+    return STS_OK;
+}
+
 sts_status sts_launch_count(unsigned long long *count) {
     if (!count) return set_error(STS_ERR_INVALID_ARG, "sts_launch_count: count is NULL");
     *count = g_launches.load(std::memory_order_relaxed);

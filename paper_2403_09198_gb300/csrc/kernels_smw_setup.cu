@@ -757,6 +757,7 @@ inline int grid_for(long long n, int block) {
 
 sts_status smw_setup(sts_jac_s *h) {
     SmwPlan &M = h->smw;
+    const bool was_ready = M.ready;
     M.ready = false;
     SetupArgs a;
     a.Sd = M.Sd; a.Ud = M.Ud; a.Vd = M.Vd;
@@ -867,7 +868,8 @@ sts_status smw_setup(sts_jac_s *h) {
                          "block-Jacobi setup: cell %d has a pivot below 1e-14 x its row maximum "
                          "(static pivot order) or a singular capacitance matrix C_k", flags[1]);
     }
-    M.ready = true;
+    // a wait that gave up earlier is this call's error: what was not set up stays so
+    M.ready = was_ready || !flags[0];
     return report_wait(h, flags[0]);
 }
 
