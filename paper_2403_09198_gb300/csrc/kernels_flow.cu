@@ -266,7 +266,7 @@ enum { fUi, fUj,            // U of the first pair: ui q_i - uj q_j (both with d
        fU = fG + 4,         // flow components of the pairs: U [2][3], V [4][3]
        fV = fU + 6,
        fB = fV + 12,        // the neighbour block
-       fH = fB + kBlockFields,      // da/dq of q_j: G0, G1, G2
+       fH = fB + kBlockFields,      // da/dq of q_j: G0, G1, G2 (0 where q_j gives no wave speed)
        kFaceFields = fH + 3 };
 enum { cKap, cVT,           // source pair: kap beta_c, and its T component
        cB,                  // the diagonal block (without the band K and H's identity)
@@ -309,7 +309,8 @@ __global__ void __launch_bounds__(64) k_flow_face_jac(FlowDev F) {
         put(fU + 3 + e, dt * (cj[e] - ci[e]));
     }
     // V = (sR^k dsL - sL^k dsR) / den^2 (k = 1, 2) with dsL = n - da where this side
-    // gives s_L, dsR = n + da where it gives s_R: A n - G da, n along the velocities
+    // gives s_L, dsR = n + da where it gives s_R: A n - G da, n along the velocities.  A
+    // side that gives neither has V = 0 even where its da is no number (T <= 0)
     const double i2 = f.inv_den * f.inv_den;
     auto pair = [&](bool l, bool r, int s, double gT) {
         double A1 = 0.0, G1 = 0.0, A2 = 0.0, G2 = 0.0;
@@ -331,10 +332,10 @@ __global__ void __launch_bounds__(64) k_flow_face_jac(FlowDev F) {
         put(fG + s + 1, -G2);
         put(fV + 3 * s, A1 * nx);
         put(fV + 3 * s + 1, A1 * ny);
-        put(fV + 3 * s + 2, -G1 * gT);
+        put(fV + 3 * s + 2, l || r ? -G1 * gT : 0.0);
         put(fV + 3 * s + 3, A2 * nx);
         put(fV + 3 * s + 4, A2 * ny);
-        put(fV + 3 * s + 5, -G2 * gT);
+        put(fV + 3 * s + 5, l || r ? -G2 * gT : 0.0);
     };
     pair(f.iL == 1, f.iR == 1, 0, M[mGT * (size_t)nc + L.i]);
     pair(f.iL == 2, f.iR == 2, 2, M[mGT * (size_t)nc + L.j]);
@@ -346,7 +347,7 @@ __global__ void __launch_bounds__(64) k_flow_face_jac(FlowDev F) {
         for (int e = 0; e < 9; ++e) to[(bCorner + e) * stride] = B.corner[e / 3][e % 3];
     };
 #pragma unroll
-    for (int e = 0; e < 3; ++e) put(fH + e, M[(mG0 + e) * (size_t)nc + L.j]);
+    for (int e = 0; e < 3; ++e) put(fH + e, f.iL == 2 || f.iR == 2 ? M[(mG0 + e) * (size_t)nc + L.j] : 0.0);
     put_block(o + fB * 32, 32, block_coef(mj, dt * (wR * nx), dt * (wR * ny), dt * cf));
     // the diagonal block's face sum is A_n at the summed weighted normal
     const double sx = face_sum(L.on ? wL * nx : 0.0, lane, L.nf), sy = face_sum(L.on ? wL * ny : 0.0, lane, L.nf);
@@ -439,8 +440,12 @@ __global__ void __launch_bounds__(kFlowCells * 32) k_flow_jac(FlowDev F, const d
                 U[(pd + 1) * b + c] = u2;
                 U[po * b + c] = u1;
                 U[(po + 1) * b + c] = u2;
-                V[pd * b + c] = o[4 * fG] * ga;
-                V[(pd + 1) * b + c] = o[4 * fG + 4] * ga;
+                // q_i gives this face no wave speed where both its G are 0, and 0 times a da that
+                // is no number is none: a test of bits, not an FP64 comparison
+                const double G1 = o[4 * fG], G2 = o[4 * fG + 4];
+                const double gf = (__double2hiint(G1) | __double2hiint(G2)) << 1 ? ga : 0.0;
+                V[pd * b + c] = G1 * gf;
+                V[(pd + 1) * b + c] = G2 * gf;
                 V[po * b + c] = o[4 * fG + 8] * gj;
                 V[(po + 1) * b + c] = o[4 * fG + 12] * gj;
                 // the normal is along one axis: one momentum row is constant over the species

@@ -4,6 +4,7 @@ warp and the 32 of a mixture block, species about the 32 lanes, the largest bloc
 sides of a face.  Same oracle, scales and tolerance as tests/test_gpu_flow.py.
 """
 import numpy as np
+import numpy as np
 import pytest
 
 from oracle import flux
@@ -36,4 +37,26 @@ def test_edges(Lx, Ly, N, w, uniform):
         for key, got in zip("SUV", f.jacobian(dev(c.Q))):
             assert _scaled_err(host(got), ref[key], ref["scales"][key]) <= TOL_RES, key
         assert _res_err(R, m, c) <= TOL_RES
+    f.close()
+
+
+@pytest.mark.parametrize("T", [-0.7, 0.0])
+@pytest.mark.parametrize("Lx,Ly,N", [(6, 5, 7), (5, 4, 40)])
+def test_a_cell_without_a_sound_speed(T, Lx, Ly, N):
+    """A Newton iterate with T <= 0 in one cell: da/dq is no number there, but the cell gives
+    its faces no wave speed, so every entry that the model defines stays finite."""
+    c = inputs.make_flow_case(Lx, Ly, N=N, w=1, seed=3, dt=0.3)
+    c.Q[Lx + 2, N + 2] = T
+    m = flux.model_of(c)
+    with np.errstate(invalid="ignore", divide="ignore"):
+        ref = flux.jacobian_blocks(m, Lx, Ly, c.Q)
+    f = StsFlow(c)
+    for key, got in zip("SUV", f.jacobian(dev(c.Q))):
+        got, r, scale = host(got).ravel(), np.ravel(ref[key]), np.ravel(ref["scales"][key])
+        if key == "S":              # T < 0: the terms of an energy entry may cancel, its scale does not show them
+            scale = np.full_like(scale, scale.max())
+        on = np.isfinite(r)
+        assert on.sum() >= r.size - 1                    # T = 0: the source's kap / T^2 alone
+        assert np.array_equal(np.isfinite(got), on), key
+        assert _scaled_err(got[on], r[on], scale[on]) <= TOL_RES, key
     f.close()
