@@ -29,6 +29,7 @@
 #include <type_traits>
 #include <vector>
 
+#include "ring.cuh"
 #include "sts_internal.h"
 
 namespace sts {
@@ -84,6 +85,8 @@ __global__ void __launch_bounds__(128) k_flow_mix(FlowDev F, const double *Q, co
     extern __shared__ double rows[];             // [32][b | 1], species constants [N][4], partial sums [4][5][32]
     const int b = F.b, N = F.N, st = b | 1, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int c0 = blockIdx.x * kMixCells, n = min(kMixCells, F.nc - c0);
+    pdl_wait();
+    pdl_trigger();
     const double *src = (blockIdx.y ? Qn : Q) + (size_t)c0 * b;
     double *cst = rows + 32 * st;
     double(*part)[5][32] = reinterpret_cast<double(*)[5][32]>(cst + 4 * N);
@@ -286,6 +289,8 @@ __global__ void __launch_bounds__(64) k_flow_face_jac(FlowDev F) {
     const double dt = F.dt;
     const double *M = F.mix;
     const FaceLane L = face_lane(F, blk, lane);
+    pdl_wait();
+    pdl_trigger();
     const Mix mi = mix_of(M, nc, L.i), mj = mix_of(M, nc, L.j);
     double nx, ny;
     normal_of(F.Lx, L.i, L.j, nx, ny);
@@ -385,11 +390,6 @@ __global__ void __launch_bounds__(kFlowCells * 32) k_flow_jac(FlowDev F, const d
     const double *M = F.mix;
     const int i = blockIdx.x * kFlowCells + warp;
     if (i >= nc) return;
-    // this cell's coefficients: fc[field * 4 + face], cc[field]
-    double *fc = sh[warp], *cc = fc + kFaceFields * 4;
-    const double *gf = F.face + (size_t)blockIdx.x * kFaceFields * 32 + warp * 4;
-    for (int e = lane; e < kFaceFields * 4; e += 32) fc[e] = gf[(e >> 2) * 32 + (e & 3)];
-    if (lane < kCellFields) cc[lane] = F.cell[((size_t)blockIdx.x * kCellFields + lane) * kFlowCells + warp];
     const int k0 = F.bptr[i], nf = F.bptr[i + 1] - k0 - 1;
     // lane k of the row's at most five blocks
     const int col = lane <= nf ? F.bidx[k0 + lane] : -1;
@@ -400,6 +400,12 @@ __global__ void __launch_bounds__(kFlowCells * 32) k_flow_jac(FlowDev F, const d
         spo[warp][f] = F.pip[k0 + lane];
         sk[warp][f] = F.soff[k0 + lane];
     }
+    pdl_wait();
+    // this cell's coefficients: fc[field * 4 + face], cc[field]
+    double *fc = sh[warp], *cc = fc + kFaceFields * 4;
+    const double *gf = F.face + (size_t)blockIdx.x * kFaceFields * 32 + warp * 4;
+    for (int e = lane; e < kFaceFields * 4; e += 32) fc[e] = gf[(e >> 2) * 32 + (e & 3)];
+    if (lane < kCellFields) cc[lane] = F.cell[((size_t)blockIdx.x * kCellFields + lane) * kFlowCells + warp];
     __syncwarp();
     const double *qi = Q + (size_t)i * b;
     const double g0 = M[mG0 * (size_t)nc + i], g1 = M[mG1 * (size_t)nc + i], g2 = M[mG2 * (size_t)nc + i];
@@ -512,6 +518,8 @@ __global__ void __launch_bounds__(64) k_flow_face_res(FlowDev F, double *R) {
     if (blk * kFlowCells >= nc) return;
     const double *M = F.mix, *Mn = F.mix + (size_t)kMixFields * nc;
     const FaceLane L = face_lane(F, blk, lane);
+    pdl_wait();
+    pdl_trigger();
     const Mix mi = mix_of(M, nc, L.i), mj = mix_of(M, nc, L.j);
     double nx, ny;
     normal_of(F.Lx, L.i, L.j, nx, ny);
@@ -553,6 +561,7 @@ __global__ void __launch_bounds__(kFlowCells * 32) k_flow_res(FlowDev F, const d
         if (f < nf && F.bidx[k] == i) ++k;
         j[f] = f < nf ? F.bidx[k] : i;
     }
+    pdl_wait();
     const double *gf = F.face + (size_t)blockIdx.x * kFaceFields * 32 + warp * 4;
     const double *gc = F.cell + (size_t)blockIdx.x * kCellFields * kFlowCells + warp;
     double fb[4], fd[4];
@@ -656,22 +665,33 @@ sts_status flow_mix(sts_flow_s *f, const double *Q, const double *Qn) {
     return STS_OK;
 }
 
-sts_status flow_res(sts_flow_s *f, const double *Q, const double *Qn, double *R) {
-    STS_TRY(flow_mix(f, Q, Qn));
-    k_flow_face_res<<<(f->dev.nc + 2 * kFlowCells - 1) / (2 * kFlowCells), 64, 0, f->stream>>>(f->dev, R);
-    STS_LAUNCHED();
-    k_flow_res<<<(f->dev.nc + kFlowCells - 1) / kFlowCells, kFlowCells * 32, 0, f->stream>>>(f->dev, Q, Qn, R);
+// Launch a kernel that reads what the kernel before it has written, `cells` cells a block.
+// On small grids it is launched early (programmatic dependent launch): there the launches
+// set the time, and as three dependent ones the calls had become slower than the single
+// kernel they came from (a column of 200 cells, N = 20: residual 22.3, then 25.4, now
+// 20.7 us).  Early blocks take room from the kernel they wait for: a Jacobian of 32 x 32
+// cells (128 blocks) takes 38.6 and 39.0 us, of 48 x 48 47.8 and 54.8, of 24 x 24 (72) 39.1
+// and 33.8; so early below one block of the last kernel per two SMs.
+constexpr int kEarlyCells = 152 / 2 * kFlowCells;
+template <typename... KArgs, typename... Args>
+sts_status flow_next(sts_flow_s *f, void (*kern)(KArgs...), int cells, int threads, Args... args) {
+    const unsigned blocks = (f->dev.nc + cells - 1) / cells;
+    if (f->dev.nc < kEarlyCells) STS_CK(launch_pdl(kern, dim3(blocks), dim3(threads), 0, f->stream, args...));
+    else kern<<<blocks, threads, 0, f->stream>>>(args...);
     STS_LAUNCHED();
     return STS_OK;
 }
 
+sts_status flow_res(sts_flow_s *f, const double *Q, const double *Qn, double *R) {
+    STS_TRY(flow_mix(f, Q, Qn));
+    STS_TRY(flow_next(f, k_flow_face_res, 2 * kFlowCells, 64, f->dev, R));
+    return flow_next(f, k_flow_res, kFlowCells, kFlowCells * 32, f->dev, Q, Qn, R);
+}
+
 sts_status flow_jac(sts_flow_s *f, const double *Q, double *S, double *U, double *V) {
     STS_TRY(flow_mix(f, Q, nullptr));
-    k_flow_face_jac<<<(f->dev.nc + 2 * kFlowCells - 1) / (2 * kFlowCells), 64, 0, f->stream>>>(f->dev);
-    STS_LAUNCHED();
-    k_flow_jac<<<(f->dev.nc + kFlowCells - 1) / kFlowCells, kFlowCells * 32, 0, f->stream>>>(f->dev, Q, S, U, V);
-    STS_LAUNCHED();
-    return STS_OK;
+    STS_TRY(flow_next(f, k_flow_face_jac, 2 * kFlowCells, 64, f->dev));
+    return flow_next(f, k_flow_jac, kFlowCells, kFlowCells * 32, f->dev, Q, S, U, V);
 }
 
 // ||x||_2 of a device vector of the generator's stream (synchronous)

@@ -60,3 +60,23 @@ def test_a_cell_without_a_sound_speed(T, Lx, Ly, N):
         assert np.array_equal(np.isfinite(got), on), key
         assert _scaled_err(got[on], r[on], scale[on]) <= TOL_RES, key
     f.close()
+
+
+@pytest.mark.parametrize("Lx,Ly", [(1, 3), (101, 6), (1, 607), (1, 608), (1, 609)])
+def test_calls_behind_one_another(Lx, Ly):
+    """Kernels that start early, on both sides of the line: calls with two states in turn, each
+    of which overwrites the scalars that the one before it used, give what they give alone."""
+    c = inputs.make_flow_case(Lx, Ly, N=9, w=1, seed=5, dt=0.3)
+    f = StsFlow(c)
+    states = [dev(c.Q), dev(c.Qn)]
+    alone = []
+    for q, qn in (states, states[::-1]):
+        alone.append([host(t) for t in (f.residual(q, qn), *f.jacobian(q))])
+    got = []
+    for i in range(20):
+        q, qn = states[i % 2], states[1 - i % 2]
+        got.append((f.residual(q, qn), *f.jacobian(q)))
+    for i, g in enumerate(got):
+        for a, b in zip(g, alone[i % 2]):
+            assert np.array_equal(host(a), b)
+    f.close()
