@@ -146,10 +146,17 @@ __global__ void __launch_bounds__(128) k_dots(MvArgs<T> a) {
 // serially.  A chunk's values and operands are loaded one chunk ahead: an operand's
 // address comes out of its descriptor, so a load at its use is two memory latencies
 // per position.  With few tiles a group is one row and a warp's own instructions set
-// the time (41 x 37 cells, b = 33, 15% filled: 22 us, now 10).  Chunks of 8 there; FP64
-// grids of more warps than fit beside chunks of 8 take 4 (whole products, 128 / 800
-// tiles: 26 / 91 us, 30 / 98 with longer chunks; the products of 47 tiles 20.5 and 21.7).
-constexpr int kMainWarps = 20;      // resident warps per SM with chunks of 8
+// the time (41 x 37 cells, b = 33, 15% filled: 22 us, now 10): chunks of 8, and the group's
+// values are brought into L2 at once.  FP64 grids of more warps than fit beside chunks of 8
+// (114 registers) take chunks of 4 and leave that out: their resident warps' groups together
+// are more than L2 holds.  Whole FP64 products, in us, with chunks of 8 / of 4 (cold L2):
+//   b = 33, 15% filled: 8 tiles 14.4 / 14.5 (23.1 / 27.9), 32 18.5 / 18.5 (24.1 / 29.3), 53
+//     20.5 / 18.5 (27.0 / 29.3), 98 (19 warps per SM) 26.7 / 21.4, 162 28.8 / 26.7;
+//   b = 63, 10% filled: 32 tiles 22.9 / 21.6 (31.4 / 33.4), 128 (17) 47.0 / 37.0.
+// Chunks of 4 that bring the values in / as here / one position at a time:
+//   b = 33: 288 tiles 42.5 / 40.0 / 41.1, 512 67.9 / 63.6 / 74.4, 800 90.8 / 86.1 / 103.3;
+//   b = 63: 288 tiles 90.4 / 81.1 / 87.4, 392 107.7 / 88.0 / 94.3, 704 172.5 / 136.1 / 181.2.
+constexpr int kMainWarps = 16;      // resident warps per SM with chunks of 8
 template <typename T, int CH>
 __global__ void __launch_bounds__(128) k_mv_main(MvArgs<T> a) {
     __shared__ int snb[4][kMaxSlots][kTile];
@@ -161,15 +168,19 @@ __global__ void __launch_bounds__(128) k_mv_main(MvArgs<T> a) {
     const int p0 = grp.x, L = grp.y;
     const long long q0 = (long long)(unsigned)grp.z | ((long long)grp.w << 32);
     const T *__restrict__ sv = a.main + ((size_t)t * a.tile_len + q0) * kTile + lane;
-    if (lane == 0) prefetch_l2_bulk(sv, (unsigned)L * kTile * (unsigned)sizeof(T));
+    if (CH == 8 && lane == 0) prefetch_l2_bulk(sv, (unsigned)L * kTile * (unsigned)sizeof(T));
     const int *__restrict__ nb = a.nbr + (size_t)t * a.n_slots * kTile + lane;
-    // offset of a slot's cell in x; complemented where the neighbour is absent, whose own cell
-    // is read and not used.  Offsets fit 32 bits: a vector has fewer than 2^31 values
+    // offset of a slot's cell in x, or -1 where the neighbour is absent: its operand is 0.
+    // FP64 in chunks of 8 complements the own cell's offset there, which is read and not used:
+    // the loads that a test switches off cost a warp on its own more than the operand's
+    // selection (256 and 576 cells, b = 33: 14.4 and 16.4 us), with more warps less (cell
+    // count 25600: 90.3 and 86.2).  Offsets fit 32 bits: a vector has fewer than 2^31 values
+    constexpr bool BITS = CH == 8 && sizeof(T) == 8;
     const int own = min(t * kTile + lane, a.x.cells - 1), xc = (int)a.x.sc, xq = (int)a.x.sq;
 #pragma unroll 8
     for (int s = 0; s < a.n_slots; ++s) {
         const int j = __ldg(nb + s * kTile);
-        snb[wib][s][lane] = j >= 0 ? j * xc : ~(own * xc);
+        snb[wib][s][lane] = j >= 0 ? j * xc : BITS ? ~(own * xc) : -1;
     }
     __syncwarp();
     const unsigned *__restrict__ dd = a.desc + q0;
@@ -196,8 +207,11 @@ __global__ void __launch_bounds__(128) k_mv_main(MvArgs<T> a) {
         for (int i = 0; i < CH; ++i) {
             const int k = (int)(dn[i] & 0xffffu), off = snb[wib][(dn[i] >> 16) & 0x1fu][lane];
             const bool pair = dn[i] & kDescPair;
-            gone_n |= !pair && off < 0 ? 1u << i : 0u;
-            on[i] = __ldg((pair ? cc : xp) + (pair ? (unsigned)(k * kTile) : (unsigned)k * (unsigned)xq + (unsigned)(off >= 0 ? off : ~off)));
+            if (BITS) gone_n |= !pair && off < 0 ? 1u << i : 0u;
+            const T *from = (pair ? cc : xp) + (pair ? (unsigned)(k * kTile)
+                                                     : (unsigned)k * (unsigned)xq + (unsigned)(!BITS || off >= 0 ? off : ~off));
+            on[i] = T(0);
+            if (BITS || off >= 0) on[i] = __ldg(from);      // a pair's descriptor names slot 0, the own cell
         }
         fetch_desc(base + CH);
     };
@@ -216,7 +230,7 @@ __global__ void __launch_bounds__(128) k_mv_main(MvArgs<T> a) {
 #pragma unroll
         for (int i = 0; i < CH; ++i) {
             if (base + i >= L) break;
-            acc = fma(v[i], gone >> i & 1u ? T(0) : o[i], acc);
+            acc = fma(v[i], BITS && (gone >> i & 1u) ? T(0) : o[i], acc);
             if (d[i] & kDescEnd) {
                 *yp = acc;
                 yp += ystep;
