@@ -26,10 +26,9 @@ namespace sts {
 namespace {
 
 template <typename T>
-struct MvArgs {
+struct MvBase {
     const T *main;          // [n_tiles][tile_len][32]
     const T *dotv;          // [n_tiles][n_dtasks][Lp][32]
-    Vec<T> x, y;
     T *c;                   // [n_tiles][n_dtasks][32]
     int *err;               // set when a bounded wait gave up
     unsigned *sched;        // [2] pass-2 item counter and finished warps, zero between launches
@@ -38,13 +37,27 @@ struct MvArgs {
     const unsigned *slot_mask;
     const int4 *grp;        // [n_groups] generic main pass: first row, positions, first position
     const int *dtask_slot;  // [n_dtasks]
-    const int *pat_ptr;     // [2][b+1]
-    const int *pat_idx;
     const unsigned *desc;   // [tile_len] program of the generic main pass
     long long tile_len;
-    int n_tiles, n_slots, n_pslots, n_dtasks, Lp, n_groups, b, ncp, nnz_d;
+    int n_tiles, n_slots, n_pslots, n_dtasks, Lp, n_groups, b, ncp;
     int sN, s_rl, s_gl, n_lgroups, wd, structured;   // structured layout (see MvPlan)
 };
+// INT: x and y are in the internal layout, the common case.  Without the strides (and
+// without three fields that no kernel read) the FP32 products take, in us, 128 x 128 cells,
+// N = 60: 38.2 -> 37.4, 64 x 64: 15.3 -> 14.5, 96 x 96, N = 100: 39.1 -> 37.1; FP64 the same
+// (98.1, 31.7, 100.6; 96 x 96, N = 30 47.3 -> 47.6).
+template <typename T, bool INT = false>
+struct MvArgs : MvBase<T> {
+    std::conditional_t<INT, Bare<T>, Vec<T>> x, y;
+};
+template <typename T>
+MvArgs<T, true> bare(const MvArgs<T> &a) {
+    MvArgs<T, true> r;
+    static_cast<MvBase<T> &>(r) = a;
+    r.x.p = a.x.p;
+    r.y.p = a.y.p;
+    return r;
+}
 
 // Chunk of stream positions held in registers (two chunks in flight per lane).
 // FP64: 4 positions measured faster than 8 (100.6 against 102.2 us per matvec
@@ -81,7 +94,7 @@ __device__ __forceinline__ float dot_el(const float4 &v, int i) { return vel(v, 
 // INT: x is in the internal layout, the common case: its addresses then cost a warp,
 // whose 63 FMAs at N = 60 are soon done, about 1% less.
 template <typename T, bool INT>
-__global__ void __launch_bounds__(128) k_dots(MvArgs<T> a) {
+__global__ void __launch_bounds__(128) k_dots(MvArgs<T, INT> a) {
     using V = typename DotVec<T>::type;
     constexpr int CH = Chunk<T>::CH;
     constexpr int VEC = DotVec<T>::n, NV = CH / VEC;
@@ -109,7 +122,9 @@ __global__ void __launch_bounds__(128) k_dots(MvArgs<T> a) {
         // an absent neighbour reads the lane's own cell: its coefficients are zero
         const T *__restrict__ xj = a.x.template cell<INT>(j >= 0 ? j : t * kTile + lane);
         const int bm1 = a.b - 1;
-        const size_t sq = INT ? (size_t)a.ncp : (size_t)a.x.sq;
+        size_t sq;
+        if constexpr (INT) sq = (size_t)a.ncp;
+        else sq = (size_t)a.x.sq;
         if (!a.pre) {
 #pragma unroll
             for (int i = 0; i < NV; ++i) va[i] = __ldcs(dv + i * kTile);
@@ -268,14 +283,20 @@ __host__ __device__ inline size_t mv_struct_warp_bytes(int rl, int elem) {
 }
 
 template <typename T, int WD, int NREG, bool INT>
-__global__ void __launch_bounds__(64) k_mv_struct(MvArgs<T> a) {
+__global__ void __launch_bounds__(64) k_mv_struct(MvArgs<T, INT> a) {
     static_assert(NREG == 0 || NREG == 8 || NREG == 2 * kStructDuff, "register pair slots");
     constexpr int NF = kStructNF;
     constexpr int NS = kStructMaxSlots;
     constexpr int BANDW = 2 * WD + 1;
     const int lane = threadIdx.x & 31;
     const int ns = a.n_slots, nps = a.n_pslots, N = a.sN;
-    const size_t sq = INT ? (size_t)a.ncp : (size_t)a.x.sq, ysq = INT ? sq : (size_t)a.y.sq;
+    size_t sq, ysq;
+    if constexpr (INT) sq = ysq = (size_t)a.ncp;
+    else sq = (size_t)a.x.sq, ysq = (size_t)a.y.sq;
+    auto written = [&](int c) {             // padding lanes of a vector in place write nothing
+        if constexpr (INT) return true;
+        else return c < a.y.cells;
+    };
     const int RL = a.s_rl;
     const uint32_t row_bytes = (uint32_t)RL * kTile * (uint32_t)sizeof(T);
     extern __shared__ __align__(128) unsigned char mv_smem[];
@@ -330,7 +351,7 @@ __global__ void __launch_bounds__(64) k_mv_struct(MvArgs<T> a) {
             for (int s = 0; s < ns; ++s) acc += __ldg(cc + (size_t)(nps + f * ns + s) * kTile);
             for (int k = 0; k < nps; ++k)
                 acc = fma(__ldg(su + (size_t)(f * nps + k) * kTile), __ldg(cc + (size_t)k * kTile), acc);
-            if (INT || cell < a.y.cells) a.y.template cell<INT>(cell)[(size_t)(N + f) * ysq] = acc;
+            if (written(cell)) a.y.template cell<INT>(cell)[(size_t)(N + f) * ysq] = acc;
         }
         continue;
     }
@@ -379,7 +400,7 @@ __global__ void __launch_bounds__(64) k_mv_struct(MvArgs<T> a) {
 #pragma unroll
     for (int s = 1; s < NS; ++s) xn[s] = s < ns ? __ldg(xs[s] + (size_t)p0 * sq) : T(0);
     T *yp = a.y.template cell<INT>(cell) + (size_t)p0 * ysq;
-    const bool on = INT || cell < a.y.cells;
+    const bool on = written(cell);
     T ylag = T(0);          // row p-1's result, stored during row p (its FMA has long completed)
     for (int p = p0; p < p1; ++p) {
         const int sg = (p - p0) & 1;
@@ -567,8 +588,6 @@ MvArgs<T> make_args(sts_jac_s *h, int dir, const T *main, const T *dotv, const V
     a.slot_mask = P.slot_mask;
     a.grp = P.grp;
     a.dtask_slot = P.dtask_slot;
-    a.pat_ptr = P.pat_ptr;
-    a.pat_idx = P.pat_idx;
     a.desc = P.desc;
     a.tile_len = P.tile_len;
     a.n_tiles = h->n_tiles;
@@ -579,7 +598,6 @@ MvArgs<T> make_args(sts_jac_s *h, int dir, const T *main, const T *dotv, const V
     a.n_groups = P.n_groups;
     a.b = h->b;
     a.ncp = h->ncp;
-    a.nnz_d = h->nnz_d;
     a.sN = P.sN;
     a.s_rl = P.s_rl;
     a.s_gl = P.s_gl;
@@ -593,21 +611,24 @@ template <typename T>
 sts_status dots_launch(sts_jac_s *h, const MvArgs<T> &a) {
     if (a.n_dtasks == 0) return STS_OK;
     const long long warps = (long long)a.n_tiles * a.n_dtasks;
-    const auto kern = a.x.internal(a.ncp) ? k_dots<T, true> : k_dots<T, false>;
-    kern<<<(unsigned)((warps + 3) / 4), 128, 0, h->stream>>>(a);
+    const unsigned grid = (unsigned)((warps + 3) / 4);
+    if (a.x.internal(a.ncp)) k_dots<T, true><<<grid, 128, 0, h->stream>>>(bare(a));
+    else k_dots<T, false><<<grid, 128, 0, h->stream>>>(a);
     STS_LAUNCHED();
     h->streams_dirty = false;
     return STS_OK;
 }
 
 template <typename T, int WD, bool INT>
-void (*mv_struct_kernel_of(int nreg))(MvArgs<T>) {
+void (*mv_struct_kernel(int nreg))(MvArgs<T, INT>) {
     return nreg == 8 ? k_mv_struct<T, WD, 8, INT> : nreg ? k_mv_struct<T, WD, 2 * kStructDuff, INT>
                                                           : k_mv_struct<T, WD, 0, INT>;
 }
-template <typename T, int WD>
-void (*mv_struct_kernel(int nreg, bool internal))(MvArgs<T>) {
-    return internal ? mv_struct_kernel_of<T, WD, true>(nreg) : mv_struct_kernel_of<T, WD, false>(nreg);
+template <typename T, bool INT>
+void (*mv_struct_kernel(int wd, int nreg))(MvArgs<T, INT>) {
+    return wd == 0 ? mv_struct_kernel<T, 0, INT>(nreg) : wd == 1 ? mv_struct_kernel<T, 1, INT>(nreg)
+           : wd == 2 ? mv_struct_kernel<T, 2, INT>(nreg) : wd == 3 ? mv_struct_kernel<T, 3, INT>(nreg)
+                                                         : mv_struct_kernel<T, 4, INT>(nreg);
 }
 
 // Level rows per pass-2 item.  The persistent grid runs n_tiles x (groups + 1)
@@ -643,28 +664,23 @@ sts_status mv_launch(sts_jac_s *h, const MvArgs<T> &args) {
     if (a.structured) {
         constexpr int kWarpsPerBlock = 2;      // two row stages per warp; small blocks pack the SM finely
         const size_t smem = (size_t)kWarpsPerBlock * mv_struct_warp_bytes(a.s_rl, (int)sizeof(T));
-        void (*kern)(MvArgs<T>) = nullptr;
         const int nreg = a.n_pslots <= 8 ? 8 : a.n_pslots <= 2 * kStructDuff ? 2 * kStructDuff : 0;
         const bool in = a.x.internal(a.ncp) && a.y.internal(a.ncp);
-        switch (a.wd) {
-            case 0: kern = mv_struct_kernel<T, 0>(nreg, in); break;
-            case 1: kern = mv_struct_kernel<T, 1>(nreg, in); break;
-            case 2: kern = mv_struct_kernel<T, 2>(nreg, in); break;
-            case 3: kern = mv_struct_kernel<T, 3>(nreg, in); break;
-            default: kern = mv_struct_kernel<T, 4>(nreg, in); break;
-        }
+        const auto kern_in = mv_struct_kernel<T, true>(a.wd, nreg);
+        const auto kern_at = mv_struct_kernel<T, false>(a.wd, nreg);
+        const void *kern = in ? reinterpret_cast<const void *>(kern_in) : reinterpret_cast<const void *>(kern_at);
         // blocks resident at once, found once per kernel instance and shared-memory
         // size: the instance (pair slots) and the row length differ between the
         // forward and transposed plans
         int resident = 0;
         for (const auto &e : h->mvs_resident)
-            if (e.kern == reinterpret_cast<const void *>(kern) && e.smem == smem) resident = e.blocks;
+            if (e.kern == kern && e.smem == smem) resident = e.blocks;
         if (!resident) {
-            if (smem > 48 * 1024) STS_CK(allow_all_smem(kern));
+            if (smem > 48 * 1024) STS_CK(in ? allow_all_smem(kern_in) : allow_all_smem(kern_at));
             int per_sm = 0;
             STS_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kWarpsPerBlock * kTile, smem));
             resident = std::max(per_sm, 1) * h->nsm;
-            h->mvs_resident.push_back({reinterpret_cast<const void *>(kern), smem, resident});
+            h->mvs_resident.push_back({kern, smem, resident});
         }
         a.s_gl = pass2_group_rows(a.sN, a.n_tiles, (long long)resident * kWarpsPerBlock, a.s_gl, a.s_rl,
                                  sizeof(T) == 8);
@@ -676,7 +692,9 @@ sts_status mv_launch(sts_jac_s *h, const MvArgs<T> &args) {
         // programmatic dependent launch: the blocks start, and copy their first
         // rows, while pass 1 finishes; items are taken from a counter, so
         // blocks that start late do not finish late
-        STS_CK(launch_pdl(kern, dim3((unsigned)blocks), dim3(kWarpsPerBlock * kTile), smem, h->stream, a));
+        const dim3 persistent((unsigned)blocks), block(kWarpsPerBlock * kTile);
+        if (in) STS_CK(launch_pdl(kern_in, persistent, block, smem, h->stream, bare(a)));
+        else STS_CK(launch_pdl(kern_at, persistent, block, smem, h->stream, a));
     } else {
         const bool full = sizeof(T) == 8 && warps > (long long)kMainWarps * h->nsm;
         (full ? k_mv_main<T, sizeof(T) == 8 ? 4 : 8> : k_mv_main<T, 8>)<<<grid, 128, 0, h->stream>>>(a);

@@ -137,6 +137,16 @@ struct Vec {
     }
 };
 
+// A vector known to be in the internal layout, by its address alone: kernels that take it
+// so get no strides as arguments.  (Unused fields among a kernel's arguments are not free:
+// they move the others, and with them the registers that ptxas finds; figures at MvArgs.)
+template <typename T>
+struct Bare {
+    T *p;
+    template <bool INT>
+    __device__ __forceinline__ T *cell(int c) const { return p + c; }
+};
+
 // Device allocation tracked by the handle.
 struct DevBuf {
     void *p = nullptr;
