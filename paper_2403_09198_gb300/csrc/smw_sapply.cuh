@@ -51,11 +51,11 @@ namespace {
 // whole chunks, so one tile's stream is Lt contiguous positions stored as
 // [tile][position / VEC][lane][VEC]: a chunk is one bulk copy and a lane reads
 // VEC positions with one 16-byte shared-memory load.
-template <typename T>
+template <typename T, bool BARE>
 struct SApplyArgs {
     const T *st;            // [n_tiles][Lt / VEC][32][VEC]
     const double *Cinv;     // [r][r][ncp] (instances that do not fold only)
-    Vec<T> x, y;            // internal layout where the working vector lives in y
+    std::conditional_t<BARE, Bare<T>, Vec<T>> x, y;     // internal layout where the working vector lives in y
     int *err;               // set when a bounded wait gave up
     int Lt, b, N, r, ncp, trans, n_tiles;
     int pre;                // the stream and C^-1 may be read before the grid-dependency wait
@@ -126,9 +126,13 @@ __host__ __device__ inline size_t sap_warp_bytes(int b, int elem) {
 //
 // INT: the vectors are in the internal layout (GW always is), whose addresses the FP32
 // kernel, bound by its instructions, cannot spare (11.2 against 12.8 us through strides on
-// 128 x 128 cells, N = 60).
+// 128 x 128 cells, N = 60).  FP32 and GW instances on it do without the strides as arguments,
+// too: unused, they still cost 2-6% (96 x 96 cells: N = 30 FP32 7.07 -> 7.33 us, N = 100
+// FP64 in y 90.8 -> 96.2); FP64 in shared memory is as fast or faster beside them (W = 2,
+// two pairs 44.5 against 45.1 us, 248 registers against 255).
+__host__ __device__ constexpr bool sap_bare(int elem, bool gw, bool in) { return gw || (in && elem == 4); }
 template <typename T, int W, int RMAX, bool GW, bool INT>
-__global__ void __launch_bounds__((kApWarps + 1) * 32) k_smw_sapply(SApplyArgs<T> a) {
+__global__ void __launch_bounds__((kApWarps + 1) * 32) k_smw_sapply(SApplyArgs<T, sap_bare((int)sizeof(T), GW, INT)> a) {
     static_assert(INT || !GW, "the working vector in y needs the internal layout");
     constexpr int NF = kStructNF, VEC = 16 / (int)sizeof(T);
     constexpr int K = kSApChunkBytes / (kTile * (int)sizeof(T));
@@ -232,7 +236,8 @@ __global__ void __launch_bounds__((kApWarps + 1) * 32) k_smw_sapply(SApplyArgs<T
                           (uint32_t)(kTile * sizeof(T)), xbar);
     } else if constexpr (!GW) {
         const T *x0 = a.x.template cell<INT>(gw * kTile + lane);
-        const size_t xq = INT ? P : (size_t)a.x.sq;
+        size_t xq = P;
+        if constexpr (!INT) xq = (size_t)a.x.sq;
         for (int i = 0; i < b; ++i) cp_async_elem(wl + i * kTile, x0 + (size_t)i * xq);
         cp_async_commit();
     }
@@ -367,11 +372,16 @@ __global__ void __launch_bounds__((kApWarps + 1) * 32) k_smw_sapply(SApplyArgs<T
                     z[i] = (T)sacc;
                 }
             }
-            const T *xn = INT ? a.x.p + (size_t)cell + (size_t)nw * kTile : a.x.at(cell + nw * kTile);
-            const size_t sq = INT ? P : (size_t)a.x.sq;         // of x and of y
-            // padding lanes of a vector in place write nothing
-            const bool on = INT || cell < a.y.cells;
-            T *y = INT ? a.y.p + cell : a.y.p + (size_t)cell * (size_t)a.y.sc;
+            const T *xn = a.x.p + (size_t)cell + (size_t)nw * kTile;
+            T *y = a.y.p + cell;
+            size_t sq = P;                  // of x and of y
+            bool on = true;                 // padding lanes of a vector in place write nothing
+            if constexpr (!INT) {
+                xn = a.x.at(cell + nw * kTile);
+                y = a.y.p + (size_t)cell * (size_t)a.y.sc;
+                sq = (size_t)a.x.sq;
+                on = cell < a.y.cells;
+            }
             // the next tile's x is copied in one group of rows at a time, at
             // the group's last row (all its rows have been read by then): a
             // test of the runtime flag on every row measured about 25 cycles
@@ -416,21 +426,21 @@ fail:
 inline bool sap_in_y(int b, int elem) { return (size_t)(227 * 1024) / sap_warp_bytes(b, elem) < (size_t)kApWarps; }
 
 template <typename T, int W, bool GW, bool INT>
-void (*sap_kernel_of(int rmax))(SApplyArgs<T>) {
+void (*sap_kernel_of(int rmax))(SApplyArgs<T, sap_bare((int)sizeof(T), GW, INT)>) {
     return rmax == 2 ? k_smw_sapply<T, W, 2, GW, INT> : rmax == 4 ? k_smw_sapply<T, W, 4, GW, INT>
                                                                    : k_smw_sapply<T, W, sap_rmax_big(W), GW, INT>;
 }
-template <typename T, int W>
-void (*sap_kernel(int rmax, bool gw, bool internal))(SApplyArgs<T>) {
-    return gw ? sap_kernel_of<T, W, true, true>(rmax) : internal ? sap_kernel_of<T, W, false, true>(rmax)
-                                                                  : sap_kernel_of<T, W, false, false>(rmax);
+template <typename T, bool GW, bool INT>
+auto sap_kernel(int w, int rmax) {
+    return w == 0 ? sap_kernel_of<T, 0, GW, INT>(rmax) : w == 1 ? sap_kernel_of<T, 1, GW, INT>(rmax)
+           : w == 2 ? sap_kernel_of<T, 2, GW, INT>(rmax) : w == 3 ? sap_kernel_of<T, 3, GW, INT>(rmax)
+                                                                 : sap_kernel_of<T, 4, GW, INT>(rmax);
 }
-
 
 template <typename T>
 sts_status smw_sapply_t(sts_jac_s *h, int dir, const T *st, const Vec<T> &x, const Vec<T> &z) {
     const SmwPlan &M = h->smw;
-    SApplyArgs<T> a;
+    SApplyArgs<T, false> a;
     a.st = st; a.Cinv = M.Cinv; a.x = x; a.y = z; a.err = h->d_err;
     a.Lt = M.s_lt[sizeof(T) == 8 ? 0 : 1]; a.b = h->b; a.N = h->b - kStructNF; a.r = h->r_diag; a.ncp = h->ncp;
     a.trans = dir; a.n_tiles = h->n_tiles;
@@ -444,21 +454,22 @@ sts_status smw_sapply_t(sts_jac_s *h, int dir, const T *st, const Vec<T> &x, con
     if (wpb < 1)
         return set_error(STS_ERR_INVALID_ARG, "block size %d needs %zu bytes of shared memory per warp", h->b, per_warp);
     const size_t smem = (size_t)wpb * per_warp;
-    void (*kern)(SApplyArgs<T>) = nullptr;
     const int rm = sap_rmax(h->r_diag, M.s_w);
-    switch (M.s_w) {
-        case 0: kern = sap_kernel<T, 0>(rm, gw, in); break;
-        case 1: kern = sap_kernel<T, 1>(rm, gw, in); break;
-        case 2: kern = sap_kernel<T, 2>(rm, gw, in); break;
-        case 3: kern = sap_kernel<T, 3>(rm, gw, in); break;
-        default: kern = sap_kernel<T, 4>(rm, gw, in); break;
-    }
     bool &attr = h->sap_attr[sizeof(T) == 8 ? 0 : 1][in ? 1 : 0];
-    if (!attr && smem > 48 * 1024) STS_CK(allow_all_smem(kern));
-    attr = true;
     const int blocks = std::max(1, std::min(h->nsm, (h->n_tiles + wpb - 1) / wpb));
-    STS_CK(launch_pdl(kern, dim3(blocks), dim3((wpb + 1) * kTile), smem, h->stream, a));
-    STS_LAUNCHED();
+    auto launch = [&](auto kern, const auto &args) -> sts_status {
+        if (!attr && smem > 48 * 1024) STS_CK(allow_all_smem(kern));
+        attr = true;
+        STS_CK(launch_pdl(kern, dim3(blocks), dim3((wpb + 1) * kTile), smem, h->stream, args));
+        STS_LAUNCHED();
+        return STS_OK;
+    };
+    const SApplyArgs<T, true> bare{a.st, a.Cinv, {a.x.p}, {a.y.p}, a.err, a.Lt, a.b, a.N, a.r, a.ncp, a.trans,
+                                   a.n_tiles, a.pre, a.evict_first, a.bulk};
+    if (gw) STS_TRY(launch(sap_kernel<T, true, true>(M.s_w, rm), bare));
+    else if (!in) STS_TRY(launch(sap_kernel<T, false, false>(M.s_w, rm), a));
+    else if constexpr (sap_bare((int)sizeof(T), false, true)) STS_TRY(launch(sap_kernel<T, false, true>(M.s_w, rm), bare));
+    else STS_TRY(launch(sap_kernel<T, false, true>(M.s_w, rm), a));
     h->streams_dirty = false;
     return STS_OK;
 }
