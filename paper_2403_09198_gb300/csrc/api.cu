@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <climits>
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
@@ -593,15 +594,18 @@ sts_status create_impl(const sts_jac_desc *d, sts_jac_t *out) {
 // cell-major vector is a sector of its own: one write per row hides behind the FP64 pipe
 // and merges in L2, but a product reads its operand about 25 times, against the launch
 // that a transpose takes.  Measured on cell-major vectors, us per call:
-//   apply, both vectors transposed and in place, N = 10: 18.6 and 10.5 at 2 tiles of 32
-//     cells, 30.9 and 19.9 at 1152; N = 60: 51.4 and 42.3 at 2, 104.8 and 90.0 at 1152: always;
+//   apply, both vectors transposed and in place, FP64: N = 10 17.5 and 9.7 at 2 tiles of 32
+//     cells, 30.9 and 19.7 at 1152, 166.4 and 128.2 at 8192; N = 60: 51.2 and 42.3 at 2, 106.6
+//     and 89.8 at 1152, 201.5 and 174.6 at 2048; FP32: N = 10 12.3 and 3.9 at 2, 78.1 and 44.6
+//     at 8192; N = 60 18.5 and 12.0 at 2, 22.6 and 15.8 at 512, 72.7 and 58.8 at 2048; N = 100
+//     26.5 and 23.7 at 128, 64.9 and 52.5 at 1152: always (it reads its operand once);
 //   matvec, both vectors transposed and x alone, N = 60: 112.7 and 106.7 at 512 tiles, 384.3
 //     and 371.9 at 2048; N = 200 at 512 tiles 350.6 and 337.9; FP32 52.8 and 49.4 (N = 60, 512);
 //   matvec, x transposed and in place, FP64: N = 60 20.6 and 14.5 at 4 K values, 39.0 and 39.0
 //     at 258 K, 66.1 and 69.7 at 488 K; N = 20 38.9 and 39.0 at 212 K, 63.4 and 67.2 at 451 K;
 //     N = 10 36.9 and 34.7 at 213 K.  FP32, where no pipe hides the reads: N = 60 14.8 and
 //     12.3 at 16 K, 16.4 and 18.5 at 36 K; N = 20 16.4 and 14.8 at 24 K, 22.8 and 25.7 at 212 K.
-constexpr long long kMatvecDirect = 1 << 18, kMatvecDirect32 = 1 << 15, kApplyDirect = 1LL << 62;
+constexpr long long kMatvecDirect = 1 << 18, kMatvecDirect32 = 1 << 15, kAlways = LLONG_MAX;
 
 template <typename T, typename F>
 sts_status with_layout(sts_jac_s *h, bool any_layout, long long direct_max, const T *x, T *y, T *bin, T *bout, F op) {
@@ -756,7 +760,7 @@ sts_status sts_jac_bjacobi_apply(sts_jac_t h, const double *x, double *z, int tr
         return set_error(STS_ERR_INVALID_ARG, "sts_jac_bjacobi_apply: trans = 1 needs enable_transpose");
     const int dir = trans ? 1 : 0;
     const bool fact = h->rep == STS_REP_FACTORED;
-    STS_GUARD(return with_layout<double>(h, fact && smw_apply_any_layout(h, 8), kApplyDirect, x, z, h->vin, h->vout,
+    STS_GUARD(return with_layout<double>(h, fact && smw_apply_any_layout(h, 8), kAlways, x, z, h->vin, h->vout,
                                          [&](const Vec<double> &a, const Vec<double> &b) {
         return fact ? smw_apply64(h, dir, a, b) : op_apply64(h, dir, a.p, b.p);
     });)
@@ -769,7 +773,7 @@ sts_status sts_jac_bjacobi_apply_f32(sts_jac_t h, const float *x, float *z, int 
     if (!h->smw.ready) return set_error(STS_ERR_NOT_SETUP, "sts_jac_bjacobi_apply_f32: call sts_jac_bjacobi_setup first");
     if (trans && !h->has_T) return set_error(STS_ERR_INVALID_ARG, "sts_jac_bjacobi_apply_f32: no transposed operators");
     const int dir = trans ? 1 : 0;
-    STS_GUARD(return with_layout<float>(h, smw_apply_any_layout(h, 4), kApplyDirect, x, z, h->vin32, h->vout32,
+    STS_GUARD(return with_layout<float>(h, smw_apply_any_layout(h, 4), kAlways, x, z, h->vin32, h->vout32,
                                         [&](const Vec<float> &a, const Vec<float> &b) {
         return smw_apply32(h, dir, a, b);
     });)

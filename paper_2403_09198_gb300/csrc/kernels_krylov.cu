@@ -274,15 +274,17 @@ using OrthKernel = void (*)(double *, const double *, long long, const double *,
                             unsigned int *, Givens);
 template <int MODE, int... I>
 OrthKernel orth_kernel(int cnt, std::integer_sequence<int, I...>) {
-    static const OrthKernel k[] = {k_orth<I, MODE>...};
-    return k[cnt];
+    // kDots without vectors is the norm; the other modes have at least one
+    constexpr int least = MODE == kDots ? 0 : 1;
+    static const OrthKernel k[] = {k_orth<I + least, MODE>...};
+    return k[cnt - least];
 }
 
 sts_status orth_launch(int mode, int cnt, double *w, const double *V, long long n, const double *hcoef,
                        double *partial, double *out, int n_out, unsigned int *ticket, cudaStream_t st,
                        const Givens &G = {}) {
-    using All = std::make_integer_sequence<int, kOrthChunk + 1>;
-    const OrthKernel k = mode == kDots ? orth_kernel<kDots>(cnt, All{})
+    using All = std::make_integer_sequence<int, kOrthChunk>;
+    const OrthKernel k = mode == kDots ? orth_kernel<kDots>(cnt, std::make_integer_sequence<int, kOrthChunk + 1>{})
                          : mode == kDotsOnly ? orth_kernel<kDotsOnly>(cnt, All{})
                          : mode == kUpdateDots ? orth_kernel<kUpdateDots>(cnt, All{}) : orth_kernel<kUpdateNorm>(cnt, All{});
     const int blocks = orth_blocks(n, cnt, mode == kUpdateNorm);

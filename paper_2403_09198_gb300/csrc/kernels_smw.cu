@@ -216,9 +216,9 @@ sts_status smw_build(sts_jac_s *h) {
     M.h_src_slot.assign(h->nnz_d, 0);
     for (int p = 0; p < b; ++p)
         for (int e = h->dptr[p]; e < h->dptr[p + 1]; ++e) M.h_src_slot[e] = slot[(size_t)p * b + h->didx[e]];
-    // factorisation schedule
+    // factorisation schedule (the structured family's setup has arithmetic indices instead)
     std::vector<int> colL_ptr(b + 1, 0), colL_slot, upd_ptr(1, 0), upd_tgt, upd_src;
-    for (int k = 0; k < b; ++k) {
+    for (int k = 0; k < b && !M.structured; ++k) {
         for (int i = k + 1; i < b; ++i) {
             if (slot[(size_t)i * b + k] < 0) continue;
             colL_slot.push_back(slot[(size_t)i * b + k]);
@@ -236,7 +236,7 @@ sts_status smw_build(sts_jac_s *h) {
     //                  dir 1 (A0^T): forward  U cols   (j<i, i), coefficient U_ji * dinv_j
     //                               backward L cols   (j>i, i), coefficient L_ji
     // Setup solves use the unscaled LU slots with the same row lists.
-    for (int dir = 0; dir < 2; ++dir) {
+    for (int dir = 0; dir < 2 && !M.structured; ++dir) {
         std::vector<int> fptr(b + 1, 0), fcol, fslot, fscale, bptr(b + 1, 0), bcol, bslot, bscale;
         // the setup's unscaled solves use (fcol, fslot) and (bcol, bslot); the
         // apply streams carry the scaled coefficients described by (fscale, bscale)
@@ -269,7 +269,6 @@ sts_status smw_build(sts_jac_s *h) {
         STS_TRY(upload(h, &M.ap_bwd_slot[dir], bslot));
         // apply program of any other pattern (k_smw_apply): columns forward, the pivot
         // inverses, columns backward, every column's rows dealt to the warps
-        if (M.structured) continue;
         struct Entry {
             int row, slot, scale;
         };
@@ -454,14 +453,16 @@ sts_status smw_build(sts_jac_s *h) {
             }
         }
     }
-    STS_TRY(upload(h, &M.lu_diag, M.h_lu_diag));
-    STS_TRY(upload(h, &M.src_slot, M.h_src_slot));
-    STS_TRY(upload(h, &M.d_ptr, h->dptr));
-    STS_TRY(upload(h, &M.f_colL_ptr, colL_ptr));
-    STS_TRY(upload(h, &M.f_colL_slot, colL_slot));
-    STS_TRY(upload(h, &M.f_upd_ptr, upd_ptr));
-    STS_TRY(upload(h, &M.f_upd_tgt, upd_tgt));
-    STS_TRY(upload(h, &M.f_upd_src, upd_src));
+    if (!M.structured) {
+        STS_TRY(upload(h, &M.lu_diag, M.h_lu_diag));
+        STS_TRY(upload(h, &M.src_slot, M.h_src_slot));
+        STS_TRY(upload(h, &M.d_ptr, h->dptr));
+        STS_TRY(upload(h, &M.f_colL_ptr, colL_ptr));
+        STS_TRY(upload(h, &M.f_colL_slot, colL_slot));
+        STS_TRY(upload(h, &M.f_upd_ptr, upd_ptr));
+        STS_TRY(upload(h, &M.f_upd_tgt, upd_tgt));
+        STS_TRY(upload(h, &M.f_upd_src, upd_src));
+    }
     const size_t P = h->ncp;
     const int r = h->r_diag;
     // zero in the padding cells and in the pairs that a block does not have (u = v = 0

@@ -270,10 +270,10 @@ struct Krylov {
     float *Z32 = nullptr;        // [m][n]   (mixed)
     float *t32a = nullptr, *t32b = nullptr;   // [n]
     double *w = nullptr, *r = nullptr, *xb = nullptr, *bb = nullptr, *tmp = nullptr;  // [n]
-    double *partial = nullptr;   // [kRedBlocks][m+2]
+    double *partial = nullptr;   // [kRedMax][32] sums per block of a reduction
     double *red = nullptr;       // [3][m+2] reduced dots and norms
     unsigned int *ticket = nullptr;   // [2] finished-block counters of the last-block reductions (0 between launches)
-    double *h_pinned = nullptr;  // host pinned [m+2]
+    double *h_pinned = nullptr;  // host pinned [3][m+2]
     double *c = nullptr;         // pair dots scratch [n_tiles*n_pslots*32]
     float *c32 = nullptr;
     // A cycle's Arnoldi steps as one CUDA graph (sts_gmres_opts.arnoldi): the
