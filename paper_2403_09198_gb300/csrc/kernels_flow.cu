@@ -81,12 +81,15 @@ __device__ __forceinline__ Mix mix_of(const double *M, int nc, int i) {
 // and the Jacobian needed it at the cell and at each of its neighbours.
 // da/dq_c = G0 + G1 cv_c + G2 r_c for a species (from a^2 = T g, g = (C + R) R / (rho C),
 // with R - g rho = -R^2 / C), GT for T, 0 for the velocities.
+template <bool EARLY>
 __global__ void __launch_bounds__(128) k_flow_mix(FlowDev F, const double *Q, const double *Qn) {
     extern __shared__ double rows[];             // [32][b | 1], species constants [N][4], partial sums [4][5][32]
     const int b = F.b, N = F.N, st = b | 1, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int c0 = blockIdx.x * kMixCells, n = min(kMixCells, F.nc - c0);
-    pdl_wait();
-    pdl_trigger();
+    if (EARLY) {
+        pdl_wait();
+        pdl_trigger();
+    }
     const double *src = (blockIdx.y ? Qn : Q) + (size_t)c0 * b;
     double *cst = rows + 32 * st;
     double(*part)[5][32] = reinterpret_cast<double(*)[5][32]>(cst + 4 * N);
@@ -283,14 +286,17 @@ static_assert(bCorner + 9 == kBlockFields, "block coefficients");
 // face from both of its cells.  In a kernel of its own: as the first step of the
 // kernels that use the coefficients it left seven of eight warps waiting at a barrier
 // (k_flow_jac 280 us on 128 x 128 cells, N = 60).
+template <bool EARLY>
 __global__ void __launch_bounds__(64) k_flow_face_jac(FlowDev F) {
     const int lane = threadIdx.x & 31, blk = blockIdx.x * 2 + (threadIdx.x >> 5), nc = F.nc;
     if (blk * kFlowCells >= nc) return;
     const double dt = F.dt;
     const double *M = F.mix;
     const FaceLane L = face_lane(F, blk, lane);
-    pdl_wait();
-    pdl_trigger();
+    if (EARLY) {
+        pdl_wait();
+        pdl_trigger();
+    }
     const Mix mi = mix_of(M, nc, L.i), mj = mix_of(M, nc, L.j);
     double nx, ny;
     normal_of(F.Lx, L.i, L.j, nx, ny);
@@ -379,6 +385,7 @@ __global__ void __launch_bounds__(64) k_flow_face_jac(FlowDev F) {
 }
 
 // Jacobian entries, one warp per cell, lanes over the species.
+template <bool EARLY>
 __global__ void __launch_bounds__(kFlowCells * 32) k_flow_jac(FlowDev F, const double *Q, double *S, double *U,
                                                               double *V) {
     __shared__ double sh[kFlowCells][kFaceFields * 4 + kCellFields];
@@ -391,6 +398,12 @@ __global__ void __launch_bounds__(kFlowCells * 32) k_flow_jac(FlowDev F, const d
     const int i = blockIdx.x * kFlowCells + warp;
     if (i >= nc) return;
     const int k0 = F.bptr[i], nf = F.bptr[i + 1] - k0 - 1;
+    if (EARLY) pdl_wait();
+    // this cell's coefficients: fc[field * 4 + face], cc[field]
+    double *fc = sh[warp], *cc = fc + kFaceFields * 4;
+    const double *gf = F.face + (size_t)blockIdx.x * kFaceFields * 32 + warp * 4;
+    for (int e = lane; e < kFaceFields * 4; e += 32) fc[e] = gf[(e >> 2) * 32 + (e & 3)];
+    if (lane < kCellFields) cc[lane] = F.cell[((size_t)blockIdx.x * kCellFields + lane) * kFlowCells + warp];
     // lane k of the row's at most five blocks
     const int col = lane <= nf ? F.bidx[k0 + lane] : -1;
     const int at = __ffs(__ballot_sync(0xffffffffu, col == i)) - 1, kd = k0 + at;
@@ -400,12 +413,6 @@ __global__ void __launch_bounds__(kFlowCells * 32) k_flow_jac(FlowDev F, const d
         spo[warp][f] = F.pip[k0 + lane];
         sk[warp][f] = F.soff[k0 + lane];
     }
-    pdl_wait();
-    // this cell's coefficients: fc[field * 4 + face], cc[field]
-    double *fc = sh[warp], *cc = fc + kFaceFields * 4;
-    const double *gf = F.face + (size_t)blockIdx.x * kFaceFields * 32 + warp * 4;
-    for (int e = lane; e < kFaceFields * 4; e += 32) fc[e] = gf[(e >> 2) * 32 + (e & 3)];
-    if (lane < kCellFields) cc[lane] = F.cell[((size_t)blockIdx.x * kCellFields + lane) * kFlowCells + warp];
     __syncwarp();
     const double *qi = Q + (size_t)i * b;
     const double g0 = M[mG0 * (size_t)nc + i], g1 = M[mG1 * (size_t)nc + i], g2 = M[mG2 * (size_t)nc + i];
@@ -446,12 +453,8 @@ __global__ void __launch_bounds__(kFlowCells * 32) k_flow_jac(FlowDev F, const d
                 U[(pd + 1) * b + c] = u2;
                 U[po * b + c] = u1;
                 U[(po + 1) * b + c] = u2;
-                // q_i gives this face no wave speed where both its G are 0, and 0 times a da that
-                // is no number is none: a test of bits, not an FP64 comparison
-                const double G1 = o[4 * fG], G2 = o[4 * fG + 4];
-                const double gf = (__double2hiint(G1) | __double2hiint(G2)) << 1 ? ga : 0.0;
-                V[pd * b + c] = G1 * gf;
-                V[(pd + 1) * b + c] = G2 * gf;
+                V[pd * b + c] = o[4 * fG] * ga;
+                V[(pd + 1) * b + c] = o[4 * fG + 4] * ga;
                 V[po * b + c] = o[4 * fG + 8] * gj;
                 V[(po + 1) * b + c] = o[4 * fG + 12] * gj;
                 // the normal is along one axis: one momentum row is constant over the species
@@ -474,6 +477,15 @@ __global__ void __launch_bounds__(kFlowCells * 32) k_flow_jac(FlowDev F, const d
             }
         }
     }
+    // where da/dq_i is no number, 0 times it was none: the pairs of the faces that take no bound
+    // from q_i (both G are 0), after the loop, which has no instruction to spare for them
+    if (!isfinite(g0 + g1 + g2))
+        for (int f = 0; f < nf; ++f) {
+            const double *o = fc + f;
+            if (o[4 * fG] != 0.0 || o[4 * fG + 4] != 0.0) continue;
+            double *v = V + (ps + 1 + 2 * f) * b;
+            for (int c = lane; c < N; c += 32) v[c] = v[b + c] = 0.0;       // the lane that wrote them
+        }
     // ---- flow components: computed by k_flow_face_jac, only written here
     for (int f = 0; f < nf; ++f) {
         const double *o = fc + f;
@@ -513,13 +525,16 @@ __global__ void __launch_bounds__(kFlowCells * 32) k_flow_jac(FlowDev F, const d
 // Residual scalars, as k_flow_face_jac; the flow components are complete here.  With
 // the flux (s_R f_i - s_L f_j + s_L s_R (u_j - u_i)) / (s_R - s_L) the species flux of a
 // face is ca q_i - cb q_j + cd (q_j - q_i).
+template <bool EARLY>
 __global__ void __launch_bounds__(64) k_flow_face_res(FlowDev F, double *R) {
     const int lane = threadIdx.x & 31, blk = blockIdx.x * 2 + (threadIdx.x >> 5), nc = F.nc;
     if (blk * kFlowCells >= nc) return;
     const double *M = F.mix, *Mn = F.mix + (size_t)kMixFields * nc;
     const FaceLane L = face_lane(F, blk, lane);
-    pdl_wait();
-    pdl_trigger();
+    if (EARLY) {
+        pdl_wait();
+        pdl_trigger();
+    }
     const Mix mi = mix_of(M, nc, L.i), mj = mix_of(M, nc, L.j);
     double nx, ny;
     normal_of(F.Lx, L.i, L.j, nx, ny);
@@ -548,6 +563,7 @@ __global__ void __launch_bounds__(64) k_flow_face_res(FlowDev F, double *R) {
 }
 
 // Residual of the species, one warp per cell, lanes over the species.
+template <bool EARLY>
 __global__ void __launch_bounds__(kFlowCells * 32) k_flow_res(FlowDev F, const double *Q, const double *Qn,
                                                               double *R) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -561,7 +577,7 @@ __global__ void __launch_bounds__(kFlowCells * 32) k_flow_res(FlowDev F, const d
         if (f < nf && F.bidx[k] == i) ++k;
         j[f] = f < nf ? F.bidx[k] : i;
     }
-    pdl_wait();
+    if (EARLY) pdl_wait();
     const double *gf = F.face + (size_t)blockIdx.x * kFaceFields * 32 + warp * 4;
     const double *gc = F.cell + (size_t)blockIdx.x * kCellFields * kFlowCells + warp;
     double fb[4], fd[4];
@@ -656,42 +672,51 @@ sts_status flow_alloc(sts_flow_s *f, double **p, size_t n) {
     return STS_OK;
 }
 
-sts_status flow_mix(sts_flow_s *f, const double *Q, const double *Qn) {
-    const int b = f->dev.b;
-    const size_t smem = (32 * (size_t)(b | 1) + 4 * (size_t)f->dev.N + 4 * 5 * 32) * sizeof(double);
-    if (smem > 48 * 1024) STS_CK(allow_all_smem(k_flow_mix));
-    k_flow_mix<<<dim3((f->dev.nc + kMixCells - 1) / kMixCells, Qn ? 2 : 1), 128, smem, f->stream>>>(f->dev, Q, Qn);
-    STS_LAUNCHED();
-    return STS_OK;
-}
-
-// Launch a kernel that reads what the kernel before it has written, `cells` cells a block.
-// On small grids it is launched early (programmatic dependent launch): there the launches
-// set the time, and as three dependent ones the calls had become slower than the single
-// kernel they came from (a column of 200 cells, N = 20: residual 22.3, then 25.4, now
-// 20.7 us).  Early blocks take room from the kernel they wait for: a Jacobian of 32 x 32
-// cells (128 blocks) takes 38.6 and 39.0 us, of 48 x 48 47.8 and 54.8, of 24 x 24 (72) 39.1
-// and 33.8; so early below one block of the last kernel per two SMs.
+// Small grids: the launches set the time, so each kernel after the first is launched early
+// (EARLY instances: programmatic dependent launch).  As three dependent kernels the calls
+// had become slower there than the single kernel they came from (a column of 200 cells, N =
+// 20: residual 22.3, then 25.4, now 20.6 us).  Early blocks take room from the kernel they
+// wait for: a Jacobian of 24 x 24 cells (72 blocks) takes 39.1 and 34.7 us, of 32 x 32 (128)
+// 38.6 and 39.0, of 48 x 48 47.8 and 54.8; so below one block of the last kernel per two SMs.
 constexpr int kEarlyCells = 152 / 2 * kFlowCells;
-template <typename... KArgs, typename... Args>
-sts_status flow_next(sts_flow_s *f, void (*kern)(KArgs...), int cells, int threads, Args... args) {
+
+template <bool EARLY, typename... KArgs, typename... Args>
+sts_status flow_launch(sts_flow_s *f, void (*kern)(KArgs...), int cells, int threads, Args... args) {
     const unsigned blocks = (f->dev.nc + cells - 1) / cells;
-    if (f->dev.nc < kEarlyCells) STS_CK(launch_pdl(kern, dim3(blocks), dim3(threads), 0, f->stream, args...));
+    if (EARLY) STS_CK(launch_pdl(kern, dim3(blocks), dim3(threads), 0, f->stream, args...));
     else kern<<<blocks, threads, 0, f->stream>>>(args...);
     STS_LAUNCHED();
     return STS_OK;
 }
 
-sts_status flow_res(sts_flow_s *f, const double *Q, const double *Qn, double *R) {
-    STS_TRY(flow_mix(f, Q, Qn));
-    STS_TRY(flow_next(f, k_flow_face_res, 2 * kFlowCells, 64, f->dev, R));
-    return flow_next(f, k_flow_res, kFlowCells, kFlowCells * 32, f->dev, Q, Qn, R);
+template <bool EARLY>
+sts_status flow_mix(sts_flow_s *f, const double *Q, const double *Qn) {
+    const int b = f->dev.b;
+    const size_t smem = (32 * (size_t)(b | 1) + 4 * (size_t)f->dev.N + 4 * 5 * 32) * sizeof(double);
+    if (smem > 48 * 1024) STS_CK(allow_all_smem(k_flow_mix<EARLY>));
+    k_flow_mix<EARLY><<<dim3((f->dev.nc + kMixCells - 1) / kMixCells, Qn ? 2 : 1), 128, smem, f->stream>>>(f->dev, Q, Qn);
+    STS_LAUNCHED();
+    return STS_OK;
 }
 
+template <bool EARLY>
+sts_status flow_res_as(sts_flow_s *f, const double *Q, const double *Qn, double *R) {
+    STS_TRY(flow_mix<EARLY>(f, Q, Qn));
+    STS_TRY(flow_launch<EARLY>(f, k_flow_face_res<EARLY>, 2 * kFlowCells, 64, f->dev, R));
+    return flow_launch<EARLY>(f, k_flow_res<EARLY>, kFlowCells, kFlowCells * 32, f->dev, Q, Qn, R);
+}
+sts_status flow_res(sts_flow_s *f, const double *Q, const double *Qn, double *R) {
+    return f->dev.nc < kEarlyCells ? flow_res_as<true>(f, Q, Qn, R) : flow_res_as<false>(f, Q, Qn, R);
+}
+
+template <bool EARLY>
+sts_status flow_jac_as(sts_flow_s *f, const double *Q, double *S, double *U, double *V) {
+    STS_TRY(flow_mix<EARLY>(f, Q, nullptr));
+    STS_TRY(flow_launch<EARLY>(f, k_flow_face_jac<EARLY>, 2 * kFlowCells, 64, f->dev));
+    return flow_launch<EARLY>(f, k_flow_jac<EARLY>, kFlowCells, kFlowCells * 32, f->dev, Q, S, U, V);
+}
 sts_status flow_jac(sts_flow_s *f, const double *Q, double *S, double *U, double *V) {
-    STS_TRY(flow_mix(f, Q, nullptr));
-    STS_TRY(flow_next(f, k_flow_face_jac, 2 * kFlowCells, 64, f->dev));
-    return flow_next(f, k_flow_jac, kFlowCells, kFlowCells * 32, f->dev, Q, S, U, V);
+    return f->dev.nc < kEarlyCells ? flow_jac_as<true>(f, Q, S, U, V) : flow_jac_as<false>(f, Q, S, U, V);
 }
 
 // ||x||_2 of a device vector of the generator's stream (synchronous)
