@@ -44,7 +44,7 @@ struct MvBase {
 };
 // INT: x and y are in the internal layout, the common case.  Without the strides (and
 // without three fields that no kernel read) the FP32 products take, in us, 128 x 128 cells,
-// N = 60: 38.2 -> 37.4, 64 x 64: 15.3 -> 14.5, 96 x 96, N = 100: 39.1 -> 37.1; FP64 the same
+// N = 60: 38.2 -> 37.4, 64 x 64: 15.3 -> 14.5, 96 x 96, N = 100: 39.1 -> 35.3; FP64 the same
 // (98.1, 31.7, 100.6; 96 x 96, N = 30 47.3 -> 47.6).
 template <typename T, bool INT = false>
 struct MvArgs : MvBase<T> {
@@ -649,10 +649,14 @@ inline int pass2_group_rows(int N, int n_tiles, long long W, int s_plan, int s_r
     // a warp's serial rows, not the number of items, set the time (whole products, cell-major
     // in place, us: N = 10, 32 tiles 22.1 -> 14.6, 128 tiles 26.0 -> 16.7; N = 60, 32 tiles
     // 36.3 -> 21.9, 128 tiles 43.6 -> 39.9).  Not in FP32 (spread = false), whose rows are
-    // short against an item's start: N = 60, 8 / 128 tiles 10.3 / 17.6 us, spread 12.1 / 19.2
-    if (!spread) return s;
-    const long long per_tile = W / n_tiles - 1;
-    return per_tile > 0 ? (int)std::min<long long>(s, (N + per_tile - 1) / per_tile) : s;
+    // short against an item's start: N = 60, 8 / 128 tiles 10.3 / 17.6 us, spread 12.1 / 19.2.
+    // FP32 items that just do not get a warp each take that many rows instead (its instances
+    // of 80 registers keep 24 warps per SM, those of 72 had 28; N = 60, 288 tiles 25.2 -> 23.4 us, 338
+    // 28.2 -> 25.9, N = 100, 242 tiles 34.3 -> 30.9; of 26 such sizes none slower)
+    const long long per_tile = W / n_tiles - 1, fit = per_tile > 0 ? (N + per_tile - 1) / per_tile : 0;
+    if (spread) return per_tile > 0 ? (int)std::min<long long>(s, fit) : s;
+    const long long of_s = (long long)n_tiles * ((N + s - 1) / s + 1);
+    return of_s > W && 2 * of_s < 3 * W && fit <= 2 * s ? (int)fit : s;
 }
 
 template <typename T>
