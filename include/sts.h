@@ -161,12 +161,13 @@ typedef struct {
     int arnoldi;          /* STS_ARNOLDI_GRAPH (default, 0): for right preconditioning in
                              FP64 with restart <= 64, each cycle's Arnoldi steps run as
                              one CUDA graph, every step under a conditional node nested
-                             in the previous step's body, which a device-side Givens
-                             kernel switches off once the cycle is done: the host
-                             synchronises once per cycle.  The graph of a (direction,
+                             in the previous step's body, which the step's last sweep,
+                             rotating on the device, switches off once the cycle is
+                             done: the host synchronises once per cycle.  The graph of a (direction,
                              preconditioning) is built on first use and kept.
                              STS_ARNOLDI_HOST (1): the host rotates after every step (a
-                             synchronisation per step); left and mixed solves always do */
+                             synchronisation per step); left and mixed solves always
+                             do.  The two agree to rounding, not in every bit           */
 } sts_gmres_opts;
 
 /* Result of sts_gmres_solve. */
@@ -275,7 +276,8 @@ sts_status sts_jac_bjacobi_apply_f32(sts_jac_t h, const float *x, float *z, int 
 /*
  * Solve J x = b (or J^T x = b) by restarted right-preconditioned GMRES(m)
  * (Section 6, Eq. right_precond_system; Saad & Schultz), classical Gram-Schmidt
- * with a second pass, Givens rotations on the host in FP64.  x holds the
+ * with a second pass, Givens rotations in FP64 (on the device or on the host, see
+ * sts_gmres_opts.arnoldi).  x holds the
  * initial guess on entry and the solution on exit (pass zeros for x0 = 0).  A
  * zero guess (||x0|| = 0, found in the same pass as ||b||) starts from r = b
  * without the product J x0.

@@ -4,9 +4,9 @@
 // cycle starts from the true FP64 residual r = b - A x, builds the Krylov basis
 // by classical Gram-Schmidt with a second pass (CGS2: dots, update and dots
 // in one sweep, update and norm; same result as modified Gram-Schmidt in exact
-// arithmetic), reduces the Hessenberg matrix with Givens rotations on the host
-// in FP64 and updates x += Z y with Z = [M v_0, ..., M v_{k-1}] (for a fixed M
-// this equals x += M (V y)).  Convergence is declared on the recomputed true
+// arithmetic), reduces the Hessenberg matrix with Givens rotations in FP64 (on the
+// device in cycles that run as a graph, on the host in the others) and updates
+// x += Z y with Z = [M v_0, ..., M v_{k-1}] (for a fixed M this equals x += M (V y)).  Convergence is declared on the recomputed true
 // residual only.  Mixed mode (flexible GMRES): z_j = M32(v_j) and w = A32 z_j in
 // FP32; the basis, the orthogonalisation, x and the residual refresh stay FP64.
 // Left preconditioning (Eq. left_precond_system, (M A) x = M b): the cycle's
@@ -530,7 +530,10 @@ sts_status ensure_workspace(sts_jac_s *h, int m, bool mixed) {
 // conditional (IF) node, nested in step j - 1's body: z_j = M v_j, w = A z_j,
 // the two Gram-Schmidt passes,
 // of which the last folds the new Hessenberg column into the rotations on
-// the device (the host loop's arithmetic, in the same order), records the
+// the device (the host loop's rotations, rounded otherwise: FMAs of products formed
+// beforehand, reciprocals for quotients, a square root for hypot, and a breakdown
+// judged against ||w||^2 from the first pass's coefficients, the basis being
+// orthonormal, instead of w . w; the two need not agree in the last bits), records the
 // rotated residual, and switches step j + 1 on or off, and finally v_{j+1} =
 // w / h(j+1, j).  The host launches the graph once per cycle and reads the
 // rotated system back once, instead of synchronising after every step.
