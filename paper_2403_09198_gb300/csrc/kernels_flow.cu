@@ -17,7 +17,7 @@
 // is A_n(q_i) at the summed normal.
 //
 // Measured on 128 x 128 cells, N = 60 (band 2): Jacobian (571 MB written) 1326 us with the
-// scalars formed by every warp and every entry on its own, now 27 + 28 + 238 us (scalars
+// scalars formed by every warp and every entry on its own, now 24 + 29 + 238 us (scalars
 // of cells, of faces, entries); residual 540 us, now 26 + 12 + 47.  The entries keep the
 // FP64 pipe 63% busy (134 of the 238 us are pipe time); more warps per SM or four faces
 // at once without branches between them left the time as it was.

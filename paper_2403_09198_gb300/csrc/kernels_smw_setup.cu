@@ -387,8 +387,8 @@ __global__ void __launch_bounds__(kTile) k_smw_lu_arrow(SetupArgs a) {
 // registers and the flow rows accumulate beside them, so a row is W + 3 FMAs in
 // each sweep; rows are taken U at a time with the next U rows' coefficients
 // loaded ahead.  Bound by the FP64 pipe once a sub-partition holds a few warps.
-// Measured on 128 x 128 cells, N = 60, W = 2: nine pairs 300 -> 194 us (80% of the
-// pipe), two pairs in both directions 302 -> 114 us.
+// Measured on 128 x 128 cells, N = 60, W = 2: nine pairs 300 -> 201 us (FP64 pipe
+// busy 77% of it), two pairs in both directions 302 -> 114 us.
 template <int W, int DIR>
 __device__ __forceinline__ void arrow_solve(const SetupArgs &a, const double *src, double *w, int cell) {
     constexpr int NF = kStructNF, U = W <= 2 ? 4 : 2, R = W + NF;
@@ -705,7 +705,7 @@ __global__ void __launch_bounds__(kPackWarps * kTile) k_smw_spack(PackArgs<T> A)
 // by memory, is packed beside it by `parts` of the blocks of every tile, which alternate
 // with the folding ones as far as they go.  Nine pairs on 128 x 128 cells, N = 60:
 // 280 us in one kernel that formed a fold entry per position, 68 + 173 us as two kernels
-// (133 us of FP64 pipe time), 216 us here.
+// (133 us of FP64 pipe time), 217 us here.
 constexpr int kFoldWarps = 4;
 
 template <int R>

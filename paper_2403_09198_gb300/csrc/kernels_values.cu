@@ -13,7 +13,7 @@
 // the streams are allocated and never written again.
 //
 // Bound by HBM.  Measured on 128 x 128 cells, N = 60: 9 / 2 pairs (1.46 GB read and
-// written) 654 -> 289 us, 5.0 TB/s; 2 / 1 pairs, both directions, 790 -> 396 us.
+// written) 654 -> 287 us, 5.1 TB/s; 2 / 1 pairs, both directions, 790 -> 396 us.
 // Before, one thread per stream position gathered its value from the public array,
 // once for every destination.  The runs' loads have to be issued before the first
 // value is used (490 us otherwise, the warps waiting on one load after another).
