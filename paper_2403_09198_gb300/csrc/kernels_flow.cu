@@ -478,8 +478,10 @@ __global__ void __launch_bounds__(kFlowCells * 32) k_flow_jac(FlowDev F, const d
         }
     }
     // where da/dq_i is no number, 0 times it was none: the pairs of the faces that take no bound
-    // from q_i (both G are 0), after the loop, which has no instruction to spare for them
-    if (!isfinite(g0 + g1 + g2))
+    // from q_i (both G are 0), after the loop, which has no instruction to spare for them; by the
+    // exponents, since two sums and a comparison are FP64 instructions of the whole warp
+    auto no_number = [](double v) { return (__double2hiint(v) & 0x7ff00000) == 0x7ff00000; };
+    if (no_number(g0) || no_number(g1) || no_number(g2))
         for (int f = 0; f < nf; ++f) {
             const double *o = fc + f;
             if (o[4 * fG] != 0.0 || o[4 * fG + 4] != 0.0) continue;
